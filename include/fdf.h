@@ -169,8 +169,7 @@ typedef struct fdf_params {
                                   of the particle pass, a persistent grid of this many blocks
                                   of 256 threads per SM: 2 = two particles per thread (128
                                   registers), 1 or 3 = one particle per thread (80 registers);
-                                  0 = automatic (2: measured fastest on the 3 x 256^3
-                                  workload, 714 ms per run against 736 ms with 3).  The
+                                  0 = automatic (2, or 3 with interp_order = 2).  The
                                   results are the same bit for bit.  Ignored by the other
                                   forms. */
     int32_t  gather_tile;      /* the split-state forms: 1 = each block's kicks read the grid from a

@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "fdf_internal.cuh"
+#include "wide_poly.cuh"
 
 using namespace fdf;
 
@@ -373,6 +374,7 @@ struct fdf_ctx {
     // fitted integral polynomials of the FP64-state form by interval (ln a ends) and
     // kind (0 drift, 1 kick 1/eps, 2 kick eps), with whether the fit passed
     std::map<std::tuple<double, double, int>, std::pair<bool, WidePoly>> wide_fits;
+    double q_unit = 1;                // the kick integrals' momentum unit (PushArgs::q_unit2)
     Layout lay{};
     char* block = nullptr;
     bool own_block = false;
@@ -542,8 +544,10 @@ void fill_pass(const fdf_ctx* c, PushArgs& a)
     a.order = c->p.interp_order == 2 ? 2 : 1;
     a.eom = c->p.eom;
     a.wide_series = 1;
+    a.q_unit2 = (float)(c->q_unit * c->q_unit);
     for (int s = 0; s < kMaxSpecies; ++s) a.m2[s] = c->p.m_ev[s] * c->p.m_ev[s];
-    const int pb = c->p.pass_blocks > 0 ? c->p.pass_blocks : 2;
+    // order-2 reads run faster with three blocks of one particle per thread (k_push_wide)
+    const int pb = c->p.pass_blocks > 0 ? c->p.pass_blocks : a.order == 2 ? 3 : 2;
     a.grid_blocks = c->sm_count * pb;
     a.pair = pb == 2 ? 1 : 0;
     a.ctr = c->pass_ctr;
@@ -605,6 +609,42 @@ void fill_wide(fdf_ctx* c, bool drift, double d1, double d2, const double* Wd, c
     }
 }
 
+// The kick's integrals for the FP32 pipe (w_kick), once it is known whether the pass uses
+// the fits (series) or sums the nodes: u.wide.kick_fast says whether they serve it.
+void fill_kick_fast(const fdf_ctx* c, bool series, SubStep& u)
+{
+    WideCoef& w = u.wide;
+    const double unit = c->q_unit, a2c = std::exp(u.k1 + u.k2);
+    w.kick_fast = kKickFp64;
+    if (!u.do_kick) {
+        w.kick_fast = series ? kKickSeries : kKickNodes;
+        return;
+    }
+    for (int s = 0; s < c->p.n_species; ++s) {
+        const double mu = c->p.m_ev[s] * c->p.m_ev[s] * a2c * unit * unit;
+        w.fmuh[s] = (float)mu;
+        w.fmul[s] = (float)(mu - (double)w.fmuh[s]);
+    }
+    if (series) {
+        auto pack = [&](const WidePoly& P, double scale, KickPoly& K) {
+            for (int k = KickLen<true>::kDeg; k <= kWideDeg; ++k)
+                if (P.c32[k] != 0.f) return false;      // a longer fit than w_kick evaluates
+            std::memset(&K, 0, sizeof(K));
+            kick_coef(K, 0, P.c64[0] * scale);
+            for (int k = 1; k <= KickLen<true>::kDeg; ++k) kick_coef(K, k, (double)P.c32[k - 1] * scale);
+            return true;
+        };
+        if (pack(w.kphi, unit, w.fphi) && pack(w.kpsi, 1.0 / unit, w.fpsi)) w.kick_fast = kKickSeries;
+    } else {
+        double W[kMaxGL], e[kMaxGL];
+        nodes(c, u.k1, u.k2, W, e, true);
+        for (int j = 0; j < c->nkick; ++j) e[j] = e[j] / a2c - 1.0;
+        if (kick_node_poly(W, e, c->nkick, -0.5, unit, w.fphi) &&
+            kick_node_poly(W, e, c->nkick, 0.5, 1.0 / unit, w.fpsi))
+            w.kick_fast = kKickNodes;
+    }
+}
+
 // Coefficients of one sub-step: drift over [d1, d2] (if any), kick over [k1, k2] (if any).
 // The split form's drift weights carry the factor 2^32/L (position quanta per Mpc).
 void fill_substep(fdf_ctx* c, bool drift, double d1, double d2, bool kick, double k1, double k2, SubStep& u)
@@ -612,6 +652,8 @@ void fill_substep(fdf_ctx* c, bool drift, double d1, double d2, bool kick, doubl
     std::memset(&u, 0, sizeof(u));
     u.do_drift = drift;
     u.do_kick = kick;
+    u.k1 = k1;
+    u.k2 = k2;
     double Wd[kMaxGL], ad[kMaxGL], Wk[kMaxGL], ak[kMaxGL];
     if (drift) nodes(c, d1, d2, Wd, ad);
     if (kick) nodes(c, k1, k2, Wk, ak, true);
@@ -1033,6 +1075,7 @@ int fdf_create(const fdf_params* p, const fdf_tables* t, void* stream, void* are
     }
     gauss_legendre(c->ngl, c->glx, c->glw);
     gauss_legendre(c->nkick, c->glxk, c->glwk);
+    c->q_unit = std::ldexp(1.0, (int)std::min(50.0, std::max(-50.0, std::round(-std::log2(c->T_ev)))));
     c->uniform = 1;
     for (int s = 1; s < p->n_species; ++s)
         if (p->m_ev[s] != p->m_ev[0]) c->uniform = 0;
@@ -1342,6 +1385,15 @@ int slice_next(fdf_ctx* c, PushArgs& a)
         if (!a.sub[u].wide_ok) a.wide_series = 0;
     }
     const int form = form_of(c->p.precision);
+    if (form == kWide) {
+        // the node sums have one particle per thread, so three of their blocks are resident
+        if (!a.wide_series && a.pair) a.grid_blocks = c->sm_count * 3;
+        a.kick_fast = a.wide_series ? kKickSeries : kKickNodes;
+        for (int u = 0; u < a.nsub; ++u) {
+            fill_kick_fast(c, a.wide_series != 0, a.sub[u]);
+            if (a.sub[u].wide.kick_fast == kKickFp64) a.kick_fast = kKickFp64;
+        }
+    }
     if ((form == kWide && !a.wide_series) || (form == kFixed && !a.drift_series) || form == kPlain)
         c->pass_series = 0;
     ++c->pass_count;

@@ -9,6 +9,20 @@
 
 namespace fdf {
 
+// 1/sqrt(v) of a normal v, the FP32 hardware estimate (relative error below 2^-22)
+__device__ __forceinline__ float w_rsqrt(float v)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(v));
+    return y;
+}
+
+}  // namespace fdf
+
+#include "wide_math.cuh"
+
+namespace fdf {
+
 // The three state forms of the precision settings (FDF_PREC_*): the plain FP64 form,
 // the FP64-state form with FP32 or BF16 grids, and the split-state form with
 // fixed-point positions.
@@ -77,6 +91,8 @@ struct WidePoly {
     float c32[kWideDeg + 1];    // coefficients kWideD64.. (kick: kWideK64..), FP32, zero-padded
 };
 
+enum KickFast { kKickFp64 = 0, kKickSeries = 1, kKickNodes = 2 };
+
 struct WideCoef {
     // The drift in the variable v = 1 + |q|^2 / (m^2 a_c^2) (per species, m > 0): then
     // t = 1/v = r_v^2 with r_v = v^(-1/2), and D = r gm(t) = r_v gm(t) / (m a_c), the
@@ -90,6 +106,11 @@ struct WideCoef {
     WidePoly kphi;              // gm of the kick interval: K_phi = r gm(t)
     WidePoly kpsi;              // gp of the kick interval: K_psi = u r gp(t)
     float dtau_k;               // conformal time of the kick interval
+    // the kick's integrals on the FP32 pipe (w_kick): the polynomials and m^2 a_c^2 in the
+    // run's momentum unit (PushArgs::q_unit), of the fits or of the node sums
+    int kick_fast;              // KickFast
+    KickPoly fphi, fpsi;
+    float fmuh[kMaxSpecies], fmul[kMaxSpecies];
 };
 
 // One sub-step of a particle pass: an optional drift over [ln a_k, ln a_k+1] and an
@@ -99,6 +120,7 @@ struct SubStep {
     int do_kick;
     double emax;                // largest |e_j| of any species (the series converges for <= 1/4)
     int wide_ok;                // the FP64-state form's fits of this sub-step passed
+    double k1, k2;              // the kick's interval in ln a
     SpeciesCoef sp[kMaxSpecies];
     WideCoef wide;              // the FP64-state form
 };
@@ -123,6 +145,9 @@ struct PushArgs {
     int tile_gather;            // the split-state form: kicks gather from shared-memory tiles
     int wide_series;            // the FP64-state form: every fitted polynomial of this pass passed
                                 // its check (else the integrals loop over the nodes)
+    int kick_fast;              // the FP64-state form: the KickFast that every sub-step allows
+    float q_unit2;              // the FP64-state form: the square of the kick integrals' momentum unit, a
+                                // power of two near 1/T (keeps their FP32 squares within FP32's exponents)
     double m2[kMaxSpecies];     // m^2 per species (eV^2)
     int N;                      // grid side
     int nsub;                   // sub-steps in this pass, 1..kMaxSub

@@ -189,13 +189,53 @@ __device__ __forceinline__ void gather_order(int order, const Gt* __restrict__ G
 __device__ __forceinline__ void float_cell(double x, float invh, uint32_t N, uint32_t& i0, uint32_t& i1, float& f)
 {
     const float u = d2f_bits(x) * invh;       // x in [0, L): u in [0, N]
-    uint32_t i = (uint32_t)u;
-    f = u - (float)i;
+    // the whole part by a sum with 2^23 rounded down (u < 2^22): no conversion instruction
+    const float s = __fadd_rz(u, 8388608.f);
+    uint32_t i = __float_as_uint(s) & 0x7FFFFFu;
+    f = __fsub_rn(u, __fsub_rn(s, 8388608.f));
     i = i >= N ? i - N : i;                    // u rounded up to N: node 0
     i = i < N ? i : N - 1u;                    // (never taken for x in [0, L); keeps reads in the grid)
     i0 = i;
     i1 = i + 1u == N ? 0u : i + 1u;
 }
+
+// Two FP32 lanes in one register pair: one instruction per two fused multiply-adds.
+__device__ __forceinline__ uint64_t pack2(float a, float b)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t r, float& a, float& b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// A cell's 8 slots as 4 pairs.
+template <typename Gt> struct Cell2;
+template <> struct Cell2<float> {
+    __device__ static void load(const float* G, uint32_t c, uint64_t v[4])
+    {
+        asm("ld.global.nc.L1::no_allocate.v4.b64 {%0, %1, %2, %3}, [%4];"
+            : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3])
+            : "l"(G + 8 * (size_t)c));
+    }
+};
+template <> struct Cell2<__nv_bfloat16> {
+    __device__ static void load(const __nv_bfloat16* G, uint32_t c, uint64_t v[4])
+    {
+        float f[8];
+        Cell<__nv_bfloat16>::load(G, c, f);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = pack2(f[2 * k], f[2 * k + 1]);
+    }
+};
 
 template <typename Gt>
 __device__ __forceinline__ void gather_wide(int order, const Gt* __restrict__ G, uint32_t N, float invh,
@@ -232,6 +272,7 @@ __device__ __forceinline__ void gather_wide(int order, const Gt* __restrict__ G,
         }
         return;
     }
+    uint64_t a[4] = {0, 0, 0, 0};
     float fx, fy, fz;
     float_cell(x[0], invh, N, ix[0], ix[1], fx);
     float_cell(x[1], invh, N, iy[0], iy[1], fy);
@@ -240,11 +281,14 @@ __device__ __forceinline__ void gather_wide(int order, const Gt* __restrict__ G,
     for (int c = 0; c < 8; ++c) {
         const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;
         const float w = (cx ? fx : 1.f - fx) * (cy ? fy : 1.f - fy) * (cz ? fz : 1.f - fz);
-        float v[8];
-        Cell<Gt>::load(G, (iz[cz] * N + iy[cy]) * N + ix[cx], v);
+        uint64_t v[4];
+        Cell2<Gt>::load(G, (iz[cz] * N + iy[cy]) * N + ix[cx], v);
+        const uint64_t ww = pack2(w, w);
 #pragma unroll
-        for (int s = 0; s < 8; ++s) g[s] = fmaf(w, v[s], g[s]);
+        for (int k = 0; k < 4; ++k) a[k] = fma2(ww, v[k], a[k]);
     }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) unpack2(a[k], g[2 * k], g[2 * k + 1]);
 }
 
 // FP64 read at an FP64 position in [0, L).
@@ -709,14 +753,42 @@ void push_split(cudaStream_t s, unsigned b, const PushArgs& a, const ParticleSta
 
 // ---- the fused leapfrog pass, FP64-state form --------------------------------------
 // x and q are FP64 in HBM and in registers and are accumulated in FP64; q_0 is FP32.
-// Every step integral is evaluated in FP64 (WideCoef):
+// Every step integral has the value that FP64 arithmetic gives it (WideCoef):
 //   drift  D = int dtau / sqrt(q^2 + m^2 a^2) = r gm(t),  r = (q^2 + m^2 a_c^2)^(-1/2),
 //   kick   K_phi = int dtau / eps_0 = r0 gm(t0),  K_psi = int eps_0 dtau = (u0 r0) gp(t0),
 // with the polynomial's leading terms in FP64 and the rest in FP32 (they add less
 // than 1e-7 of the integral).  The kick, at most ~1e-3 of |q| per step, is formed in
-// FP32 from the FP32 gradients and added to q in FP64.  GB300 runs FP64 arithmetic
-// and FP64 <-> FP32 conversions at 1/64 of its FP32 rate, so every conversion goes
-// through the integer pipe (d2f_bits, f2d_bits).
+// FP32 from the FP32 gradients and added to q in FP64.
+//
+// Bound: the FP64 pipe.  GB300 runs FP64 arithmetic and FP64 <-> FP32 conversions at 1/64
+// of its FP32 rate, so conversions are bit operations (d2f_bits, f2d_bits), and the
+// inverse square roots and the kick's integrals get the bits of their FP64 formulas from
+// the integer and FP32 pipes (wide_math.cuh): 17 FP64 instructions per particle-step (|q|^2
+// 3, v 1, t 1, polynomial 5, D 1, x 3, q 3), 30 with the formulas in FP64.  3 x 256^3
+// particles, 200 steps, passes of 8: 563 -> 376 ms in the pass; node sums, 160^3
+// particles, 100 steps: 61.4 -> 19.6 ms.  A stage handles all P particles of a thread
+// before its rare branch, so that their chains interleave (422 ms with a branch each).
+
+// Periodic wrap into [0, L) (wrap_f64, a result equal to L mapping to 0), taken only
+// when x left the box.  The test runs on the bit patterns (IEEE doubles order like
+// integers when positive; a negative value, as an unsigned integer, is above them all),
+// so only a warp with a wrapping particle spends FP64 instructions on it.
+template <int P>
+__device__ __forceinline__ void wrap_rare(double (&x)[P][3], double L, double invL, unsigned long long Lbits)
+{
+    bool out = false;
+#pragma unroll
+    for (int p = 0; p < P; ++p)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) out |= (unsigned long long)__double_as_longlong(x[p][d]) >= Lbits;
+    if (out) {
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                if ((unsigned long long)__double_as_longlong(x[p][d]) >= Lbits) x[p][d] = wrap_f64(x[p][d], L, invL);
+    }
+}
 
 // p(t) = sum_k c_k t^k: the terms from k = NF64 up in FP32 (Horner, from tf, t in FP32),
 // then the terms below NF64 in FP64
@@ -732,46 +804,61 @@ __device__ __forceinline__ double wide_poly(const WidePoly& P, double t, float t
     return acc;
 }
 
-// Periodic wrap into [0, L) (wrap_f64, a result equal to L mapping to 0), taken only
-// when x left the box.  The test runs on the bit patterns (IEEE doubles order like
-// integers when positive; a negative value has the sign bit), so only a warp with a
-// wrapping particle spends FP64 instructions on it.
-__device__ __forceinline__ double wrap_rare(double x, double L, double invL, long long Lbits)
+// rsqrt_fp64 of P values without its FP64 instructions, except for the few arguments that
+// w_rsqrt53 leaves to it (one branch for all P, so that their chains interleave).
+template <int P>
+__device__ __forceinline__ void rsqrt_int(const double (&u)[P], double (&r)[P])
 {
-    const long long b = __double_as_longlong(x);
-    if (b >= Lbits || b < 0) x = wrap_f64(x, L, invL);
-    return x;
-}
-
-// The step integrals of one sub-step.  The drift's D depends on |q|^2, the kick's K_phi
-// and K_psi on |q0|^2 only: the two chains are independent of each other and of the
-// gather, so the pass issues them back to back and the FP64 pipe overlaps their
-// latencies and the gather's.
-template <bool SERIES>
-__device__ __forceinline__ double drift_integral(const SubStep& st, int s, int n_gl, const double q[3])
-{
-    if constexpr (SERIES) {
-        if (!st.wide.massless[s]) {
-            const double inv = st.wide.inv_muc[s];
-            // v = 1 + |q|^2 / (m^2 a_c^2), t = 1/v, D = v^(-1/2) gm(t) / (m a_c)
-            const double v = fma(fma(q[0], q[0], fma(q[1], q[1], q[2] * q[2])), inv, 1.0);
-            const double rv = rsqrt_fp64(v);
-            const double t = rv * rv;
-            return rv * wide_poly<kWideD64>(st.wide.drift[s], t, d2f_bits(t));
-        }
-        return rsqrt_fp64(fma(q[0], q[0], fma(q[1], q[1], q[2] * q[2]))) * st.wide.wsum[s];
-    } else {
-        const double qq = fma(q[0], q[0], fma(q[1], q[1], q[2] * q[2]));
-        const SpeciesCoef& sc = st.sp[s];
-        double D = 0.0;
-        for (int j = 0; j < n_gl; ++j) D = fma(sc.Wd[j], rsqrt_fp64(qq + sc.mud[j]), D);
-        return D;
+    bool ok[P], all = true;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        ok[p] = w_rsqrt53(u[p], rsqrtf(d2f_bits(u[p])), r[p]);
+        all &= ok[p];
+    }
+    if (!all) {
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            if (!ok[p]) r[p] = rsqrt_fp64(u[p]);
     }
 }
 
+// The drift integrals of one sub-step.
+template <bool SERIES, int P>
+__device__ __forceinline__ void drift_integrals(const SubStep& st, const int (&s)[P], int n_gl, const double (&q)[P][3],
+                                                double (&D)[P])
+{
+    double qq[P], u[P], r[P];
+#pragma unroll
+    for (int p = 0; p < P; ++p) qq[p] = fma(q[p][0], q[p][0], fma(q[p][1], q[p][1], q[p][2] * q[p][2]));
+    if constexpr (SERIES) {
+        // v = 1 + |q|^2 / (m^2 a_c^2), t = 1/v, D = v^(-1/2) gm(t) / (m a_c); a massless
+        // species takes D = |q|^-1 sum_j W_j
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            u[p] = st.wide.massless[s[p]] ? qq[p] : fma(qq[p], st.wide.inv_muc[s[p]], 1.0);
+        rsqrt_int(u, r);
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            const double t = r[p] * r[p];
+            const double g = wide_poly<kWideD64>(st.wide.drift[s[p]], t, d2f_bits(t));
+            D[p] = r[p] * (st.wide.massless[s[p]] ? st.wide.wsum[s[p]] : g);
+        }
+    } else {
+#pragma unroll
+        for (int p = 0; p < P; ++p) D[p] = 0.0;
+        for (int j = 0; j < n_gl; ++j) {
+#pragma unroll
+            for (int p = 0; p < P; ++p) u[p] = qq[p] + st.sp[s[p]].mud[j];
+            rsqrt_int(u, r);
+#pragma unroll
+            for (int p = 0; p < P; ++p) D[p] = fma(st.sp[s[p]].Wd[j], r[p], D[p]);
+        }
+    }
+}
+
+// The kick's integrals in FP64, rounded to FP32.
 template <bool SERIES>
-__device__ __forceinline__ void kick_integrals(const SubStep& st, int s, int n_kick, double s0, float& Kpsif,
-                                               float& Kphif)
+__device__ __noinline__ float2 kick_fp64(const SubStep& st, int s, int n_kick, double s0)
 {
     double Kpsi, Kphi;
     if constexpr (SERIES) {
@@ -796,65 +883,58 @@ __device__ __forceinline__ void kick_integrals(const SubStep& st, int s, int n_k
             Kphi = fma(sc.Wk[j], ie, Kphi);
         }
     }
-    Kpsif = d2f_bits(Kpsi);
-    Kphif = d2f_bits(Kphi);
+    return make_float2(d2f_bits(Kpsi), d2f_bits(Kphi));
 }
 
-// One particle through the sub-steps of a pass of the FP64-state form.
-template <typename Gt, bool SERIES, bool UNI>
-__device__ __forceinline__ void wide_particle(const PushArgs& a, double* __restrict__ xd, double* __restrict__ qd,
-                                              const float* __restrict__ q0f, int64_t i)
+// |q_0|^2 in FP64 (exact products of the FP32 components) and, in the kick integrals' unit,
+// as a pair of floats; once per pass.
+struct Norm0 {
+    double s;
+    float h, l;
+};
+__device__ __forceinline__ Norm0 norm0(const PushArgs& a, float qa, float qb, float qc, float& q02)
 {
-    const int64_t n = a.n;
-    const uint32_t N = (uint32_t)a.N;
-    const float invh = (float)a.invh;
-    const long long Lbits = __double_as_longlong(a.L);
-    const int s = UNI ? 0 : species_of(a, i);
-    double x[3] = {__ldcs(xd + i), __ldcs(xd + n + i), __ldcs(xd + 2 * n + i)};
-    double q[3] = {__ldcs(qd + i), __ldcs(qd + n + i), __ldcs(qd + 2 * n + i)};
-    const float qa = __ldcs(q0f + i), qb = __ldcs(q0f + n + i), qc = __ldcs(q0f + 2 * n + i);
-    // |q0|^2: exact products of the FP32 components, summed in FP64 (once per pass)
+    Norm0 n;
     const double da = f2d_bits(qa), db = f2d_bits(qb), dc = f2d_bits(qc);
-    const double s0 = fma(da, da, fma(db, db, dc * dc));
-    const float q02 = d2f_bits(s0);
-    bool moved = false, kicked = false;
-    for (int u = 0; u < a.nsub; ++u) {
-        const SubStep& st = a.sub[u];
-        float Kpsif = 0.f, Kphif = 0.f;
-        if (st.do_kick) kick_integrals<SERIES>(st, s, a.n_kick, s0, Kpsif, Kphif);
-        if (st.do_drift) {
-            const double D = drift_integral<SERIES>(st, s, a.n_gl, q);
+    n.s = fma(da, da, fma(db, db, dc * dc));
+    q02 = d2f_bits(n.s);
+    n.h = q02 * a.q_unit2;
+    // in the unit first: the low part of a tiny |q_0|^2 would leave FP32's exponents
+    n.l = d2f_bits((n.s - f2d_bits(q02)) * (double)a.q_unit2);
+    return n;
+}
+
+template <bool SERIES, int P>
+__device__ __forceinline__ void kick_integrals(const PushArgs& a, const SubStep& st, const int (&s)[P],
+                                               const Norm0 (&n0)[P], float (&Kpsi)[P], float (&Kphi)[P])
+{
+    constexpr int FAST = SERIES ? kKickSeries : kKickNodes;
+    bool ok[P], all = a.kick_fast == FAST;
 #pragma unroll
-            for (int d = 0; d < 3; ++d) x[d] = wrap_rare(fma(q[d], D, x[d]), a.L, a.invL, Lbits);
-            moved = true;
-        }
-        if (st.do_kick) {
-            float g[8];
-            gather_wide<Gt>(a.order, reinterpret_cast<const Gt*>(a.G[u]), N, invh, x, g);
-            const float qdphi = qa * g[3] + qb * g[4] + qc * g[5];
-            const float b = qdphi * Kphif + g[6] * st.wide.dtau_k;
-            const float a2 = q02 * Kphif;
-            q[0] += f2d_bits(-g[0] * Kpsif - g[3] * a2 + qa * b);
-            q[1] += f2d_bits(-g[1] * Kpsif - g[4] * a2 + qb * b);
-            q[2] += f2d_bits(-g[2] * Kpsif - g[5] * a2 + qc * b);
-            kicked = true;
+    for (int p = 0; p < P; ++p) ok[p] = false;
+    if (all) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            ok[p] = w_kick<SERIES>(n0[p].h, n0[p].l, st.wide.fmuh[s[p]], st.wide.fmul[s[p]], st.wide.fpsi, st.wide.fphi,
+                                   Kpsi[p], Kphi[p]);
+            all &= ok[p];
         }
     }
-    if (moved) {
-        __stcs(xd + i, x[0]);
-        __stcs(xd + n + i, x[1]);
-        __stcs(xd + 2 * n + i, x[2]);
-    }
-    if (kicked) {
-        __stcs(qd + i, q[0]);
-        __stcs(qd + n + i, q[1]);
-        __stcs(qd + 2 * n + i, q[2]);
+    if (!all) {
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            if (ok[p]) continue;
+            const float2 K = kick_fp64<SERIES>(st, s[p], a.n_kick, n0[p].s);
+            Kpsi[p] = K.x;
+            Kphi[p] = K.y;
+        }
     }
 }
 
-// P particles per thread in lockstep (i0 + 32 p, p < P; i0 < n): their chains are
-// independent, so the FP64 pipe overlaps one particle's result latencies with the
-// others' work.  A particle at or past n repeats particle i0's work and stores nothing.
+// P particles through the sub-steps of a pass of the FP64-state form, in lockstep (i0 + 32 p,
+// p < P; i0 < n): their chains are independent, so one particle's result latencies overlap
+// with the others' work.  A particle at or past n repeats particle i0's work and stores
+// nothing.
 template <typename Gt, bool SERIES, bool UNI, int P>
 __device__ __forceinline__ void wide_particles(const PushArgs& a, double* __restrict__ xd, double* __restrict__ qd,
                                                const float* __restrict__ q0f, int64_t i0)
@@ -862,11 +942,12 @@ __device__ __forceinline__ void wide_particles(const PushArgs& a, double* __rest
     const int64_t n = a.n;
     const uint32_t N = (uint32_t)a.N;
     const float invh = (float)a.invh;
-    const long long Lbits = __double_as_longlong(a.L);
+    const unsigned long long Lbits = (unsigned long long)__double_as_longlong(a.L);
     int64_t idx[P];
     bool ok[P];
     int s[P];
-    double x[P][3], q[P][3], s0[P];
+    double x[P][3], q[P][3];
+    Norm0 n0[P];
     float q0[P][3], q02[P];
 #pragma unroll
     for (int p = 0; p < P; ++p) {
@@ -881,41 +962,36 @@ __device__ __forceinline__ void wide_particles(const PushArgs& a, double* __rest
             q[p][d] = __ldcs(qd + d * n + i);
             q0[p][d] = __ldcs(q0f + d * n + i);
         }
-        const double da = f2d_bits(q0[p][0]), db = f2d_bits(q0[p][1]), dc = f2d_bits(q0[p][2]);
-        s0[p] = fma(da, da, fma(db, db, dc * dc));
-        q02[p] = d2f_bits(s0[p]);
+        n0[p] = norm0(a, q0[p][0], q0[p][1], q0[p][2], q02[p]);
     }
     bool moved = false, kicked = false;
     for (int u = 0; u < a.nsub; ++u) {
         const SubStep& st = a.sub[u];
-        float Kpsif[P], Kphif[P];
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-            Kpsif[p] = 0.f;
-            Kphif[p] = 0.f;
-            if (st.do_kick) kick_integrals<SERIES>(st, s[p], a.n_kick, s0[p], Kpsif[p], Kphif[p]);
-        }
         if (st.do_drift) {
+            double D[P];
+            drift_integrals<SERIES>(st, s, a.n_gl, q, D);
 #pragma unroll
-            for (int p = 0; p < P; ++p) {
-                const double D = drift_integral<SERIES>(st, s[p], a.n_gl, q[p]);
+            for (int p = 0; p < P; ++p)
 #pragma unroll
-                for (int d = 0; d < 3; ++d) x[p][d] = wrap_rare(fma(q[p][d], D, x[p][d]), a.L, a.invL, Lbits);
-            }
+                for (int d = 0; d < 3; ++d) x[p][d] = fma(q[p][d], D[p], x[p][d]);
+            wrap_rare(x, a.L, a.invL, Lbits);
             moved = true;
         }
         if (st.do_kick) {
+            float Kpsi[P], Kphi[P];
+            kick_integrals<SERIES>(a, st, s, n0, Kpsi, Kphi);
 #pragma unroll
             for (int p = 0; p < P; ++p) {
                 float g[8];
                 gather_wide<Gt>(a.order, reinterpret_cast<const Gt*>(a.G[u]), N, invh, x[p], g);
+                const float Kpsif = Kpsi[p], Kphif = Kphi[p];
                 const float qa = q0[p][0], qb = q0[p][1], qc = q0[p][2];
                 const float qdphi = qa * g[3] + qb * g[4] + qc * g[5];
-                const float b = qdphi * Kphif[p] + g[6] * st.wide.dtau_k;
-                const float a2 = q02[p] * Kphif[p];
-                q[p][0] += f2d_bits(-g[0] * Kpsif[p] - g[3] * a2 + qa * b);
-                q[p][1] += f2d_bits(-g[1] * Kpsif[p] - g[4] * a2 + qb * b);
-                q[p][2] += f2d_bits(-g[2] * Kpsif[p] - g[5] * a2 + qc * b);
+                const float b = qdphi * Kphif + g[6] * st.wide.dtau_k;
+                const float a2 = q02[p] * Kphif;
+                q[p][0] += f2d_bits(-g[0] * Kpsif - g[3] * a2 + qa * b);
+                q[p][1] += f2d_bits(-g[1] * Kpsif - g[4] * a2 + qb * b);
+                q[p][2] += f2d_bits(-g[2] * Kpsif - g[5] * a2 + qc * b);
             }
             kicked = true;
         }
@@ -934,9 +1010,10 @@ __device__ __forceinline__ void wide_particles(const PushArgs& a, double* __rest
 }
 
 // The pass kernel: P particles per thread, with three resident blocks per SM for P = 1
-// (80 registers, 24 warps) and two for P = 2 (128 registers, 16 warps carrying 32
-// particles each); the second shape measured faster (its pairs give the FP64 pipe two
-// independent chains per thread to overlap).  Work is handed out at run time, 32 P
+// (80 registers, 24 warps) and two for P = 2 (128 registers, 16 warps carrying 64
+// particles each).  Trilinear reads: 376 ms (P = 2) against 378 (P = 1) on 3 x 256^3
+// particles; order-2 reads, whose 27 cells P = 1's third block hides better: 43.2
+// against 40.5 ms on 2 x 101^3 particles, 250 steps.  Work is handed out at run time, 32 P
 // consecutive particles to a warp at a time (a.ctr[0] counts the chunks taken; each
 // warp claims its next chunk before working on the current one, so that the atomic's
 // round trip overlaps the work): the pass ends together on every SM however its
@@ -959,10 +1036,7 @@ __global__ void __launch_bounds__(kThreads, P == 2 ? 2 : 3) k_push_wide(const __
         if (i0 >= a.n) break;
         if (lane == 0) next = (unsigned)atomicAdd(a.ctr, 1ull);
         const int64_t i = i0 + lane;
-        if (i < a.n) {
-            if constexpr (P == 1) wide_particle<Gt, SERIES, UNI>(a, xd, qd, q0f, i);
-            else wide_particles<Gt, SERIES, UNI, P>(a, xd, qd, q0f, i);
-        }
+        if (i < a.n) wide_particles<Gt, SERIES, UNI, P>(a, xd, qd, q0f, i);
     }
     if (lane == 0) {
         const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x / 32);
@@ -988,25 +1062,26 @@ __global__ void __launch_bounds__(kThreads, 3) k_push_wide_multi(const __grid_co
         while (k + 1 < m.nseg && g >= m.seg[k + 1].begin) ++k;
         const MultiPass::Seg& sg = m.seg[k];
         const PushArgs& a = *sg.args;
-        if (a.wide_series) wide_particle<Gt, true, false>(a, sg.xd, sg.qd, sg.q0f, g - sg.begin);
-        else wide_particle<Gt, false, false>(a, sg.xd, sg.qd, sg.q0f, g - sg.begin);
+        if (a.wide_series) wide_particles<Gt, true, false, 1>(a, sg.xd, sg.qd, sg.q0f, g - sg.begin);
+        else wide_particles<Gt, false, false, 1>(a, sg.xd, sg.qd, sg.q0f, g - sg.begin);
     }
+}
+
+template <typename Gt, bool SERIES, int P>
+void push_wide_p(cudaStream_t s, unsigned b, const PushArgs& a, const ParticleState& st)
+{
+    if (a.uniform_species) launch_pass(k_push_wide<Gt, SERIES, true, P>, b, s, a, st.xd, st.qd, st.q0f);
+    else launch_pass(k_push_wide<Gt, SERIES, false, P>, b, s, a, st.xd, st.qd, st.q0f);
 }
 
 template <typename Gt>
 void push_wide(cudaStream_t s, unsigned b, const PushArgs& a, const ParticleState& st)
 {
-    // two particles per thread with the fitted integrals (the node loops keep one)
-    if (a.pair && a.wide_series) {
-        if (a.uniform_species) launch_pass(k_push_wide<Gt, true, true, 2>, b, s, a, st.xd, st.qd, st.q0f);
-        else launch_pass(k_push_wide<Gt, true, false, 2>, b, s, a, st.xd, st.qd, st.q0f);
-    } else if (a.wide_series) {
-        if (a.uniform_species) launch_pass(k_push_wide<Gt, true, true, 1>, b, s, a, st.xd, st.qd, st.q0f);
-        else launch_pass(k_push_wide<Gt, true, false, 1>, b, s, a, st.xd, st.qd, st.q0f);
-    } else {
-        if (a.uniform_species) launch_pass(k_push_wide<Gt, false, true, 1>, b, s, a, st.xd, st.qd, st.q0f);
-        else launch_pass(k_push_wide<Gt, false, false, 1>, b, s, a, st.xd, st.qd, st.q0f);
-    }
+    // two particles per thread with the fitted integrals (the node sums keep one: 22.1 ms
+    // with two, 19.6 ms with one on 160^3 particles, 100 steps)
+    if (!a.wide_series) push_wide_p<Gt, false, 1>(s, b, a, st);
+    else if (a.pair) push_wide_p<Gt, true, 2>(s, b, a, st);
+    else push_wide_p<Gt, true, 1>(s, b, a, st);
 }
 
 // ---- the fused leapfrog pass, plain FP64 form --------------------------------

@@ -1,0 +1,175 @@
+// wide_math.cuh -- FP64 results of the FP64-state particle pass computed on the FP32 and
+// integer pipes, bit for bit.
+//
+// GB300 issues two FP64 instructions per clock and SM against 128 FP32 or integer ones, so
+// an FP64 instruction costs as much as 64 others.  The two functions here give the bits of
+// an FP64 formula without its FP64 instructions: each forms the formula's last, rounded
+// value with some bits to spare and a bound on its distance from what FP64 arithmetic
+// gets; where that value lies so near a rounding boundary that the bound could cross it
+// (one evaluation in 2^11 or rarer), it says so and the caller runs the FP64 formula.
+//   w_rsqrt53: rsqrt_fp64's four FP64 instructions (~50 others);
+//   w_kick:    the kick's integrals as the FP32 values their user reads (9 FP64
+//              instructions as polynomials, 8 per node as sums).
+// tests/test_wide_math.py compares both with the FP64 formulas, bit for bit.
+//
+// Plain C++ besides the intrinsics, so that the test compiles it for the host.
+#pragma once
+
+#include <cstdint>
+
+namespace fdf {
+
+#define FDF_DEV __device__ __forceinline__
+
+// ---- rsqrt_fp64 (device_math.cuh) in integers -------------------------------------------
+// For v in the FP32 normal range and its FP32 estimate yf = rsqrtf(d2f_bits(v)), the bits of
+//   r = fma(y, s, y),  s = eh + 1.5f eh^2,  eh = fma(-(v y), y/2, 0.5)
+// v = m 4^k with 1 <= m < 4 and y = h 2^-k: every operation scales exactly, so m and h
+// serve as integers M 2^-52 and Y 2^-24 (54 and 24 bits).  m h is rounded to 53 bits as
+// FP64 rounds it; eh is exact (FP64 drops at most two of its bits); the FP32 term 1.5f eh^2
+// is formed in FP32 as well; h s and the final sum are exact to 2^-69.  What FP64 rounds
+// differently before the final rounding (eh and s below 2^-76, the FP32 square below
+// 2^-66) amounts to less than 12 of these units; the final rounding is at 2^-53, so a
+// value within 16 units of a tie (33 of 65536) is left to FP64, as is one whose
+// intermediate values leave the binades assumed (m within 2^-20 of 1 or 4).
+FDF_DEV bool w_rsqrt53(double v, float yf, double& r)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    const int ex = (int)(hi >> 20) - 1023, k = ex >> 1, odd = ex & 1;
+    const uint32_t m1 = (hi & 0xFFFFFu) | 0x100000u;
+    const uint32_t Mh = odd ? (m1 << 1) | (lo >> 31) : m1, Ml = lo << odd;
+    const uint32_t yb = __float_as_uint(yf);
+    const uint32_t Y = (yb & 0x7FFFFFu) | 0x800000u;
+    bool ok = (int)(yb >> 23) + k == 126;                        // 1/2 <= h < 1
+    // V = m h in units of 2^-52, rounded to nearest, ties to even
+    const uint64_t a = (uint64_t)Ml * Y;
+    const uint64_t b = (uint64_t)Mh * Y + (a >> 32);
+    const uint32_t al = (uint32_t)a, bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
+    uint64_t V = ((uint64_t)__funnelshift_l(bl, bh, 8) << 32) | __funnelshift_l(al, bl, 8);
+    V += (al >> 23) & (uint32_t)((al & 0x7FFFFFu) != 0u || (V & 1u));
+    const uint32_t Vh = (uint32_t)(V >> 32), Vl = (uint32_t)V;
+    ok = ok && (Vh >> 20) == 1u;                                 // 1 <= m h < 2
+    // E = 1/2 - V h / 2 in units of 2^-77 (the low 64 bits hold it)
+    const int64_t E = -(int64_t)((uint64_t)Vl * Y + ((uint64_t)(Vh * Y) << 32));
+    const float eh = __fmul_rn(__int2float_rn((int)(E >> 25)), 2.220446049250313081e-16f);   // 2^-52
+    const float kap = __fmul_rn(__fmul_rn(1.5f, eh), eh);
+    // h (E + kap) in units of 2^-69
+    const float h69 = __fmul_rn(__uint2float_rn(Y), 35184372088832.f);                       // h 2^69
+    const int64_t W = (int64_t)(int)Y * (int)(E >> 32) + (int64_t)(((uint64_t)(uint32_t)E * Y) >> 32) +
+                      __float2int_rn(__fmul_rn(kap, h69));
+    ok = ok && ((uint32_t)W & 0xFFFFu) - (0x8000u - 16u) > 32u;
+    const int64_t R = ((int64_t)Y << 29) + ((W + 0x8000) >> 16); // r 2^k in units of 2^-53
+    const uint32_t Rh = (uint32_t)(R >> 32);
+    ok = ok && (Rh >> 20) == 1u;
+    r = __hiloint2double((int)(Rh + ((uint32_t)(1021 - k) << 20)), (int)(uint32_t)R);
+    return ok;
+}
+
+// ---- pairs of floats (value = hi + lo, 48 bits) -----------------------------------------
+FDF_DEV void w_two_sum(float a, float b, float& s, float& e)
+{
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+
+// (sh, sl) = c + t (sh, sl)
+FDF_DEV void w_horner(float ch, float cl, float th, float tl, float& sh, float& sl)
+{
+    const float p = __fmul_rn(th, sh);
+    float e = __fmaf_rn(th, sh, -p);
+    e = __fmaf_rn(th, sl, e);
+    e = __fmaf_rn(tl, sh, e);
+    float l;
+    w_two_sum(ch, p, sh, l);
+    sl = __fadd_rn(l, __fadd_rn(cl, e));
+}
+
+// ---- the kick's integrals ---------------------------------------------------------------
+// Polynomials in t = m^2 a_c^2 / u_0 (WideCoef says of what), coefficients h[k] + l[k].
+constexpr int kKickDeg = 10;    // highest degree
+// SERIES: the pass's fitted polynomials (c_0 in FP64, the others FP32), evaluated as the
+// FP64 formula does: u^(-1/2) to first order, t and the terms above c_0 in FP32.
+// !SERIES: the sums over the nodes themselves, from polynomials that agree with them to
+// 2^-47 (wide_poly.cuh); c_1 .. c_6 as pairs.
+template <bool SERIES> struct KickLen {
+    static constexpr int kDeg = SERIES ? 5 : 10;
+    static constexpr int kPair = SERIES ? 1 : 7;
+};
+struct KickPoly {
+    float h[kKickDeg + 1], l[kKickDeg + 1];
+};
+
+// K_psi = u_0^(1/2) psi(t) and K_phi = u_0^(-1/2) phi(t) as FP32, u_0 = s_0 + mu, s_0 = |q_0|^2
+// and mu = m^2 a_c^2 as pairs in the run's momentum unit.  Pairs carry 2^-44 of the result;
+// the FP64 formula and the pairs differ by less than 2^-42, so a result that +-2^-41 does not
+// move to another float is FP64's (rounded to FP32).  Returns whether both are.
+template <bool SERIES>
+FDF_DEV bool w_kick(float s0h, float s0l, float muh, float mul, const KickPoly& psi, const KickPoly& phi, float& Kpsi,
+                    float& Kphi)
+{
+    float uh, ul;
+    w_two_sum(s0h, muh, uh, ul);
+    ul = __fadd_rn(ul, __fadd_rn(s0l, mul));
+    const float y = w_rsqrt(uh);
+    const float y2 = __fmul_rn(y, y), y2e = __fmaf_rn(y, y, -y2);
+    float e = __fmaf_rn(-uh, y2, 1.f);
+    e = __fmaf_rn(-uh, y2e, e);
+    e = __fmaf_rn(-ul, y2, e);
+    // u^(-1/2) = y (1 + c)
+    const float c = SERIES ? __fmul_rn(0.5f, e) : __fmul_rn(e, __fmaf_rn(0.375f, e, 0.5f));
+    bool ok = true;
+    float t, tl = 0.f;
+    if (SERIES) {
+        const float r = __fmaf_rn(y, c, y);
+        ok = __fmaf_rn(y, __fadd_rn(c, 2.2737368e-13f), y) == __fmaf_rn(y, __fsub_rn(c, 2.2737368e-13f), y);  // 2^-42
+        t = __fmul_rn(__fmul_rn(muh, r), r);
+    } else {
+        t = __fmul_rn(muh, y2);
+        tl = __fmaf_rn(muh, y2, -t);
+        tl = __fmaf_rn(muh, y2e, tl);
+        tl = __fmaf_rn(mul, y2, tl);
+        tl = __fmaf_rn(t, __fmaf_rn(e, e, e), tl);
+    }
+    constexpr int DEG = KickLen<SERIES>::kDeg, PAIR = KickLen<SERIES>::kPair;
+    float a = phi.h[DEG], b = psi.h[DEG], a1 = 0.f, b1 = 0.f;
+#pragma unroll
+    for (int k = DEG - 1; k >= PAIR; --k) {
+        a = __fmaf_rn(a, t, phi.h[k]);
+        b = __fmaf_rn(b, t, psi.h[k]);
+    }
+#pragma unroll
+    for (int k = PAIR - 1; k >= 1; --k) {
+        w_horner(phi.h[k], phi.l[k], t, tl, a, a1);
+        w_horner(psi.h[k], psi.l[k], t, tl, b, b1);
+    }
+    const float pa = __fmul_rn(a, t), pb = __fmul_rn(b, t);
+    float qa = __fmaf_rn(a, t, -pa), qb = __fmaf_rn(b, t, -pb);
+    if (!SERIES) {
+        qa = __fmaf_rn(a1, t, __fmaf_rn(a, tl, qa));
+        qb = __fmaf_rn(b1, t, __fmaf_rn(b, tl, qb));
+    }
+    const float ah = __fadd_rn(phi.h[0], pa), bh = __fadd_rn(psi.h[0], pb);
+    const float al = __fadd_rn(__fsub_rn(pa, __fsub_rn(ah, phi.h[0])), __fadd_rn(phi.l[0], qa));
+    const float bl = __fadd_rn(__fsub_rn(pb, __fsub_rn(bh, psi.h[0])), __fadd_rn(psi.l[0], qb));
+    // K_phi = y (1 + c) (ah + al)
+    float h = __fmul_rn(y, ah);
+    float l = __fmaf_rn(y, __fmaf_rn(ah, c, al), __fmaf_rn(y, ah, -h));
+    float d = __fmul_rn(h, 4.5474735e-13f);                      // 2^-41
+    Kphi = __fadd_rn(h, __fadd_rn(l, d));
+    ok = ok && Kphi == __fadd_rn(h, __fsub_rn(l, d));
+    // K_psi = u y (1 + c) (bh + bl)
+    const float w = __fmul_rn(uh, y);
+    float wl = __fmaf_rn(uh, y, -w);
+    wl = __fmaf_rn(ul, y, wl);
+    wl = __fmaf_rn(w, c, wl);
+    h = __fmul_rn(w, bh);
+    l = __fmaf_rn(w, bh, -h);
+    l = __fmaf_rn(w, bl, l);
+    l = __fmaf_rn(wl, bh, l);
+    d = __fmul_rn(h, 4.5474735e-13f);
+    Kpsi = __fadd_rn(h, __fadd_rn(l, d));
+    return ok && Kpsi == __fadd_rn(h, __fsub_rn(l, d));
+}
+
+}  // namespace fdf
