@@ -103,6 +103,58 @@ int auto_nodes(double dlna)
 }
 
 // ---- the FP64-state form's step integrals as polynomials (WideCoef) ---------------
+// Sums and products to ~104 bits as pairs of doubles (value = h + l): the fits below need
+// more than FP64 (their high coefficients cancel), and the host's long double is software
+// quad precision on the GPU's Arm CPUs, 40 times slower (1.0 ms a step for three fits).
+struct DD {
+    double h, l;
+};
+inline DD dd_add(DD a, DD b)
+{
+    const double s = a.h + b.h, bb = s - a.h;
+    const double e = (a.h - (s - bb)) + (b.h - bb) + (a.l + b.l);
+    const double h = s + e;
+    return {h, e - (h - s)};
+}
+inline DD dd_mul(DD a, DD b)
+{
+    const double p = a.h * b.h;
+    const double e = std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h);
+    const double h = p + e;
+    return {h, e - (h - p)};
+}
+
+// Chebyshev interpolation of degree K on [0, 1] as monomial coefficients: the values at t[i],
+// times m[k][i].
+struct FitTable {
+    int K;
+    double t[kWideDeg + 1];
+    DD m[kWideDeg + 1][kWideDeg + 1];
+    explicit FitTable(int K_) : K(K_)
+    {
+        const long double pi = 3.14159265358979323846264338327950288L;
+        // T_q(2t - 1) as polynomials in t: T_0 = 1, T_1 = 2t - 1, T_{q+1} = 2 (2t - 1) T_q - T_{q-1}
+        long double Tm1[kWideDeg + 2] = {1}, T[kWideDeg + 2] = {-1, 2}, mm[kWideDeg + 1][kWideDeg + 1] = {};
+        for (int q = 0; q <= K; ++q) {
+            for (int i = 0; i <= K; ++i) {
+                const long double c = std::cos(pi * q * (i + 0.5L) / (K + 1)) * (q ? 2 : 1) / (K + 1);
+                for (int k = 0; k <= q; ++k) mm[k][i] += c * Tm1[k];
+            }
+            long double Tn[kWideDeg + 2];
+            for (int k = 0; k <= kWideDeg + 1; ++k) Tn[k] = (k ? 4 * T[k - 1] : 0) - 2 * T[k] - Tm1[k];
+            std::memcpy(Tm1, T, sizeof(T));
+            std::memcpy(T, Tn, sizeof(T));
+        }
+        for (int i = 0; i <= K; ++i) {
+            t[i] = (double)((1.0L + std::cos(pi * (i + 0.5L) / (K + 1))) / 2);
+            for (int k = 0; k <= K; ++k) {
+                m[k][i].h = (double)mm[k][i];
+                m[k][i].l = (double)(mm[k][i] - (long double)m[k][i].h);
+            }
+        }
+    }
+};
+
 // g(t) = sum_j W_j (1 + e_j t)^power on t in [0, 1] (power -1/2 or +1/2), interpolated at
 // the Chebyshev points of [0, 1] and written as monomial coefficients in t.  The degree
 // is the smallest in [max(nf64, 3), kWideDeg] for which the polynomial agrees with the sum
@@ -112,65 +164,64 @@ int auto_nodes(double dlna)
 // then integrates node by node) if no degree does.
 bool fit_wide_poly(const double* W, const double* e, int n, double power, int nf64, double tol, WidePoly& P)
 {
+    static const FitTable tables[] = {FitTable(3), FitTable(4), FitTable(5), FitTable(6),
+                                      FitTable(7), FitTable(8), FitTable(9), FitTable(10)};
+    static_assert(kWideDeg == 10, "a table per degree from 3 to kWideDeg");
     std::memset(&P, 0, sizeof(P));
-    auto g = [&](long double t) {
-        long double v = 0;
+    auto g = [&](double t) {
+        DD v{0, 0};
         for (int j = 0; j < n; ++j) {
-            const double b = std::sqrt(1.0 + e[j] * (double)t);
-            v += (long double)W[j] * (power < 0 ? 1.0L / b : (long double)b);
+            const double b = std::sqrt(1.0 + e[j] * t);
+            const double q = power < 0 ? 1.0 / b : b;
+            const double r = power < 0 ? std::fma(-q, b, 1.0) / b : 0.0;      // 1/b = q + r
+            v = dd_add(v, dd_mul({q, r}, {W[j], 0}));
         }
         return v;
     };
     constexpr int kCheck = 64;   // check points t = i / kCheck
-    long double gmax = 0;
-    for (int i = 0; i <= kCheck; ++i) gmax = std::max(gmax, std::fabs(g((long double)i / kCheck)));
+    double gc[kCheck + 1], gmax = 0;
+    for (int i = 0; i <= kCheck; ++i) {
+        gc[i] = 0;
+        for (int j = 0; j < n; ++j) {
+            const double b = std::sqrt(1.0 + e[j] * ((double)i / kCheck));
+            gc[i] += power < 0 ? W[j] / b : W[j] * b;
+        }
+        gmax = std::max(gmax, std::fabs(gc[i]));
+    }
     if (gmax == 0) return true;
     for (int K = std::max(nf64, 3); K <= kWideDeg; ++K) {
-        // Chebyshev coefficients of g(t(s)), s = 2t - 1, from its values at the K + 1 points
-        long double cc[kWideDeg + 1] = {};
-        long double gv[kWideDeg + 1];
-        for (int i = 0; i <= K; ++i) {
-            const long double th = 3.14159265358979323846264338327950288L * (i + 0.5L) / (K + 1);
-            gv[i] = g((1.0L + std::cos(th)) / 2);
+        const FitTable& T = tables[K - 3];
+        DD gv[kWideDeg + 1], a[kWideDeg + 1];
+        for (int i = 0; i <= K; ++i) gv[i] = g(T.t[i]);
+        double tail = 0;
+        for (int k = 0; k <= K; ++k) {
+            a[k] = {0, 0};
+            for (int i = 0; i <= K; ++i) a[k] = dd_add(a[k], dd_mul(T.m[k][i], gv[i]));
+            if (k >= nf64) tail += std::fabs(a[k].h);
         }
-        for (int m = 0; m <= K; ++m) {
-            long double acc = 0;
-            for (int i = 0; i <= K; ++i)
-                acc += gv[i] * std::cos(3.14159265358979323846264338327950288L * m * (i + 0.5L) / (K + 1));
-            cc[m] = acc * 2 / (K + 1);
-        }
-        cc[0] /= 2;
-        // T_m(2t - 1) as polynomials in t: T_0 = 1, T_1 = 2t - 1, T_{m+1} = 2 (2t - 1) T_m - T_{m-1}
-        long double Tm1[kWideDeg + 2] = {}, Tm[kWideDeg + 2] = {}, a[kWideDeg + 1] = {};
-        Tm1[0] = 1;
-        Tm[0] = -1;
-        Tm[1] = 2;
-        a[0] += cc[0];
-        for (int m = 1; m <= K; ++m) {
-            for (int k = 0; k <= m; ++k) a[k] += cc[m] * Tm[k];
-            long double Tn[kWideDeg + 2] = {};
-            for (int k = 0; k <= m; ++k) {
-                Tn[k + 1] += 4 * Tm[k];
-                Tn[k] -= 2 * Tm[k];
-            }
-            for (int k = 0; k <= m + 1; ++k) Tn[k] -= Tm1[k];
-            std::memcpy(Tm1, Tm, sizeof(Tm));
-            std::memcpy(Tm, Tn, sizeof(Tn));
-        }
-        // the device's evaluation: FP64 coefficients below nf64, FP32 ones above
-        long double tail = 0;
-        for (int k = nf64; k <= K; ++k) tail += std::fabs(a[k]);
-        const long double tail_bound = tail * 4 * 5.9604644775390625e-8L;
-        long double err = 0;
+        const double tail_bound = tail * 4 * 5.9604644775390625e-8;
+        if (tail_bound > tol * gmax) continue;
+        // the device's evaluation: FP64 coefficients below nf64, FP32 ones above.  FP64
+        // settles the comparison unless it is closer than FP64's own error here.
+        double c[kWideDeg + 1], err = 0;
+        for (int k = 0; k <= K; ++k) c[k] = k < nf64 ? a[k].h : (double)(float)a[k].h;
         for (int i = 0; i <= kCheck; ++i) {
-            const long double t = (long double)i / kCheck;
-            long double pt = 0;
-            for (int k = K; k >= 0; --k) pt = pt * t + (k < nf64 ? (long double)(double)a[k] : (long double)(float)a[k]);
-            err = std::max(err, std::fabs(pt - g(t)));
+            double pt = 0;
+            for (int k = K; k >= 0; --k) pt = pt * ((double)i / kCheck) + c[k];
+            err = std::max(err, std::fabs(pt - gc[i]));
         }
-        if ((err + tail_bound) <= tol * gmax) {
-            for (int k = 0; k < nf64; ++k) P.c64[k] = (double)a[k];
-            for (int k = nf64; k <= K; ++k) P.c32[k - nf64] = (float)a[k];
+        if (std::fabs(err + tail_bound - tol * gmax) <= 4e-15 * gmax) {
+            err = 0;
+            for (int i = 0; i <= kCheck; ++i) {
+                const DD t{(double)i / kCheck, 0}, gi = g(t.h);
+                DD pt{0, 0};
+                for (int k = K; k >= 0; --k) pt = dd_add(dd_mul(pt, t), {c[k], 0});
+                err = std::max(err, std::fabs(dd_add(pt, {-gi.h, -gi.l}).h));
+            }
+        }
+        if (err + tail_bound <= tol * gmax) {
+            for (int k = 0; k < nf64; ++k) P.c64[k] = a[k].h;
+            for (int k = nf64; k <= K; ++k) P.c32[k - nf64] = (float)a[k].h;
             return true;
         }
     }
@@ -679,10 +730,10 @@ void fill_substep(fdf_ctx* c, bool drift, double d1, double d2, bool kick, doubl
                 e[j] = sc.mud[jc] > 0 ? (sc.mud[j] - sc.mud[jc]) / sc.mud[jc] : 0.0;
                 u.emax = std::max(u.emax, std::fabs(e[j]));
             }
-            // Cd_k = c_k sum_j Wd_j e_j^k with c_k the binomial coefficients of
+            // Cd_k = c_k sum_j Wd_j e_j^k (the split-state form's series) with c_k the binomial coefficients of
             // (1 + d)^(-1/2) - 1 = sum_k c_k d^k: c_1 = -1/2, c_k = c_(k-1) (1 - 2k)/(2k)
             double ck = 1.0;
-            for (int k = 1; k <= kTaylor; ++k) {
+            for (int k = 1; k <= kTaylor && form_of(c->p.precision) == kFixed; ++k) {
                 ck *= (1.0 - 2.0 * k) / (2.0 * k);
                 double m = 0;
                 for (int j = 0; j < c->ngl; ++j) m += Wd[j] * std::pow(e[j], k);
