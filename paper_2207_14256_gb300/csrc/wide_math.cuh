@@ -40,7 +40,8 @@ FDF_DEV bool w_rsqrt53(double v, float yf, double& r)
     const uint32_t Mh = odd ? (m1 << 1) | (lo >> 31) : m1, Ml = lo << odd;
     const uint32_t yb = __float_as_uint(yf);
     const uint32_t Y = (yb & 0x7FFFFFu) | 0x800000u;
-    bool ok = (int)(yb >> 23) + k == 126;                        // 1/2 <= h < 1
+    bool ok = hi - 0x38100000u < 0x0FE00000u;                    // v in the FP32 normal range
+    ok = ok && (int)(yb >> 23) + k == 126;                       // 1/2 <= h < 1
     // V = m h in units of 2^-52, rounded to nearest, ties to even
     const uint64_t a = (uint64_t)Ml * Y;
     const uint64_t b = (uint64_t)Mh * Y + (a >> 32);
