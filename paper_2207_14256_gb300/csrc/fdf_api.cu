@@ -254,7 +254,7 @@ constexpr int kMaxBuf = 2 * (kMaxSub - 1) + 1;
 int grid_buffers(const fdf_params& p) { return std::min(kMaxBuf, 2 * steps_per_pass(p) + 1); }
 
 struct Layout {
-    size_t tabs, modeA, noise, cdf_t, cdf_F, tw, W0, W1, G[kMaxBuf], Gss[2], qs, stage, dep, flag, ctr, key, hist, bsum,
+    size_t tabs, modeA, keys, noise, cdf_t, cdf_F, tw, W, G[kMaxBuf], Gss[2], qs, stage, dep, flag, ctr, key, hist, bsum,
         recs, total;
     int nbuf;
     StateLayout s[2];
@@ -279,13 +279,14 @@ Layout make_layout(const fdf_params& p, int nk, int na, int ncdf)
         return o;
     };
     L.tabs = take(3 * (size_t)na * nk * 8);
-    L.modeA = take(4 * (size_t)mode_table_size(p.n_grid) * real_bytes(prec));
+    // an amplitude table per grid of a pass (its steps and the opening half kick)
+    L.modeA = take((steps_per_pass(p) + 1) * 4 * (size_t)mode_table_size(p.n_grid) * real_bytes(prec));
+    L.keys = take((size_t)mode_table_size(p.n_grid) * sizeof(ModeKey));
     L.noise = take(N3 * complex_bytes(prec));
     L.cdf_t = take((size_t)ncdf * 8);
     L.cdf_F = take((size_t)ncdf * 8);
     L.tw = take(N * complex_bytes(prec));
-    L.W0 = take(4 * N3 * complex_bytes(prec));
-    L.W1 = take(4 * N3 * complex_bytes(prec));
+    L.W = take(4 * N3 * complex_bytes(prec));
     L.nbuf = grid_buffers(p);
     for (int b = 0; b < L.nbuf; ++b) L.G[b] = take(N3 * grid_bytes_per_cell(prec));
     // the two super-step grids an interpolated step reads (super-steps only)
@@ -430,14 +431,16 @@ struct fdf_ctx {
     char* block = nullptr;
     bool own_block = false;
     double* tabs = nullptr;   // FP64 [3][na][nk]
-    void* modeA = nullptr;    // per-step amplitude table
+    char* modeA = nullptr;    // amplitude tables, one per slot of a pass
+    ModeKey* keys = nullptr;  // the run's modes
+    int mode_count = 0;       // the scale factors (ln a) whose tables the slots hold
+    double mode_lna[kMaxSub] = {};
     void* noise = nullptr;    // unit Gaussian field of the run
     bool noise_ready = false;
     double* cdf_t = nullptr;
     double* cdf_F = nullptr;
     void* tw = nullptr;
-    void* W0 = nullptr;
-    void* W1 = nullptr;
+    void* W = nullptr;        // the transforms' work array
     int nbuf = 0;
     void* G[kMaxBuf] = {};
     int gk[kMaxBuf];                     // step index whose fields each buffer holds (-1: none)
@@ -758,15 +761,38 @@ void fill_substep(fdf_ctx* c, bool drift, double d1, double d2, bool kick, doubl
     if (form_of(c->p.precision) == kWide) fill_wide(c, drift, d1, d2, Wd, ad, kick, k1, k2, Wk, ak, u);
 }
 
-// The unit Gaussian field of the run (a function of the seed and the mesh only),
-// on the fields stream.
+FieldArgs field_args(const fdf_ctx* c, double lna)
+{
+    return make_field_args(c->p, c->nk, c->na, c->lnk0, c->dlnk, c->lnat0, c->dlnat, lna);
+}
+
+// The unit Gaussian field of the run (a function of the seed and the mesh only) and the
+// amplitudes of its modes, on the fields stream.
 int draw_noise(fdf_ctx* c)
 {
-    const FieldArgs a = make_field_args(c->p, c->nk, c->na, c->lnk0, c->dlnk, c->lnat0, c->dlnat, c->lna0);
+    const FieldArgs a = field_args(c, c->lna0);
     int rc = timed_on(c, c->sf, FDF_K_FIELDS_Z, "noise",
                       [&] { return launch_noise(c->sf, grid_prec(c->p.precision), a, c->noise); });
+    if (rc) return rc;
+    rc = timed_on(c, c->sf, FDF_K_FIELDS_Z, "mode keys", [&] { return launch_mode_keys(c->sf, a, c->keys); });
     if (rc == FDF_OK) c->noise_ready = true;
+    c->mode_count = 0;
     return rc;
+}
+
+// The amplitude tables of scale factors lna[0..count) into the slots, on stream s.
+int mode_tables(fdf_ctx* c, const double* lna, int count, cudaStream_t s)
+{
+    ModeSteps st{};
+    for (int i = 0; i < count; ++i) st.add(field_args(c, lna[i]));
+    c->mode_count = 0;
+    int rc = timed_on(c, s, FDF_K_FIELDS_Z, "mode tables", [&] {
+        return launch_mode_tables(s, grid_prec(c->p.precision), field_args(c, c->lna0), st, c->keys, c->tabs, c->modeA);
+    });
+    if (rc) return rc;
+    std::copy(lna, lna + count, c->mode_lna);
+    c->mode_count = count;
+    return FDF_OK;
 }
 
 // The eight fields at ln a into G, on stream s; slot 7 as `slot7` says (kSlot7*).
@@ -778,20 +804,24 @@ int build_fields(fdf_ctx* c, double lna, void* G, cudaStream_t s, int slot7)
         if (rc0) return rc0;
         if (s != c->sf) FDF_CUDA(cudaStreamSynchronize(c->sf), "sync");
     }
-    FieldArgs a = make_field_args(c->p, c->nk, c->na, c->lnk0, c->dlnk, c->lnat0, c->dlnat, lna);
+    int slot = 0;
+    while (slot < c->mode_count && c->mode_lna[slot] != lna) ++slot;
+    if (slot == c->mode_count) {
+        int rc0 = mode_tables(c, &lna, 1, s);
+        if (rc0) return rc0;
+        slot = 0;
+    }
+    FieldArgs a = field_args(c, lna);
     a.slot7 = slot7;
-    const int prec = grid_prec(c->p.precision);
-    int rc = timed_on(c, s, FDF_K_FIELDS_Z, "mode table",
-                      [&] { return launch_mode_table(s, prec, a, c->tabs, c->modeA); });
+    const int prec = grid_prec(c->p.precision), N = c->p.n_grid;
+    const void* A = c->modeA + (size_t)slot * 4 * mode_table_size(N) * real_bytes(c->p.precision);
+    int rc = timed_on(c, s, FDF_K_FIELDS_Z, "fields z pass",
+                      [&] { return launch_fields_z(s, prec, a, A, c->noise, c->tw, c->W); });
     if (rc) return rc;
-    rc = timed_on(c, s, FDF_K_FIELDS_Z, "fields z pass",
-                  [&] { return launch_fields_z(s, prec, a, c->modeA, c->noise, c->tw, c->W0); });
-    if (rc) return rc;
-    rc = timed_on(c, s, FDF_K_FIELDS_Y, "fields y pass",
-                  [&] { return launch_fields_y(s, prec, a, c->tw, c->W0, c->W1); });
+    rc = timed_on(c, s, FDF_K_FIELDS_Y, "fields y pass", [&] { return launch_fields_y(s, prec, N, c->tw, c->W); });
     if (rc) return rc;
     return timed_on(c, s, FDF_K_FIELDS_X, "fields x pass",
-                    [&] { return launch_fields_x(s, prec, a, c->tw, c->W1, G); });
+                    [&] { return launch_fields_x(s, prec, N, c->tw, c->W, G); });
 }
 
 int push(fdf_ctx* c, const PushArgs& a)
@@ -1163,12 +1193,12 @@ int fdf_create(const fdf_params* p, const fdf_tables* t, void* stream, void* are
     char* b = c->block;
     c->tabs = (double*)(b + L.tabs);
     c->modeA = b + L.modeA;
+    c->keys = (ModeKey*)(b + L.keys);
     c->noise = b + L.noise;
     c->cdf_t = (double*)(b + L.cdf_t);
     c->cdf_F = (double*)(b + L.cdf_F);
     c->tw = b + L.tw;
-    c->W0 = b + L.W0;
-    c->W1 = b + L.W1;
+    c->W = b + L.W;
     c->nbuf = L.nbuf;
     c->spp = steps_per_pass(c->p);
     for (int i = 0; i < kMaxBuf; ++i) c->gk[i] = -1;
@@ -1340,6 +1370,15 @@ int slice_prepare(fdf_ctx* c, int j, std::vector<int>& bufs, std::vector<const v
     std::vector<int> ks;
     if (j == 0) ks.push_back(sl.k_start);                       // the opening half kick
     for (int i = 0; i < pass_len(c, j); ++i) ks.push_back(sl.k_start + sl.dir * (pass_first(c, j) + i + 1));
+    if (!c->frozen && !c->supersteps && c->noise_ready) {
+        // the amplitude tables of all grids to build, in one launch
+        double lna[kMaxSub];
+        int count = 0;
+        for (int kk : ks)
+            if (find_grid(c, kk) < 0) lna[count++] = c->lna(kk);
+        int rc = count > 1 ? mode_tables(c, lna, count, c->sf) : FDF_OK;
+        if (rc) return rc;
+    }
     for (int kk : ks) {
         const void* G = nullptr;
         int b = -1;
@@ -1540,6 +1579,7 @@ int fdf_run_graph(fdf_ctx* c, int32_t n)
         FDF_CUDA(cudaStreamSynchronize(c->stream), "fdf_run_graph");
         FDF_CUDA(cudaStreamSynchronize(c->sf), "fdf_run_graph");
         for (int b = 0; b < kMaxBuf; ++b) c->has_release[b] = false;
+        c->mode_count = 0;
         const int64_t l0 = c->launches, s0 = c->sorts;
         FDF_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeRelaxed), "beginning the capture");
         // the fields stream joins the capture through an event of the main stream
@@ -1565,6 +1605,7 @@ int fdf_run_graph(fdf_ctx* c, int32_t n)
         if (rc != FDF_OK) {
             // the host state describes a run that never executed
             c->sampled = c->stepped = false;
+            c->mode_count = 0;
             for (int b = 0; b < kMaxBuf; ++b) {
                 c->gk[b] = -1;
                 c->has_release[b] = false;
@@ -1597,6 +1638,7 @@ int fdf_run_graph(fdf_ctx* c, int32_t n)
     std::memcpy(c->gk, g.gk, sizeof(g.gk));
     std::memcpy(c->ssk, g.ssk, sizeof(g.ssk));
     for (int b = 0; b < kMaxBuf; ++b) c->has_release[b] = false;
+    c->mode_count = 0;
     c->slot7 = g.slot7;
     c->k = g.k;
     c->disp = g.disp;

@@ -208,20 +208,35 @@ cudaError_t launch_sample(cudaStream_t s, int64_t n, uint32_t key0, uint32_t key
                           const double* cdf_F, int ncdf, uint32_t* X, double* qs, double* pmag, uint32_t* id,
                           int* flag);
 
-// Field build: three passes.  precision: FDF_PREC_*.  W0/W1 are two complex
-// work arrays of 4 N^3 elements (float2 or double2), G the gather grid.
-// Per-step amplitude table A[4 M] (M = mode_table_size(N)) from the FP64
-// tables [3][na][nk]; read by the z pass.
+// Field build: three passes.  precision: FDF_PREC_*.  W is a complex work array of
+// 4 N^3 elements (float2 or double2), G the gather grid.
+// Amplitude tables A[count][4 M] (M = mode_table_size(N)) of count scale factors from the
+// FP64 tables [3][na][nk] and the keys of the run's modes; read by the z pass.
+struct ModeKey {
+    double amp, fk;             // sqrt(P_R(k)/V); fraction between ln k nodes ik and ik + 1
+    int ik, pad;
+};
+struct ModeSteps {              // the scale factors: FieldArgs' ia, fa and aH of each
+    int count;
+    int ia[kMaxSub];
+    double fa[kMaxSub], aH[kMaxSub];
+    void add(const FieldArgs& a)
+    {
+        ia[count] = a.ia;
+        fa[count] = a.fa;
+        aH[count++] = a.aH;
+    }
+};
 int mode_table_size(int N);
-cudaError_t launch_mode_table(cudaStream_t s, int precision, const FieldArgs& a, const double* tabs64, void* A);
+cudaError_t launch_mode_keys(cudaStream_t s, const FieldArgs& a, ModeKey* keys);
+cudaError_t launch_mode_tables(cudaStream_t s, int precision, const FieldArgs& a, const ModeSteps& st, const ModeKey* keys,
+                               const double* tabs64, void* A);
 // The unit Gaussian field R_n / sqrt(P_R/V) on the N^3 mode array (drawn once per run).
 cudaError_t launch_noise(cudaStream_t s, int precision, const FieldArgs& a, void* R);
 cudaError_t launch_fields_z(cudaStream_t s, int precision, const FieldArgs& a, const void* A, const void* R,
                             const void* tw, void* W0);
-cudaError_t launch_fields_y(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, const void* W0,
-                            void* W1);
-cudaError_t launch_fields_x(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, const void* W1,
-                            void* G);
+cudaError_t launch_fields_y(cudaStream_t s, int precision, int N, const void* tw, void* W);
+cudaError_t launch_fields_x(cudaStream_t s, int precision, int N, const void* tw, const void* W, void* G);
 // G (any precision) <-> [8][N^3] FP64; to_f64 writes the slots whose bit is set in mask.
 cudaError_t launch_fields_to_f64(cudaStream_t s, int precision, int N, const void* G, double* out,
                                  unsigned mask = 0xFFu);

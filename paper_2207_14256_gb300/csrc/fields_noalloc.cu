@@ -72,12 +72,11 @@ extern "C" int fdf_build_fields_noalloc(const fdf_params* p, const fdf_tables* t
     const size_t N = (size_t)p->n_grid, N3 = N * N * N;
     const size_t csz = f64 ? 16 : 8, rsz = f64 ? 8 : 4;
     const size_t ntab = 3 * (size_t)t->na * t->nk;
-    // scratch layout: W0 | W1 | FP64 tables | amplitude table | twiddles | noise; the
-    // interleaved grid G of the last pass reuses W0 (same size or smaller).
+    // scratch layout: W | G | FP64 tables | amplitude table | twiddles | noise | mode keys
     const size_t M = (size_t)mode_table_size(p->n_grid);
     const size_t oW0 = 0, oW1 = oW0 + align256(4 * N3 * csz), oT64 = oW1 + align256(4 * N3 * csz);
     const size_t oA = oT64 + align256(ntab * 8), oTw = oA + align256(4 * M * rsz), oR = oTw + align256(N * csz);
-    const size_t need = oR + align256(N3 * csz);
+    const size_t oK = oR + align256(N3 * csz), need = oK + align256(M * sizeof(ModeKey));
     if (need > FDF_NOALLOC_SCRATCH_BYTES) {
         char msg[200];
         snprintf(msg, sizeof msg,
@@ -108,15 +107,18 @@ extern "C" int fdf_build_fields_noalloc(const fdf_params* p, const fdf_tables* t
     void* W0 = s + oW0;
     void* W1 = s + oW1;
     if (e == cudaSuccess) e = launch_noise(st, gp, a, s + oR);
-    if (e == cudaSuccess) e = launch_mode_table(st, gp, a, T64, s + oA);
+    ModeSteps step{};
+    step.add(a);
+    if (e == cudaSuccess) e = launch_mode_keys(st, a, (ModeKey*)(s + oK));
+    if (e == cudaSuccess) e = launch_mode_tables(st, gp, a, step, (const ModeKey*)(s + oK), T64, s + oA);
     // as fdf_build_fields: slots 0-6 from a build with phi_dot transformed alone, slot 7
     // (psi) from a second build
     for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
         a.slot7 = pass == 0 ? kSlot7Zero : kSlot7Psi;
         e = launch_fields_z(st, gp, a, s + oA, s + oR, s + oTw, W0);
-        if (e == cudaSuccess) e = launch_fields_y(st, gp, a, s + oTw, W0, W1);
-        if (e == cudaSuccess) e = launch_fields_x(st, gp, a, s + oTw, W1, W0);
-        if (e == cudaSuccess) e = launch_fields_to_f64(st, gp, p->n_grid, W0, out, pass == 0 ? 0x7Fu : 0x80u);
+        if (e == cudaSuccess) e = launch_fields_y(st, gp, p->n_grid, s + oTw, W0);
+        if (e == cudaSuccess) e = launch_fields_x(st, gp, p->n_grid, s + oTw, W0, W1);
+        if (e == cudaSuccess) e = launch_fields_to_f64(st, gp, p->n_grid, W1, out, pass == 0 ? 0x7Fu : 0x80u);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess)

@@ -157,15 +157,25 @@ template <int N> struct Shape {
         constexpr int S = TXl < P ? P / TXl : 1;
         return TS0 + ((S - TS0 % P) % P + P) % P;
     }
-    // x pass: TL lines per block, lane = t + T lo; stride TSX = T (mod 16).
-    static constexpr int TL0 = 128 / T;
-    static constexpr int TL = TL0 < N ? TL0 : N;
-    static constexpr int THREADS_X = TL * T;
+    // x pass: XL lines of each of the four grids per block (256 threads, 128 for N <= 16),
+    // lane = t + T (line); transpose stride TSX = T (mod 16), result rows of XPS elements.
+    static constexpr int XL0 = (N <= 16 ? 128 : 256) / (4 * T);
+    static constexpr int XL = XL0 < N * N ? XL0 : N * N;
+    static constexpr int THREADS_X = 4 * XL * T;
     static constexpr int SX = T % 16;
     static constexpr int TSX = TS0 + ((SX - TS0 % 16) + 16) % 16;
+    static constexpr int XPS = N;
+    template <typename V> static constexpr size_t x_smem()
+    {
+        return (size_t)(N2 * (N1 + 1) + 4 * XL * (TSX > XPS ? TSX : XPS)) * sizeof(V);
+    }
     static constexpr int TWS = N2 * (N1 + 1);                  // per-thread twiddle rows, padded
-    // z pass: 128 threads (its per-thread amplitudes live in shared memory).
-    static constexpr int TZ0 = 128 / T;
+    // z pass: 128 threads (its per-thread amplitudes live in shared memory) that form all four
+    // packed grids in turn.  Up to N = 64 that would be N^2 T / 128 <= 256 blocks of a long
+    // chain for 152 SMs: there a block is 8 columns of one grid (N = 32 in FP64: 512 blocks of
+    // 32 threads for 32 of 128, 28 -> 13 us a pass).
+    static constexpr bool kSplitGrids = N <= 64;
+    static constexpr int TZ0 = kSplitGrids ? 8 : 128 / T;
     static constexpr int TZ = TZ0 < N ? TZ0 : N;
     static constexpr int THREADS_Z = TZ * T;
 };
@@ -278,46 +288,61 @@ __device__ __forceinline__ V packed(int p, V R, typename Real<V>::T Apsi, typena
     }
 }
 
-// Per scale factor, in FP64, for every m = |n|^2 in [0, M): k = k_f sqrt(m),
-// the amplitude sqrt(P_R(k)/V) = sqrt(2 pi^2 A_s / V) k^-3/2 (k/k_pivot)^((n_s-1)/2)
-// times T_psi, T_phi and a H dT_phi/dln a, read bilinearly in (ln k, ln a) with
-// clamping from the FP64 tables [3][na][nk].
-template <typename T>
-__global__ void __launch_bounds__(256) k_mode_table(FieldArgs a, int M, const double* __restrict__ tabs,
-                                                    T* __restrict__ A)
+// In FP64, for every m = |n|^2 in [0, M): k = k_f sqrt(m), the amplitude sqrt(P_R(k)/V) =
+// sqrt(2 pi^2 A_s / V) k^-3/2 (k/k_pivot)^((n_s-1)/2) and k's place in the transfer tables'
+// uniform ln k grid (clamped): what no step changes.  Once per run: its chain of a root, a
+// logarithm, an exponential and a division takes 10 us however small the grid is.
+__global__ void __launch_bounds__(256) k_mode_keys(FieldArgs a, int M, ModeKey* __restrict__ keys)
 {
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
-        double v[3] = {0.0, 0.0, 0.0};
+        ModeKey key{0.0, 0.0, 0, 0};
         if (m > 0) {
             const double k = a.kf * sqrt((double)m);
             const double lnk = log(k);
-            const double amp = a.amp0 / (k * sqrt(k)) * exp(a.half_nsm1 * (lnk - a.lnkp));
+            key.amp = a.amp0 / (k * sqrt(k)) * exp(a.half_nsm1 * (lnk - a.lnkp));
             const double pos = (lnk - a.lnk0) * a.inv_dlnk;
-            int ik;
-            double fk;
             if (pos <= 0.0) {
-                ik = 0;
-                fk = 0.0;
+                key.ik = 0;
+                key.fk = 0.0;
             } else if (pos >= a.nk - 1) {
-                ik = a.nk - 2;
-                fk = 1.0;
+                key.ik = a.nk - 2;
+                key.fk = 1.0;
             } else {
-                ik = (int)pos;
-                fk = pos - ik;
+                key.ik = (int)pos;
+                key.fk = pos - key.ik;
             }
-            for (int t = 0; t < 3; ++t) {
-                const double* r0 = tabs + ((size_t)t * a.na + a.ia) * a.nk;
-                const double* r1 = r0 + a.nk;
-                const double v0 = (1.0 - fk) * r0[ik] + fk * r0[ik + 1];
-                const double v1 = (1.0 - fk) * r1[ik] + fk * r1[ik + 1];
-                v[t] = amp * ((1.0 - a.fa) * v0 + a.fa * v1);
-            }
-            v[2] *= a.aH;
         }
-        A[4 * m] = (T)v[0];
-        A[4 * m + 1] = (T)v[1];
-        A[4 * m + 2] = (T)v[2];
-        A[4 * m + 3] = T(0);
+        keys[m] = key;
+    }
+}
+
+// Per scale factor and m: the amplitude times T_psi, T_phi and a H dT_phi/dln a, read
+// bilinearly in (ln k, ln a) from the FP64 tables [3][na][nk].  One launch makes the tables
+// of every step of a pass (blockIdx.y).
+template <typename T>
+__global__ void __launch_bounds__(256) k_mode_tables(const __grid_constant__ ModeSteps st, int M, int nk, int na,
+                                                     const ModeKey* __restrict__ keys, const double* __restrict__ tabs,
+                                                     T* __restrict__ A)
+{
+    const int b = blockIdx.y;
+    const double fa = st.fa[b], aH = st.aH[b];
+    T* out = A + (size_t)b * 4 * M;
+    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
+        const ModeKey key = keys[m];
+        double v[3];
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+            const double* r0 = tabs + ((size_t)t * na + st.ia[b]) * nk;
+            const double* r1 = r0 + nk;
+            const double v0 = (1.0 - key.fk) * r0[key.ik] + key.fk * r0[key.ik + 1];
+            const double v1 = (1.0 - key.fk) * r1[key.ik] + key.fk * r1[key.ik + 1];
+            v[t] = key.amp * ((1.0 - fa) * v0 + fa * v1);
+        }
+        v[2] *= aH;
+        out[4 * m] = (T)v[0];
+        out[4 * m + 1] = (T)v[1];
+        out[4 * m + 2] = (T)v[2];
+        out[4 * m + 3] = T(0);
     }
 }
 
@@ -391,8 +416,10 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, sizeof(V) == 8 ? 4 : 2) k
     }
     __syncthreads();
     const size_t N3 = NN * N;
+    // this block's packed grids: all four, or one of gridDim.z
+    const int p0 = gridDim.z == 1 ? 0 : blockIdx.z, p1 = gridDim.z == 1 ? 4 : p0 + 1;
 #pragma unroll 1
-    for (int p = 0; p < 4; ++p) {
+    for (int p = p0; p < p1; ++p) {
         // one branch per packed grid, so that each reads only the amplitudes it uses
         // (psi; psi and phi; phi; phi_dot and psi) from shared memory
         V v[N1];
@@ -428,11 +455,10 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, sizeof(V) == 8 ? 4 : 2) k
 }
 
 // ---- pass y: inverse DFT along y --------------------------------------------
-// Block (x-tile, jz, packed grid p): TX lines along y, read and written in rows of
-// TX consecutive x.
+// Block (x-tile, jz, packed grid p): TX lines along y, read and written in place in rows
+// of TX consecutive x.
 template <typename V, int N>
-__global__ void __launch_bounds__(Shape<N>::THREADS) k_fields_y(FieldArgs a, const V* __restrict__ tw,
-                                                                const V* __restrict__ W0, V* __restrict__ W1)
+__global__ void __launch_bounds__(Shape<N>::THREADS) k_fields_y(const V* __restrict__ tw, V* W)
 {
     using S = Shape<N>;
     constexpr int TX = S::TX, N1 = S::N1, N2 = S::N2;
@@ -444,27 +470,18 @@ __global__ void __launch_bounds__(Shape<N>::THREADS) k_fields_y(FieldArgs a, con
     const int xo = threadIdx.x % TX, t = threadIdx.x / TX;
     const int x0 = blockIdx.x * TX, jz = blockIdx.y, p = blockIdx.z;
     const size_t N3 = (size_t)N * N * N;
-    const V* src = W0 + p * N3 + (size_t)jz * N * N + x0 + xo;
+    V* dst = W + p * N3 + (size_t)jz * N * N + x0 + xo;
     V v[N1];
-    sfor<N1>([&](auto N1i) { v[N1i] = src[(size_t)(N2 * N1i + t) * N]; });
+    sfor<N1>([&](auto N1i) { v[N1i] = dst[(size_t)(N2 * N1i + t) * N]; });
     __syncthreads();
     line_first<V, N>(v, t, s_tw, tr + xo * TS);
     __syncthreads();
-    V* dst = W1 + p * N3 + (size_t)jz * N * N + x0 + xo;
     line_second<V, N>(t, tr + xo * TS, [&](int y, V val) { dst[(size_t)y * N] = val; });
 }
 
 // ---- pass x: inverse DFT along x, interleave into G[cell][8] ----------------
-// Block: TL consecutive x-lines (line index = jz * N + jy).  FP64 records go out in
-// two halves: grid 0 is parked in shared memory and written with grid 1, grid 2
-// with grid 3 (one parked grid instead of three doubles the resident blocks).  FP32
-// and BF16 records go out in one piece: grids 0..2 are parked and written with grid 3.
 template <typename Gt, typename V> struct GRec;
-// FP64 records (64 bytes) are written in two halves (grids 0-1, then grids 2-3), each
-// two whole 32-byte sectors; FP32 and BF16 records in one piece, which measured faster
-// for them (FP32 halves: 232 -> 310 us per x pass at 256^3).
 template <> struct GRec<float, float2> {
-    static constexpr bool kHalves = false;
     // one 32-byte store per record (the record is 32-byte aligned)
     __device__ static void put(float* G, size_t cell, float2 a, float2 b, float2 c, float2 d)
     {
@@ -475,16 +492,17 @@ template <> struct GRec<float, float2> {
     }
 };
 template <> struct GRec<double, double2> {
-    static constexpr bool kHalves = true;
-    __device__ static void put_half(double* G, size_t cell, int h, double2 a, double2 b)
+    // two 32-byte stores per record
+    __device__ static void put(double* G, size_t cell, double2 a, double2 b, double2 c, double2 d)
     {
-        double2* g = reinterpret_cast<double2*>(G) + 4 * cell + 2 * h;
-        g[0] = a;
-        g[1] = b;
+        double* g = G + 8 * cell;
+        asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(g), "d"(a.x), "d"(a.y), "d"(b.x), "d"(b.y)
+                     : "memory");
+        asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(g + 4), "d"(c.x), "d"(c.y), "d"(d.x), "d"(d.y)
+                     : "memory");
     }
 };
 template <> struct GRec<__nv_bfloat16, float2> {
-    static constexpr bool kHalves = false;
     __device__ static void put(__nv_bfloat16* G, size_t cell, float2 a, float2 b, float2 c, float2 d)
     {
         const __nv_bfloat162 h0 = __floats2bfloat162_rn(a.x, a.y), h1 = __floats2bfloat162_rn(b.x, b.y);
@@ -498,57 +516,49 @@ template <> struct GRec<__nv_bfloat16, float2> {
     }
 };
 
+// Block: XL consecutive x-lines (line index = jz * N + jy) of all four packed grids, one
+// line of one grid per T threads.  The transforms end in shared memory ([line][grid][x],
+// over the transpose buffers), from where each cell's four values leave as one whole
+// record.  Every grid's threads work at once: with one set of threads that transformed
+// the grids in turn and parked three of them, 69 KB of shared memory held 128 threads.
+// Bound by DRAM at N = 256 (48 (BF16) or 64 (FP32) bytes per cell): BF16 records 164 ->
+// 120 us; N = 128 in FP32 28.9 -> 23.8 us, N = 32 in FP64 22.9 -> 12.5 us.
 template <typename V, typename Gt, int N>
-__global__ void __launch_bounds__(Shape<N>::THREADS_X) k_fields_x(FieldArgs a, const V* __restrict__ tw,
-                                                                  const V* __restrict__ W1, Gt* __restrict__ G)
+__global__ void __launch_bounds__(Shape<N>::THREADS_X) k_fields_x(const V* __restrict__ tw, const V* __restrict__ W,
+                                                                  Gt* __restrict__ G)
 {
     using S = Shape<N>;
-    using Rec = GRec<Gt, V>;
-    constexpr int TL = S::TL, N1 = S::N1, N2 = S::N2, T = S::T, LS = N + 1;
+    constexpr int XL = S::XL, N1 = S::N1, N2 = S::N2, T = S::T, PS = S::XPS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* s_tw = reinterpret_cast<V*>(smem_raw);
-    V* tr = s_tw + S::TWS;          // TL * TSX
-    V* park = tr + TL * S::TSX;     // TL * LS per parked grid (1 for halves, else 3)
-    load_line_twiddles<V, N>(s_tw, tw);
-    const int t = threadIdx.x % T, lo = threadIdx.x / T;
+    V* tr = s_tw + S::TWS;          // 4 XL TSX transpose elements, then 4 XL PS results
+    const int t = threadIdx.x % T, lp = threadIdx.x / T;
+    const int lo = lp % XL, p = lp / XL;
     const size_t N3 = (size_t)N * N * N;
-    const size_t line = (size_t)blockIdx.x * TL + lo;
-    // the next packed grid's line is loaded while this one is transformed
-    V nxt[N1];
-    sfor<N1>([&](auto N1i) { nxt[N1i] = W1[line * N + N2 * N1i + t]; });
-#pragma unroll 1
-    for (int p = 0; p < 4; ++p) {
-        V v[N1];
-        sfor<N1>([&](auto N1i) { v[N1i] = nxt[N1i]; });
-        if (p < 3) {
-            const V* src = W1 + (p + 1) * N3 + line * N;
-            sfor<N1>([&](auto N1i) { nxt[N1i] = src[N2 * N1i + t]; });
-        }
-        __syncthreads();
-        line_first<V, N>(v, t, s_tw, tr + lo * S::TSX);
-        __syncthreads();
-        if constexpr (Rec::kHalves) {
-            // each thread parks and reads back only its own x values: no barrier needed
-            V* pk = park + lo * LS;
-            if ((p & 1) == 0) {
-                line_second<V, N>(t, tr + lo * S::TSX, [&](int x, V val) { pk[x] = val; });
-            } else {
-                const int h = p >> 1;
-                line_second<V, N>(t, tr + lo * S::TSX,
-                                  [&](int x, V val) { Rec::put_half(G, line * N + x, h, pk[x], val); });
-            }
-        } else {
-            if (p < 3) {
-                V* pk = park + (p * TL + lo) * LS;
-                line_second<V, N>(t, tr + lo * S::TSX, [&](int x, V val) { pk[x] = val; });
-            } else {
-                const V* p0 = park + lo * LS;
-                const V* p1 = park + (TL + lo) * LS;
-                const V* p2 = park + (2 * TL + lo) * LS;
-                line_second<V, N>(t, tr + lo * S::TSX,
-                                  [&](int x, V val) { Rec::put(G, line * N + x, p0[x], p1[x], p2[x], val); });
-            }
-        }
+    const size_t line0 = (size_t)blockIdx.x * XL;
+    V v[N1];
+    const V* src = W + p * N3 + (line0 + lo) * N;
+    sfor<N1>([&](auto N1i) { v[N1i] = src[N2 * N1i + t]; });
+    load_line_twiddles<V, N>(s_tw, tw);
+    __syncthreads();
+    line_first<V, N>(v, t, s_tw, tr + lp * S::TSX);
+    __syncthreads();
+    V r[N1];
+    sfor<S::G>([&](auto Gi) {
+        V u[N2];
+        sfor<N2>([&](auto N2i) { u[N2i] = tr[lp * S::TSX + N2i * (N1 + 1) + t + Gi * N2]; });
+        dft_reg<N2>(u);
+        sfor<N2>([&](auto K2) { r[Gi * N2 + K2] = u[K2]; });
+    });
+    __syncthreads();
+    V* park = tr + (lo * 4 + p) * PS;
+    sfor<S::G>([&](auto Gi) { sfor<N2>([&](auto K2) { park[t + Gi * N2 + N1 * K2] = r[Gi * N2 + K2]; }); });
+    __syncthreads();
+#pragma unroll
+    for (int c = threadIdx.x; c < XL * N; c += S::THREADS_X) {
+        const int l = c / N, x = c % N;
+        const V* q = tr + l * 4 * PS + x;
+        GRec<Gt, V>::put(G, (line0 + l) * N + x, q[0], q[PS], q[2 * PS], q[3 * PS]);
     }
 }
 
@@ -593,32 +603,30 @@ cudaError_t run_z(cudaStream_t s, const FieldArgs& a, const void* A, const void*
     const size_t sm = (size_t)(S::TWS + S::TZ * TSZ) * sizeof(V) + (size_t)3 * S::N1 * S::THREADS_Z * sizeof(T);
     cudaError_t e = set_smem(k_fields_z<V, N>, sm);
     if (e != cudaSuccess) return e;
-    k_fields_z<V, N><<<dim3(N / S::TZ, N), S::THREADS_Z, sm, s>>>(a, (const T*)A, (const V*)R, (const V*)tw, (V*)W0);
+    k_fields_z<V, N><<<dim3(N / S::TZ, N, S::kSplitGrids ? 4 : 1), S::THREADS_Z, sm, s>>>(a, (const T*)A, (const V*)R, (const V*)tw, (V*)W0);
     return cudaGetLastError();
 }
 
 template <typename V, int N>
-cudaError_t run_y(cudaStream_t s, const FieldArgs& a, const void* tw, const void* W0, void* W1)
+cudaError_t run_y(cudaStream_t s, const void* tw, void* W)
 {
     using S = Shape<N>;
     constexpr int TS = S::template line_stride<sizeof(V), S::TX>();
     const size_t sm = (size_t)(S::TWS + S::TX * TS) * sizeof(V);
     cudaError_t e = set_smem(k_fields_y<V, N>, sm);
     if (e != cudaSuccess) return e;
-    k_fields_y<V, N><<<dim3(N / S::TX, N, 4), S::THREADS, sm, s>>>(a, (const V*)tw, (const V*)W0, (V*)W1);
+    k_fields_y<V, N><<<dim3(N / S::TX, N, 4), S::THREADS, sm, s>>>((const V*)tw, (V*)W);
     return cudaGetLastError();
 }
 
 template <typename V, typename Gt, int N>
-cudaError_t run_x(cudaStream_t s, const FieldArgs& a, const void* tw, const void* W1, void* G)
+cudaError_t run_x(cudaStream_t s, const void* tw, const void* W, void* G)
 {
     using S = Shape<N>;
-    const int parked = GRec<Gt, V>::kHalves ? 1 : 3;
-    const size_t sm = (size_t)(S::TWS + S::TL * S::TSX + parked * S::TL * (N + 1)) * sizeof(V);
+    const size_t sm = S::template x_smem<V>();
     cudaError_t e = set_smem(k_fields_x<V, Gt, N>, sm);
     if (e != cudaSuccess) return e;
-    k_fields_x<V, Gt, N><<<(unsigned)((size_t)N * N / S::TL), S::THREADS_X, sm, s>>>(a, (const V*)tw, (const V*)W1,
-                                                                                    (Gt*)G);
+    k_fields_x<V, Gt, N><<<(unsigned)((size_t)N * N / S::XL), S::THREADS_X, sm, s>>>((const V*)tw, (const V*)W, (Gt*)G);
     return cudaGetLastError();
 }
 
@@ -697,12 +705,21 @@ cudaError_t launch_interp_grid(cudaStream_t s, int precision, int N, const void*
     return cudaGetLastError();
 }
 
-cudaError_t launch_mode_table(cudaStream_t s, int precision, const FieldArgs& a, const double* tabs64, void* A)
+cudaError_t launch_mode_keys(cudaStream_t s, const FieldArgs& a, ModeKey* keys)
 {
     const int M = mode_table_size(a.N);
-    const unsigned blocks = (unsigned)((M + 255) / 256);
-    if (precision == FDF_PREC_F64) k_mode_table<double><<<blocks, 256, 0, s>>>(a, M, tabs64, (double*)A);
-    else k_mode_table<float><<<blocks, 256, 0, s>>>(a, M, tabs64, (float*)A);
+    k_mode_keys<<<(unsigned)((M + 255) / 256), 256, 0, s>>>(a, M, keys);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mode_tables(cudaStream_t s, int precision, const FieldArgs& a, const ModeSteps& st, const ModeKey* keys,
+                               const double* tabs64, void* A)
+{
+    if (st.count < 1 || st.count > kMaxSub) return cudaErrorInvalidValue;
+    const int M = mode_table_size(a.N);
+    const dim3 g((unsigned)((M + 255) / 256), (unsigned)st.count);
+    if (precision == FDF_PREC_F64) k_mode_tables<double><<<g, 256, 0, s>>>(st, M, a.nk, a.na, keys, tabs64, (double*)A);
+    else k_mode_tables<float><<<g, 256, 0, s>>>(st, M, a.nk, a.na, keys, tabs64, (float*)A);
     return cudaGetLastError();
 }
 
@@ -726,26 +743,24 @@ cudaError_t launch_fields_z(cudaStream_t s, int precision, const FieldArgs& a, c
 #undef Z32
 }
 
-cudaError_t launch_fields_y(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, const void* W0,
-                            void* W1)
+cudaError_t launch_fields_y(cudaStream_t s, int precision, int N, const void* tw, void* W)
 {
-#define Y64(n) run_y<double2, n>(s, a, tw, W0, W1)
-#define Y32(n) run_y<float2, n>(s, a, tw, W0, W1)
-    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(a.N, Y64)
-    FDF_DISPATCH_N(a.N, Y32)
+#define Y64(n) run_y<double2, n>(s, tw, W)
+#define Y32(n) run_y<float2, n>(s, tw, W)
+    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(N, Y64)
+    FDF_DISPATCH_N(N, Y32)
 #undef Y64
 #undef Y32
 }
 
-cudaError_t launch_fields_x(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, const void* W1,
-                            void* G)
+cudaError_t launch_fields_x(cudaStream_t s, int precision, int N, const void* tw, const void* W, void* G)
 {
-#define X64(n) run_x<double2, double, n>(s, a, tw, W1, G)
-#define X32(n) run_x<float2, float, n>(s, a, tw, W1, G)
-#define X16(n) run_x<float2, __nv_bfloat16, n>(s, a, tw, W1, G)
-    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(a.N, X64)
-    if (precision == FDF_PREC_F32) FDF_DISPATCH_N(a.N, X32)
-    FDF_DISPATCH_N(a.N, X16)
+#define X64(n) run_x<double2, double, n>(s, tw, W, G)
+#define X32(n) run_x<float2, float, n>(s, tw, W, G)
+#define X16(n) run_x<float2, __nv_bfloat16, n>(s, tw, W, G)
+    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(N, X64)
+    if (precision == FDF_PREC_F32) FDF_DISPATCH_N(N, X32)
+    FDF_DISPATCH_N(N, X16)
 #undef X64
 #undef X32
 #undef X16
