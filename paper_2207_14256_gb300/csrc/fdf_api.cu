@@ -600,10 +600,8 @@ void fill_pass(const fdf_ctx* c, PushArgs& a)
     a.wide_series = 1;
     a.q_unit2 = (float)(c->q_unit * c->q_unit);
     for (int s = 0; s < kMaxSpecies; ++s) a.m2[s] = c->p.m_ev[s] * c->p.m_ev[s];
-    // order-2 reads run faster with three blocks of one particle per thread (k_push_wide)
-    const int pb = c->p.pass_blocks > 0 ? c->p.pass_blocks : a.order == 2 ? 3 : 2;
-    a.grid_blocks = c->sm_count * pb;
-    a.pair = pb == 2 ? 1 : 0;
+    // three blocks fit; 1 leaves room on the SMs for other work
+    a.grid_blocks = c->sm_count * (c->p.pass_blocks == 1 ? 1 : 3);
     a.ctr = c->pass_ctr;
     a.tile_gather = c->p.gather_tile > 0 ? 1 : 0;
     a.N = c->p.n_grid;
@@ -1476,8 +1474,6 @@ int slice_next(fdf_ctx* c, PushArgs& a)
     }
     const int form = form_of(c->p.precision);
     if (form == kWide) {
-        // the node sums have one particle per thread, so three of their blocks are resident
-        if (!a.wide_series && a.pair) a.grid_blocks = c->sm_count * 3;
         a.kick_fast = a.wide_series ? kKickSeries : kKickNodes;
         for (int u = 0; u < a.nsub; ++u) {
             fill_kick_fast(c, a.wide_series != 0, a.sub[u]);

@@ -767,33 +767,28 @@ void push_split(cudaStream_t s, unsigned b, const PushArgs& a, const ParticleSta
 // than 1e-7 of the integral).  The kick, at most ~1e-3 of |q| per step, is formed in
 // FP32 from the FP32 gradients and added to q in FP64.
 //
-// Bound: the FP64 pipe.  GB300 runs FP64 arithmetic and FP64 <-> FP32 conversions at 1/64
-// of its FP32 rate, so conversions are bit operations (d2f_bits, f2d_bits), and the
-// inverse square roots and the kick's integrals get the bits of their FP64 formulas from
-// the integer and FP32 pipes (wide_math.cuh): 17 FP64 instructions per particle-step (|q|^2
-// 3, v 1, t 1, polynomial 5, D 1, x 3, q 3), 30 with the formulas in FP64.  3 x 256^3
-// particles, 200 steps, passes of 8: 563 -> 376 ms in the pass; node sums, 160^3
-// particles, 100 steps: 61.4 -> 19.6 ms.  A stage handles all P particles of a thread
-// before its rare branch, so that their chains interleave (422 ms with a branch each).
+// GB300 runs FP64 arithmetic and FP64 <-> FP32 conversions at 1/64 of its FP32 rate, so
+// conversions are bit operations (d2f_bits, f2d_bits), and the inverse square roots, their
+// squares, the kick's integrals and q's sums get the bits of their FP64 formulas from the
+// integer and FP32 pipes (wide_math.cuh): 13 FP64 instructions per particle-step (|q|^2 3,
+// v 1, polynomial 5, D 1, x 3), 30 with everything in FP64.  3 x 256^3 particles, 200
+// steps, passes of 8: 563 -> 341 ms in the pass; node sums, 160^3 particles, 100 steps:
+// 61.4 -> 19.7 ms.
 
 // Periodic wrap into [0, L) (wrap_f64, a result equal to L mapping to 0), taken only
 // when x left the box.  The test runs on the bit patterns (IEEE doubles order like
 // integers when positive; a negative value, as an unsigned integer, is above them all),
 // so only a warp with a wrapping particle spends FP64 instructions on it.
-template <int P>
-__device__ __forceinline__ void wrap_rare(double (&x)[P][3], double L, double invL, unsigned long long Lbits)
+__device__ __forceinline__ void wrap_rare(double x[3], double L, double invL)
 {
+    const unsigned long long Lbits = (unsigned long long)__double_as_longlong(L);
     bool out = false;
 #pragma unroll
-    for (int p = 0; p < P; ++p)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) out |= (unsigned long long)__double_as_longlong(x[p][d]) >= Lbits;
+    for (int d = 0; d < 3; ++d) out |= (unsigned long long)__double_as_longlong(x[d]) >= Lbits;
     if (out) {
 #pragma unroll
-        for (int p = 0; p < P; ++p)
-#pragma unroll
-            for (int d = 0; d < 3; ++d)
-                if ((unsigned long long)__double_as_longlong(x[p][d]) >= Lbits) x[p][d] = wrap_f64(x[p][d], L, invL);
+        for (int d = 0; d < 3; ++d)
+            if ((unsigned long long)__double_as_longlong(x[d]) >= Lbits) x[d] = wrap_f64(x[d], L, invL);
     }
 }
 
@@ -811,55 +806,64 @@ __device__ __forceinline__ double wide_poly(const WidePoly& P, double t, float t
     return acc;
 }
 
-// rsqrt_fp64 of P values without its FP64 instructions, except for the few arguments that
-// w_rsqrt53 leaves to it (one branch for all P, so that their chains interleave).
-template <int P>
-__device__ __forceinline__ void rsqrt_int(const double (&u)[P], double (&r)[P])
+// rsqrt_fp64 without its FP64 instructions, except for the few arguments that
+// w_rsqrt53 leaves to it.
+__device__ __forceinline__ double rsqrt_int(double u)
 {
-    bool ok[P], all = true;
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-        ok[p] = w_rsqrt53(u[p], rsqrtf(d2f_bits(u[p])), r[p]);
-        all &= ok[p];
-    }
-    if (!all) {
-#pragma unroll
-        for (int p = 0; p < P; ++p)
-            if (!ok[p]) r[p] = rsqrt_fp64(u[p]);
-    }
+    double r;
+    if (!w_rsqrt53(u, rsqrtf(d2f_bits(u)), r)) r = rsqrt_fp64(u);
+    return r;
 }
 
-// The drift integrals of one sub-step.
-template <bool SERIES, int P>
-__device__ __forceinline__ void drift_integrals(const SubStep& st, const int (&s)[P], int n_gl, const double (&q)[P][3],
-                                                double (&D)[P])
+// The same with t = r * r.
+__device__ __forceinline__ double rsqrt_int(double u, double& t)
 {
-    double qq[P], u[P], r[P];
+    double r;
+    int64_t R;
+    int k;
+    const bool ok = w_rsqrt53(u, rsqrtf(d2f_bits(u)), r, R, k);
+    t = w_square53(R, k);
+    if (!ok) {
+        r = rsqrt_fp64(u);
+        t = r * r;
+    }
+    return r;
+}
+
+// q += d, one branch for the few sums that w_add leaves to FP64.
+__device__ __forceinline__ void add_small(double q[3], const float d[3])
+{
+    double r[3];
+    bool ok[3];
 #pragma unroll
-    for (int p = 0; p < P; ++p) qq[p] = fma(q[p][0], q[p][0], fma(q[p][1], q[p][1], q[p][2] * q[p][2]));
+    for (int c = 0; c < 3; ++c) ok[c] = w_add(q[c], d[c], r[c]);
+    if (!(ok[0] && ok[1] && ok[2])) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            if (!ok[c]) r[c] = q[c] + f2d_bits(d[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) q[c] = r[c];
+}
+
+// The drift integral of one sub-step.
+template <bool SERIES>
+__device__ __forceinline__ double drift_integral(const SubStep& st, int s, int n_gl, const double q[3])
+{
+    const double qq = fma(q[0], q[0], fma(q[1], q[1], q[2] * q[2]));
     if constexpr (SERIES) {
         // v = 1 + |q|^2 / (m^2 a_c^2), t = 1/v, D = v^(-1/2) gm(t) / (m a_c); a massless
         // species takes D = |q|^-1 sum_j W_j
-#pragma unroll
-        for (int p = 0; p < P; ++p)
-            u[p] = st.wide.massless[s[p]] ? qq[p] : fma(qq[p], st.wide.inv_muc[s[p]], 1.0);
-        rsqrt_int(u, r);
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-            const double t = r[p] * r[p];
-            const double g = wide_poly<kWideD64>(st.wide.drift[s[p]], t, d2f_bits(t));
-            D[p] = r[p] * (st.wide.massless[s[p]] ? st.wide.wsum[s[p]] : g);
-        }
+        const bool massless = st.wide.massless[s];
+        double t;
+        const double r = rsqrt_int(massless ? qq : fma(qq, st.wide.inv_muc[s], 1.0), t);
+        const double g = wide_poly<kWideD64>(st.wide.drift[s], t, d2f_bits(t));
+        return r * (massless ? st.wide.wsum[s] : g);
     } else {
-#pragma unroll
-        for (int p = 0; p < P; ++p) D[p] = 0.0;
-        for (int j = 0; j < n_gl; ++j) {
-#pragma unroll
-            for (int p = 0; p < P; ++p) u[p] = qq[p] + st.sp[s[p]].mud[j];
-            rsqrt_int(u, r);
-#pragma unroll
-            for (int p = 0; p < P; ++p) D[p] = fma(st.sp[s[p]].Wd[j], r[p], D[p]);
-        }
+        const SpeciesCoef& sc = st.sp[s];
+        double D = 0.0;
+        for (int j = 0; j < n_gl; ++j) D = fma(sc.Wd[j], rsqrt_int(qq + sc.mud[j]), D);
+        return D;
     }
 }
 
@@ -911,139 +915,91 @@ __device__ __forceinline__ Norm0 norm0(const PushArgs& a, float qa, float qb, fl
     return n;
 }
 
-template <bool SERIES, int P>
-__device__ __forceinline__ void kick_integrals(const PushArgs& a, const SubStep& st, const int (&s)[P],
-                                               const Norm0 (&n0)[P], float (&Kpsi)[P], float (&Kphi)[P])
+template <bool SERIES>
+__device__ __forceinline__ void kick_integrals(const PushArgs& a, const SubStep& st, int s, const Norm0& n0,
+                                               float& Kpsi, float& Kphi)
 {
     constexpr int FAST = SERIES ? kKickSeries : kKickNodes;
-    bool ok[P], all = a.kick_fast == FAST;
-#pragma unroll
-    for (int p = 0; p < P; ++p) ok[p] = false;
-    if (all) {
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-            ok[p] = w_kick<SERIES>(n0[p].h, n0[p].l, st.wide.fmuh[s[p]], st.wide.fmul[s[p]], st.wide.fpsi, st.wide.fphi,
-                                   Kpsi[p], Kphi[p]);
-            all &= ok[p];
-        }
-    }
-    if (!all) {
-#pragma unroll
-        for (int p = 0; p < P; ++p) {
-            if (ok[p]) continue;
-            const float2 K = kick_fp64<SERIES>(st, s[p], a.n_kick, n0[p].s);
-            Kpsi[p] = K.x;
-            Kphi[p] = K.y;
-        }
+    if (!(a.kick_fast == FAST && w_kick<SERIES>(n0.h, n0.l, st.wide.fmuh[s], st.wide.fmul[s], st.wide.fpsi,
+                                                st.wide.fphi, Kpsi, Kphi))) {
+        const float2 K = kick_fp64<SERIES>(st, s, a.n_kick, n0.s);
+        Kpsi = K.x;
+        Kphi = K.y;
     }
 }
 
-// P particles through the sub-steps of a pass of the FP64-state form, in lockstep (i0 + 32 p,
-// p < P; i0 < n): their chains are independent, so one particle's result latencies overlap
-// with the others' work.  A particle at or past n repeats particle i0's work and stores
-// nothing.
-template <typename Gt, bool SERIES, bool UNI, int P>
-__device__ __forceinline__ void wide_particles(const PushArgs& a, double* __restrict__ xd, double* __restrict__ qd,
-                                               const float* __restrict__ q0f, int64_t i0)
+// One particle through the sub-steps of a pass of the FP64-state form.
+template <typename Gt, bool SERIES, bool UNI>
+__device__ __forceinline__ void wide_particle(const PushArgs& a, double* __restrict__ xd, double* __restrict__ qd,
+                                              const float* __restrict__ q0f, int64_t i)
 {
     const int64_t n = a.n;
     const uint32_t N = (uint32_t)a.N;
     const float invh = (float)a.invh;
-    const unsigned long long Lbits = (unsigned long long)__double_as_longlong(a.L);
-    int64_t idx[P];
-    bool ok[P];
-    int s[P];
-    double x[P][3], q[P][3];
-    Norm0 n0[P];
-    float q0[P][3], q02[P];
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-        idx[p] = i0 + 32 * p;
-        ok[p] = idx[p] < n;
-        if (!ok[p]) idx[p] = i0;
-        const int64_t i = idx[p];
-        s[p] = UNI ? 0 : species_of(a, i);
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            x[p][d] = __ldcs(xd + d * n + i);
-            q[p][d] = __ldcs(qd + d * n + i);
-            q0[p][d] = __ldcs(q0f + d * n + i);
-        }
-        n0[p] = norm0(a, q0[p][0], q0[p][1], q0[p][2], q02[p]);
-    }
+    const int s = UNI ? 0 : species_of(a, i);
+    double x[3] = {__ldcs(xd + i), __ldcs(xd + n + i), __ldcs(xd + 2 * n + i)};
+    double q[3] = {__ldcs(qd + i), __ldcs(qd + n + i), __ldcs(qd + 2 * n + i)};
+    const float qa = __ldcs(q0f + i), qb = __ldcs(q0f + n + i), qc = __ldcs(q0f + 2 * n + i);
+    float q02;
+    const Norm0 n0 = norm0(a, qa, qb, qc, q02);
     bool moved = false, kicked = false;
     for (int u = 0; u < a.nsub; ++u) {
         const SubStep& st = a.sub[u];
         if (st.do_drift) {
-            double D[P];
-            drift_integrals<SERIES>(st, s, a.n_gl, q, D);
+            const double D = drift_integral<SERIES>(st, s, a.n_gl, q);
 #pragma unroll
-            for (int p = 0; p < P; ++p)
-#pragma unroll
-                for (int d = 0; d < 3; ++d) x[p][d] = fma(q[p][d], D[p], x[p][d]);
-            wrap_rare(x, a.L, a.invL, Lbits);
+            for (int d = 0; d < 3; ++d) x[d] = fma(q[d], D, x[d]);
+            wrap_rare(x, a.L, a.invL);
             moved = true;
         }
         if (st.do_kick) {
-            float Kpsi[P], Kphi[P];
-            kick_integrals<SERIES>(a, st, s, n0, Kpsi, Kphi);
-#pragma unroll
-            for (int p = 0; p < P; ++p) {
-                float g[8];
-                gather_wide<Gt>(a.order, reinterpret_cast<const Gt*>(a.G[u]), N, invh, x[p], g);
-                const float Kpsif = Kpsi[p], Kphif = Kphi[p];
-                const float qa = q0[p][0], qb = q0[p][1], qc = q0[p][2];
-                const float qdphi = qa * g[3] + qb * g[4] + qc * g[5];
-                const float b = qdphi * Kphif + g[6] * st.wide.dtau_k;
-                const float a2 = q02[p] * Kphif;
-                q[p][0] += f2d_bits(-g[0] * Kpsif - g[3] * a2 + qa * b);
-                q[p][1] += f2d_bits(-g[1] * Kpsif - g[4] * a2 + qb * b);
-                q[p][2] += f2d_bits(-g[2] * Kpsif - g[5] * a2 + qc * b);
-            }
+            float Kpsif, Kphif, g[8];
+            kick_integrals<SERIES>(a, st, s, n0, Kpsif, Kphif);
+            gather_wide<Gt>(a.order, reinterpret_cast<const Gt*>(a.G[u]), N, invh, x, g);
+            const float qdphi = qa * g[3] + qb * g[4] + qc * g[5];
+            const float b = qdphi * Kphif + g[6] * st.wide.dtau_k;
+            const float a2 = q02 * Kphif;
+            const float dq[3] = {-g[0] * Kpsif - g[3] * a2 + qa * b, -g[1] * Kpsif - g[4] * a2 + qb * b,
+                                 -g[2] * Kpsif - g[5] * a2 + qc * b};
+            add_small(q, dq);
             kicked = true;
         }
     }
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-        if (!ok[p]) continue;
-        const int64_t i = idx[p];
-        if (moved)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) __stcs(xd + d * n + i, x[p][d]);
-        if (kicked)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) __stcs(qd + d * n + i, q[p][d]);
+    if (moved) {
+        __stcs(xd + i, x[0]);
+        __stcs(xd + n + i, x[1]);
+        __stcs(xd + 2 * n + i, x[2]);
+    }
+    if (kicked) {
+        __stcs(qd + i, q[0]);
+        __stcs(qd + n + i, q[1]);
+        __stcs(qd + 2 * n + i, q[2]);
     }
 }
 
-// The pass kernel: P particles per thread, with three resident blocks per SM for P = 1
-// (80 registers, 24 warps) and two for P = 2 (128 registers, 16 warps carrying 64
-// particles each).  Trilinear reads: 376 ms (P = 2) against 378 (P = 1) on 3 x 256^3
-// particles; order-2 reads, whose 27 cells P = 1's third block hides better: 43.2
-// against 40.5 ms on 2 x 101^3 particles, 250 steps.  Work is handed out at run time, 32 P
-// consecutive particles to a warp at a time (a.ctr[0] counts the chunks taken; each
-// warp claims its next chunk before working on the current one, so that the atomic's
-// round trip overlaps the work): the pass ends together on every SM however its
-// blocks were placed, and the particles in flight stay one stretch of the cell order,
-// whose grid cells the gathers share in L2.  The last warp to finish (a.ctr[1] counts
-// them) sets both counters back to zero for the next pass.
-
-template <typename Gt, bool SERIES, bool UNI, int P>
-__global__ void __launch_bounds__(kThreads, P == 2 ? 2 : 3) k_push_wide(const __grid_constant__ PushArgs a,
-                                                                       double* __restrict__ xd,
-                                                                       double* __restrict__ qd,
-                                                                       const float* __restrict__ q0f)
+// The pass kernel: three resident blocks per SM (80 registers, 24 warps; four of 64
+// registers: 346 ms against 341 on 3 x 256^3 particles, 200 steps; two of 128 with two
+// particles per thread: 441).  Work is handed out at run time, 32 consecutive particles to
+// a warp at a time (a.ctr[0] counts the chunks taken; each warp claims its next chunk
+// before working on the current one, so that the atomic's round trip overlaps the work):
+// the pass ends together on every SM however its blocks were placed, and the particles in
+// flight stay one stretch of the cell order, whose grid cells the gathers share in L2.
+// The last warp to finish (a.ctr[1] counts them) sets both counters back to zero for the
+// next pass.
+template <typename Gt, bool SERIES, bool UNI>
+__global__ void __launch_bounds__(kThreads, 3) k_push_wide(const __grid_constant__ PushArgs a, double* __restrict__ xd,
+                                                           double* __restrict__ qd, const float* __restrict__ q0f)
 {
     const unsigned lane = threadIdx.x & 31u;
-    unsigned next = 0;   // chunk indices (n < 2^38)
+    unsigned next = 0;   // chunk indices (n < 2^37)
     if (lane == 0) next = (unsigned)atomicAdd(a.ctr, 1ull);
     for (;;) {
         const unsigned c = __shfl_sync(0xffffffffu, next, 0);
-        const int64_t i0 = (int64_t)c * (32 * P);
+        const int64_t i0 = (int64_t)c * 32;
         if (i0 >= a.n) break;
         if (lane == 0) next = (unsigned)atomicAdd(a.ctr, 1ull);
         const int64_t i = i0 + lane;
-        if (i < a.n) wide_particles<Gt, SERIES, UNI, P>(a, xd, qd, q0f, i);
+        if (i < a.n) wide_particle<Gt, SERIES, UNI>(a, xd, qd, q0f, i);
     }
     if (lane == 0) {
         const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x / 32);
@@ -1069,26 +1025,21 @@ __global__ void __launch_bounds__(kThreads, 3) k_push_wide_multi(const __grid_co
         while (k + 1 < m.nseg && g >= m.seg[k + 1].begin) ++k;
         const MultiPass::Seg& sg = m.seg[k];
         const PushArgs& a = *sg.args;
-        if (a.wide_series) wide_particles<Gt, true, false, 1>(a, sg.xd, sg.qd, sg.q0f, g - sg.begin);
-        else wide_particles<Gt, false, false, 1>(a, sg.xd, sg.qd, sg.q0f, g - sg.begin);
+        if (a.wide_series) wide_particle<Gt, true, false>(a, sg.xd, sg.qd, sg.q0f, g - sg.begin);
+        else wide_particle<Gt, false, false>(a, sg.xd, sg.qd, sg.q0f, g - sg.begin);
     }
-}
-
-template <typename Gt, bool SERIES, int P>
-void push_wide_p(cudaStream_t s, unsigned b, const PushArgs& a, const ParticleState& st)
-{
-    if (a.uniform_species) launch_pass(k_push_wide<Gt, SERIES, true, P>, b, s, a, st.xd, st.qd, st.q0f);
-    else launch_pass(k_push_wide<Gt, SERIES, false, P>, b, s, a, st.xd, st.qd, st.q0f);
 }
 
 template <typename Gt>
 void push_wide(cudaStream_t s, unsigned b, const PushArgs& a, const ParticleState& st)
 {
-    // two particles per thread with the fitted integrals (the node sums keep one: 22.1 ms
-    // with two, 19.6 ms with one on 160^3 particles, 100 steps)
-    if (!a.wide_series) push_wide_p<Gt, false, 1>(s, b, a, st);
-    else if (a.pair) push_wide_p<Gt, true, 2>(s, b, a, st);
-    else push_wide_p<Gt, true, 1>(s, b, a, st);
+    if (a.wide_series) {
+        if (a.uniform_species) launch_pass(k_push_wide<Gt, true, true>, b, s, a, st.xd, st.qd, st.q0f);
+        else launch_pass(k_push_wide<Gt, true, false>, b, s, a, st.xd, st.qd, st.q0f);
+    } else {
+        if (a.uniform_species) launch_pass(k_push_wide<Gt, false, true>, b, s, a, st.xd, st.qd, st.q0f);
+        else launch_pass(k_push_wide<Gt, false, false>, b, s, a, st.xd, st.qd, st.q0f);
+    }
 }
 
 // ---- the fused leapfrog pass, plain FP64 form --------------------------------
@@ -1116,10 +1067,9 @@ __global__ void __launch_bounds__(kThreads) k_push_f64(const __grid_constant__ P
                                                        double* __restrict__ sd)
 {
     const int64_t n = a.n;
-    const unsigned long long Lbits = (unsigned long long)__double_as_longlong(a.L);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int s = (int)(i >= a.sp_begin[0]) + (int)(i >= a.sp_begin[1]) + (int)(i >= a.sp_begin[2]);
-        double x[1][3] = {{xd[i], xd[n + i], xd[2 * n + i]}};
+        double x[3] = {xd[i], xd[n + i], xd[2 * n + i]};
         double q[3] = {qd[i], qd[n + i], qd[2 * n + i]};
         const double q0[3] = {q0d[i], q0d[n + i], q0d[2 * n + i]};
         double metric = EXACT ? sd[i] : 0.0;      // phi + psi at the next drift's start
@@ -1133,13 +1083,13 @@ __global__ void __launch_bounds__(kThreads) k_push_f64(const __grid_constant__ P
                 for (int j = 0; j < a.n_gl; ++j) D += c.Wd[j] * rsqrt_any(qq + c.mud[j]);
                 if (EXACT) D *= 1.0 + metric;
 #pragma unroll
-                for (int d = 0; d < 3; ++d) x[0][d] += D * q[d];
-                wrap_rare(x, a.L, a.invL, Lbits);
+                for (int d = 0; d < 3; ++d) x[d] += D * q[d];
+                wrap_rare(x, a.L, a.invL);
                 moved = true;
             }
             if (st.do_kick) {
                 double g[8];
-                gather_f64_order<EXACT ? 8 : 7>(a.order, reinterpret_cast<const double*>(a.G[u]), a.N, a.invh, x[0], g);
+                gather_f64_order<EXACT ? 8 : 7>(a.order, reinterpret_cast<const double*>(a.G[u]), a.N, a.invh, x, g);
                 // the kick's momentum: q0 (the separable forms) or q at the kick's start
                 const double qk[3] = {EXACT ? q[0] : q0[0], EXACT ? q[1] : q0[1], EXACT ? q[2] : q0[2]};
                 const double q02 = qk[0] * qk[0] + qk[1] * qk[1] + qk[2] * qk[2];
@@ -1168,9 +1118,9 @@ __global__ void __launch_bounds__(kThreads) k_push_f64(const __grid_constant__ P
         }
         if (EXACT && kicked) sd[i] = metric;
         if (moved) {
-            xd[i] = x[0][0];
-            xd[n + i] = x[0][1];
-            xd[2 * n + i] = x[0][2];
+            xd[i] = x[0];
+            xd[n + i] = x[1];
+            xd[2 * n + i] = x[2];
         }
         if (kicked) {
             qd[i] = q[0];

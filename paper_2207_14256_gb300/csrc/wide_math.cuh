@@ -7,7 +7,8 @@
 // value with some bits to spare and a bound on its distance from what FP64 arithmetic
 // gets; where that value lies so near a rounding boundary that the bound could cross it
 // (one evaluation in 2^11 or rarer), it says so and the caller runs the FP64 formula.
-//   w_rsqrt53: rsqrt_fp64's four FP64 instructions (~50 others);
+//   w_rsqrt53: rsqrt_fp64's four FP64 instructions (~50 others), w_square53 its square (~20);
+//   w_add:     the sum of a double and a much smaller float (~25, and no conversion);
 //   w_kick:    the kick's integrals as the FP32 values their user reads (9 FP64
 //              instructions as polynomials, 8 per node as sums).
 // tests/test_wide_math.py compares both with the FP64 formulas, bit for bit.
@@ -32,10 +33,12 @@ namespace fdf {
 // 2^-66) amounts to less than 12 of these units; the final rounding is at 2^-53, so a
 // value within 16 units of a tie (33 of 65536) is left to FP64, as is one whose
 // intermediate values leave the binades assumed (m within 2^-20 of 1 or 4).
-FDF_DEV bool w_rsqrt53(double v, float yf, double& r)
+// R and k: r = R 2^(-53 - k).
+FDF_DEV bool w_rsqrt53(double v, float yf, double& r, int64_t& R, int& k)
 {
     const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-    const int ex = (int)(hi >> 20) - 1023, k = ex >> 1, odd = ex & 1;
+    const int ex = (int)(hi >> 20) - 1023, odd = ex & 1;
+    k = ex >> 1;
     const uint32_t m1 = (hi & 0xFFFFFu) | 0x100000u;
     const uint32_t Mh = odd ? (m1 << 1) | (lo >> 31) : m1, Ml = lo << odd;
     const uint32_t yb = __float_as_uint(yf);
@@ -59,11 +62,59 @@ FDF_DEV bool w_rsqrt53(double v, float yf, double& r)
     const int64_t W = (int64_t)(int)Y * (int)(E >> 32) + (int64_t)(((uint64_t)(uint32_t)E * Y) >> 32) +
                       __float2int_rn(__fmul_rn(kap, h69));
     ok = ok && ((uint32_t)W & 0xFFFFu) - (0x8000u - 16u) > 32u;
-    const int64_t R = ((int64_t)Y << 29) + ((W + 0x8000) >> 16); // r 2^k in units of 2^-53
+    R = ((int64_t)Y << 29) + ((W + 0x8000) >> 16); // r 2^k in units of 2^-53
     const uint32_t Rh = (uint32_t)(R >> 32);
     ok = ok && (Rh >> 20) == 1u;
     r = __hiloint2double((int)(Rh + ((uint32_t)(1021 - k) << 20)), (int)(uint32_t)R);
     return ok;
+}
+
+FDF_DEV bool w_rsqrt53(double v, float yf, double& r)
+{
+    int64_t R;
+    int k;
+    return w_rsqrt53(v, yf, r, R, k);
+}
+
+// The bits of r * r for r = R 2^(-53 - k), 2^52 <= R < 2^53 (w_rsqrt53's), rounded to nearest,
+// ties to even: the 106-bit square in three 32-bit products.
+FDF_DEV double w_square53(int64_t R, int k)
+{
+    const uint32_t Rh = (uint32_t)((uint64_t)R >> 32), Rl = (uint32_t)R;
+    const uint64_t ll = (uint64_t)Rl * Rl;
+    const uint64_t mid = (((uint64_t)Rh * Rl) << 1) + (ll >> 32);
+    const uint64_t top = (uint64_t)Rh * Rh + (mid >> 32);       // the square's bits 64 ..
+    const uint32_t m = (uint32_t)mid, th = (uint32_t)(top >> 32), tl = (uint32_t)top;
+    const uint32_t big = th >> 9;                               // the square >= 2^105
+    const uint32_t sh = 12u - big;
+    const uint32_t ql = __funnelshift_l(m, tl, sh), rem = m << sh;
+    const uint32_t sticky = ((uint32_t)ll != 0u) | (ql & 1u);
+    const uint64_t q = (((uint64_t)__funnelshift_l(tl, th, sh) << 32) | ql) + (rem > 0x80000000u - sticky);
+    return __hiloint2double((int)((uint32_t)(q >> 32) + ((1020u + big - 2u * (uint32_t)k) << 20)), (int)(uint32_t)q);
+}
+
+// The bits of q + (double)d in integers (a subnormal d counts as zero, as f2d_bits takes it):
+// d's 24-bit significand in units of q's last place, rounded to nearest, ties to even, is
+// added to q's bit pattern.  False where that may not be the sum's pattern: the sum leaves q's
+// binade or comes to its lower end (below which last places are finer), |d| is above 2^-1 |q| or so, or one of them is no finite normal number.
+FDF_DEV bool w_add(double q, float d, double& r)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(q), lo = (uint32_t)__double2loint(q), db = __float_as_uint(d);
+    const int eq = (int)((hi >> 20) & 0x7FFu), ed = (int)((db >> 23) & 0xFFu);
+    const int F = ed ? (int)((db & 0x7FFFFFu) | 0x800000u) : 0;
+    const int Z = (int)(db ^ hi) < 0 ? -F : F;
+    const int s = eq - ed - 925;                                // d = Z 2^-s in units of q's last place
+    const int S = s > 31 ? 31 : (s > 0 ? s : 0), L = s < 0 ? -s : 0;
+    const uint32_t below = __funnelshift_r(0u, (uint32_t)Z, (uint32_t)S);    // the bits that go, at the top of a word
+    int X = Z >> S;
+    X += below > 0x80000000u - ((lo + (uint32_t)X) & 1u);
+    const uint64_t delta = ((uint64_t)(uint32_t)(int)__funnelshift_l((uint32_t)X, (uint32_t)(X >> 31), (uint32_t)L) << 32) |
+                           ((uint32_t)X << (L & 31));
+    const uint64_t b = (((uint64_t)hi << 32) | lo) + delta;
+    const uint32_t bh = (uint32_t)(b >> 32);
+    r = __hiloint2double((int)bh, (int)(uint32_t)b);
+    return L <= 27 && ed != 255 && (uint32_t)(eq - 1) < 0x7FEu && ((bh ^ hi) >> 20) == 0u &&
+           ((bh & 0xFFFFFu) | (uint32_t)b) != 0u;
 }
 
 // ---- pairs of floats (value = hi + lo, 48 bits) -----------------------------------------

@@ -33,6 +33,7 @@ static inline int __double2hiint(double d) { return (int)(bits<uint64_t>(d) >> 3
 static inline int __double2loint(double d) { return (int)bits<uint64_t>(d); }
 static inline double __hiloint2double(int h, int l) { return bits<double>(((uint64_t)(uint32_t)h << 32) | (uint32_t)l); }
 static inline uint32_t __funnelshift_l(uint32_t lo, uint32_t hi, uint32_t s) { return s ? (hi << s) | (lo >> (32 - s)) : hi; }
+static inline uint32_t __funnelshift_r(uint32_t lo, uint32_t hi, uint32_t s) { return s ? (lo >> s) | (hi << (32 - s)) : lo; }
 static inline float __int2float_rn(int i) { return (float)i; }
 static inline float __uint2float_rn(uint32_t i) { return (float)i; }
 static inline int __float2int_rn(float f) { return (int)std::nearbyint(f); }
@@ -62,9 +63,25 @@ extern "C" void check_rsqrt(int n, const double* v, long* counts)
         skew(i);
         const float y = w_rsqrt(d2f(v[i]));
         double r;
-        if (!w_rsqrt53(v[i], y, r)) ++counts[0];
-        else if (r != rsqrt64(v[i], y)) ++counts[1];
+        int64_t R;
+        int k;
+        if (!w_rsqrt53(v[i], y, r, R, k)) ++counts[0];
+        else if (r != rsqrt64(v[i], y) || w_square53(R, k) != r * r) ++counts[1];
     }
+}
+extern "C" void check_add(int n, const double* q, const float* d, long* counts)
+{
+    for (int i = 0; i < n; ++i) {
+        double r;
+        const double x = std::fabs(d[i]) < 1.1754943508222875e-38f ? 0.0 : (double)d[i];
+        if (!w_add(q[i], d[i], r)) ++counts[0];
+        else if (bits<uint64_t>(r) != bits<uint64_t>(q[i] + x)) ++counts[1];
+    }
+}
+extern "C" void check_square(int n, const long* R, long* counts)
+{
+    for (int i = 0; i < n; ++i)
+        if (w_square53(R[i], 0) != ((double)R[i] * 0x1p-53) * ((double)R[i] * 0x1p-53)) ++counts[1];
 }
 // a kick over nodes W, e (mu = m^2 a_c^2) at momenta q[n][3]; series: c_0 (FP64) and c_1.. (FP32)
 extern "C" int check_kick(int series, int m, const double* W, const double* e, double mu, double unit, const double* cpsi,
@@ -141,6 +158,47 @@ def test_rsqrt_bits(lib, lo, hi):
     assert counts[1] == 0
     if hi - lo > 1e-3:
         assert counts[0] <= 4 * 33 / 65536 * n
+
+
+def test_square_bits(lib):
+    rng = np.random.default_rng(7)
+    R = rng.integers(2 ** 52, 2 ** 53, 1000000)
+    root2 = int(2 ** 52 * math.sqrt(2.0))
+    # short significands, whose squares round at ties or not at all, and both ends of each binade
+    R = np.concatenate([R, (R >> 27) << 27, (R >> 26) << 26, (R >> 25) << 25, 2 ** 52 + np.arange(999),
+                        2 ** 53 - 1 - np.arange(999), root2 + np.arange(-999, 999)])
+    counts = np.zeros(2, np.int64)
+    lib.check_square(len(R), _ptr(R), _ptr(counts))
+    assert counts[1] == 0
+
+
+@pytest.mark.parametrize("scale", [1e-4, 1.0, 1e25])
+def test_add_bits(lib, scale):
+    rng = np.random.default_rng(11)
+    n = 1000000
+    q = scale * rng.normal(size=n)
+    # from |d| = 2|q| down past q's last place; zeros, and ties (odd multiples of half a last place)
+    d = (q * rng.choice([-1.0, 1.0], n) * np.exp2(-rng.uniform(-1.0, 60.0, n))).astype(np.float32)
+    d[::97] = 0.0
+    tie = np.arange(0, n, 13)
+    d[tie] = (np.spacing(np.abs(q[tie])) * (rng.integers(0, 1 << 20, len(tie)) + 0.5)).astype(np.float32)
+    q[1::101] = scale * np.exp2(rng.integers(-3, 3, len(q[1::101])))          # powers of two: the binade's edge
+    counts = np.zeros(2, np.int64)
+    lib.check_add(n, _ptr(q), _ptr(d), _ptr(counts))
+    assert counts[1] == 0
+    # refused: sums that leave the binade, likely only where |d| > 2^-7 |q|
+    small = np.abs(d) < np.exp2(-7.0) * np.abs(q)
+    small[1::101] = False
+    qs, ds = np.ascontiguousarray(q[small]), np.ascontiguousarray(d[small])
+    counts[:] = 0
+    lib.check_add(len(qs), _ptr(qs), _ptr(ds), _ptr(counts))
+    assert counts[0] <= 2.0 ** -7 * len(qs)
+    special = np.array([0.0, -0.0, 5e-324, 1e-310, np.inf, -np.inf, np.nan, 1.0, -1.0])
+    q = np.repeat(special, 6)
+    d = np.tile(np.array([0.0, -0.0, 1e-39, np.inf, -np.inf, 1e-30], np.float32), len(special))
+    counts[:] = 0
+    lib.check_add(len(q), _ptr(q), _ptr(d), _ptr(counts))
+    assert counts[1] == 0
 
 
 @pytest.mark.parametrize("T", [1.7e-4, 1e-12])
