@@ -286,7 +286,7 @@ Layout make_layout(const fdf_params& p, int nk, int na, int ncdf)
     L.cdf_t = take((size_t)ncdf * 8);
     L.cdf_F = take((size_t)ncdf * 8);
     L.tw = take(N * complex_bytes(prec));
-    L.W = take(4 * N3 * complex_bytes(prec));
+    L.W = take(5 * N3 * complex_bytes(prec));     // four packed grids; five in fdf_build_fields
     L.nbuf = grid_buffers(p);
     for (int b = 0; b < L.nbuf; ++b) L.G[b] = take(N3 * grid_bytes_per_cell(prec));
     // the two super-step grids an interpolated step reads (super-steps only)
@@ -793,8 +793,9 @@ int mode_tables(fdf_ctx* c, const double* lna, int count, cudaStream_t s)
     return FDF_OK;
 }
 
-// The eight fields at ln a into G, on stream s; slot 7 as `slot7` says (kSlot7*).
-int build_fields(fdf_ctx* c, double lna, void* G, cudaStream_t s, int slot7)
+// The transforms of the eight fields at ln a up to their y pass, into c->W on stream s;
+// slot 7 as `slot7` says (kSlot7*), `grids` packed grids.
+int build_lines(fdf_ctx* c, double lna, cudaStream_t s, int slot7, int grids)
 {
     if (!c->noise_ready) {
         if (s != c->sf) FDF_CUDA(cudaStreamSynchronize(c->stream), "sync");
@@ -811,15 +812,24 @@ int build_fields(fdf_ctx* c, double lna, void* G, cudaStream_t s, int slot7)
     }
     FieldArgs a = field_args(c, lna);
     a.slot7 = slot7;
+    a.grids = grids;
     const int prec = grid_prec(c->p.precision), N = c->p.n_grid;
     const void* A = c->modeA + (size_t)slot * 4 * mode_table_size(N) * real_bytes(c->p.precision);
     int rc = timed_on(c, s, FDF_K_FIELDS_Z, "fields z pass",
                       [&] { return launch_fields_z(s, prec, a, A, c->noise, c->tw, c->W); });
     if (rc) return rc;
-    rc = timed_on(c, s, FDF_K_FIELDS_Y, "fields y pass", [&] { return launch_fields_y(s, prec, N, c->tw, c->W); });
+    return timed_on(c, s, FDF_K_FIELDS_Y, "fields y pass",
+                    [&] { return launch_fields_y(s, prec, N, grids, c->tw, c->W); });
+}
+
+// The eight fields at ln a into G, on stream s.
+int build_fields(fdf_ctx* c, double lna, void* G, cudaStream_t s, int slot7)
+{
+    int rc = build_lines(c, lna, s, slot7, 4);
     if (rc) return rc;
-    return timed_on(c, s, FDF_K_FIELDS_X, "fields x pass",
-                    [&] { return launch_fields_x(s, prec, N, c->tw, c->W, G); });
+    return timed_on(c, s, FDF_K_FIELDS_X, "fields x pass", [&] {
+        return launch_fields_x(s, grid_prec(c->p.precision), c->p.n_grid, c->tw, c->W, G);
+    });
 }
 
 int push(fdf_ctx* c, const PushArgs& a)
@@ -1093,6 +1103,7 @@ FieldArgs fdf::make_field_args(const fdf_params& p, int nk, int na, double lnk0,
     const double H = H0 * std::sqrt(p.omega_r / (aa * aa * aa * aa) + p.omega_m / (aa * aa * aa) +
                                     (1.0 - p.omega_m - p.omega_r));
     a.aH = aa * H;
+    a.grids = 4;
     const double V = p.box_mpc * p.box_mpc * p.box_mpc;
     a.amp0 = std::sqrt(2.0 * kPi * kPi * p.A_s / V);
     a.half_nsm1 = 0.5 * (p.n_s - 1.0);
@@ -1827,23 +1838,15 @@ int fdf_build_fields(fdf_ctx* c, double lna, double* out, int32_t out_on_device)
     const size_t N3 = (size_t)N * N * N;
     FDF_CUDA(cudaStreamSynchronize(c->sf), "fdf_build_fields");
     FDF_CUDA(cudaStreamSynchronize(c->stream), "fdf_build_fields");
-    int buf = 0;
-    for (int i = 0; i < c->nbuf; ++i)
-        if (c->gk[i] != c->k) buf = i;
-    c->gk[buf] = -1;
-    // slots 0-6 as the steps' passes read them (phi_dot transformed alone), then slot 7 (psi)
-    // from a second build, as the initial transform reads it
+    // slots 0-6 as the steps' passes read them (phi_dot transformed alone) and slot 7 (psi)
+    // as the initial transform reads it, the fifth packed grid
     double* dst = out;
     if (!out_on_device) FDF_CUDA(cudaMalloc(&dst, 8 * N3 * 8), "allocating the field copy");
-    int rc = FDF_OK;
-    for (int pass = 0; pass < 2 && rc == FDF_OK; ++pass) {
-        rc = build_fields(c, lna, c->G[buf], c->stream, pass == 0 ? kSlot7Zero : kSlot7Psi);
-        if (rc) break;
-        rc = timed(c, FDF_K_OTHER, "field export", [&] {
-            return launch_fields_to_f64(c->stream, grid_prec(c->p.precision), N, c->G[buf], dst,
-                                        pass == 0 ? 0x7Fu : 0x80u);
+    int rc = build_lines(c, lna, c->stream, kSlot7Zero, 5);
+    if (!rc)
+        rc = timed(c, FDF_K_FIELDS_X, "fields x pass", [&] {
+            return launch_fields_x_planar(c->stream, grid_prec(c->p.precision), N, c->tw, c->W, dst);
         });
-    }
     if (!rc && !out_on_device) {
         cudaError_t e = cudaMemcpyAsync(out, dst, 8 * N3 * 8, cudaMemcpyDeviceToHost, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

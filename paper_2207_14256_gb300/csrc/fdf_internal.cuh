@@ -181,6 +181,7 @@ struct FieldArgs {
     uint32_t key0, key1;        // Philox key (seed)
     int fixed_amp;
     int slot7;                  // slot 7: kSlot7Psi, kSlot7Sum (phi + psi) or kSlot7Zero
+    int grids;                  // packed grids to build: 4, or 5 with phi_dot + i psi as the fifth
 };
 
 inline int ilog2_host(int v)
@@ -208,7 +209,7 @@ cudaError_t launch_sample(cudaStream_t s, int64_t n, uint32_t key0, uint32_t key
                           int* flag);
 
 // Field build: three passes.  precision: FDF_PREC_*.  W is a complex work array of
-// 4 N^3 elements (float2 or double2), G the gather grid.
+// 4 N^3 (5 N^3 with FieldArgs::grids = 5) elements (float2 or double2), G the gather grid.
 // Amplitude tables A[count][4 M] (M = mode_table_size(N)) of count scale factors from the
 // FP64 tables [3][na][nk] and the keys of the run's modes; read by the z pass.
 struct ModeKey {
@@ -234,11 +235,13 @@ cudaError_t launch_mode_tables(cudaStream_t s, int precision, const FieldArgs& a
 cudaError_t launch_noise(cudaStream_t s, int precision, const FieldArgs& a, void* R);
 cudaError_t launch_fields_z(cudaStream_t s, int precision, const FieldArgs& a, const void* A, const void* R,
                             const void* tw, void* W0);
-cudaError_t launch_fields_y(cudaStream_t s, int precision, int N, const void* tw, void* W);
+cudaError_t launch_fields_y(cudaStream_t s, int precision, int N, int grids, const void* tw, void* W);
 cudaError_t launch_fields_x(cudaStream_t s, int precision, int N, const void* tw, const void* W, void* G);
-// G (any precision) <-> [8][N^3] FP64; to_f64 writes the slots whose bit is set in mask.
-cudaError_t launch_fields_to_f64(cudaStream_t s, int precision, int N, const void* G, double* out,
-                                 unsigned mask = 0xFFu);
+// The x pass of five packed grids into out[8][N^3], each value as a gather grid holds it.
+cudaError_t launch_fields_x_planar(cudaStream_t s, int precision, int N, const void* tw, const void* W, double* out);
+// The amplitude table at one scale factor (from two-row tables or more) and the unit
+// Gaussian field, in one launch.
+cudaError_t launch_modes_once(cudaStream_t s, int precision, const FieldArgs& a, const double* tabs64, void* A, void* R);
 // G = (1 - w) A + w B over whole gather grids (super-steps, Sec. 2.1)
 cudaError_t launch_interp_grid(cudaStream_t s, int precision, int N, const void* A, const void* B, double w,
                                void* G);

@@ -9,7 +9,9 @@
 // FDF_NOALLOC_SCRATCH_BYTES that every GPU loading the library holds until the
 // process exits; the caller passes the inputs (host tables) and the output
 // (device memory).
+#include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -71,12 +73,13 @@ extern "C" int fdf_build_fields_noalloc(const fdf_params* p, const fdf_tables* t
     const bool f64 = gp == FDF_PREC_F64;
     const size_t N = (size_t)p->n_grid, N3 = N * N * N;
     const size_t csz = f64 ? 16 : 8, rsz = f64 ? 8 : 4;
-    const size_t ntab = 3 * (size_t)t->na * t->nk;
-    // scratch layout: W | G | FP64 tables | amplitude table | twiddles | noise | mode keys
-    const size_t M = (size_t)mode_table_size(p->n_grid);
-    const size_t oW0 = 0, oW1 = oW0 + align256(4 * N3 * csz), oT64 = oW1 + align256(4 * N3 * csz);
-    const size_t oA = oT64 + align256(ntab * 8), oTw = oA + align256(4 * M * rsz), oR = oTw + align256(N * csz);
-    const size_t oK = oR + align256(N3 * csz), need = oK + align256(M * sizeof(ModeKey));
+    // scratch layout: W (five packed grids) | FP64 table rows and twiddles | amplitude table | noise
+    const size_t M = (size_t)mode_table_size(p->n_grid), nk = (size_t)t->nk;
+    const size_t oT64 = align256(5 * N3 * csz), oTw = oT64 + 6 * nk * 8;
+    const size_t oA = align256(oTw + N * csz), oR = oA + align256(4 * M * rsz);
+    // the limit counts two work arrays of four grids and the tables in full
+    const size_t need = 2 * align256(4 * N3 * csz) + align256(3 * (size_t)t->na * nk * 8) + align256(4 * M * rsz) +
+                        align256(N * csz) + align256(N3 * csz);
     if (need > FDF_NOALLOC_SCRATCH_BYTES) {
         char msg[200];
         snprintf(msg, sizeof msg,
@@ -89,37 +92,31 @@ extern "C" int fdf_build_fields_noalloc(const fdf_params* p, const fdf_tables* t
     rc = scratch_address(&s);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t nt = (size_t)t->na * t->nk;
-    double* T64 = (double*)(s + oT64);
-    cudaError_t e = cudaMemcpyAsync(T64, t->T_psi, nt * 8, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(T64 + nt, t->T_phi, nt * 8, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(T64 + 2 * nt, t->dTphi_dlna, nt * 8, cudaMemcpyHostToDevice, st);
-    // the twiddles fdf_create uploads, from the same host table; the copies are from
-    // pageable host memory, so the stream is synchronised before the vectors go
-    std::vector<double> twd(2 * N);
-    twiddle_table((int)N, twd.data());
-    const std::vector<float> twf(twd.begin(), twd.end());
-    if (e == cudaSuccess)
-        e = f64 ? cudaMemcpyAsync(s + oTw, twd.data(), twd.size() * 8, cudaMemcpyHostToDevice, st)
-                : cudaMemcpyAsync(s + oTw, twf.data(), twf.size() * 4, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return set_error(FDF_ECUDA, (std::string("table upload: ") + cudaGetErrorString(e)).c_str());
+    // what the build reads of the host's tables, in one copy: the two rows around ln a of each
+    // of the three tables, and the twiddles fdf_create uploads.  The copy is from pageable
+    // host memory, so the stream is synchronised before the vector goes.
     FieldArgs a = make_field_args(*p, t->nk, t->na, lnk0, dlnk, lnat0, dlnat, lna);
-    void* W0 = s + oW0;
-    void* W1 = s + oW1;
-    if (e == cudaSuccess) e = launch_noise(st, gp, a, s + oR);
-    ModeSteps step{};
-    step.add(a);
-    if (e == cudaSuccess) e = launch_mode_keys(st, a, (ModeKey*)(s + oK));
-    if (e == cudaSuccess) e = launch_mode_tables(st, gp, a, step, (const ModeKey*)(s + oK), T64, s + oA);
-    // as fdf_build_fields: slots 0-6 from a build with phi_dot transformed alone, slot 7
-    // (psi) from a second build
-    for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
-        a.slot7 = pass == 0 ? kSlot7Zero : kSlot7Psi;
-        e = launch_fields_z(st, gp, a, s + oA, s + oR, s + oTw, W0);
-        if (e == cudaSuccess) e = launch_fields_y(st, gp, p->n_grid, s + oTw, W0);
-        if (e == cudaSuccess) e = launch_fields_x(st, gp, p->n_grid, s + oTw, W0, W1);
-        if (e == cudaSuccess) e = launch_fields_to_f64(st, gp, p->n_grid, W1, out, pass == 0 ? 0x7Fu : 0x80u);
+    std::vector<double> up(6 * nk + 2 * N), twd(2 * N);
+    const double* tables[3] = {t->T_psi, t->T_phi, t->dTphi_dlna};
+    for (int k = 0; k < 3; ++k) std::memcpy(up.data() + 2 * k * nk, tables[k] + (size_t)a.ia * nk, 2 * nk * 8);
+    twiddle_table((int)N, twd.data());
+    if (f64) std::copy(twd.begin(), twd.end(), up.begin() + 6 * nk);
+    else {
+        const std::vector<float> twf(twd.begin(), twd.end());
+        std::memcpy(up.data() + 6 * nk, twf.data(), twf.size() * 4);
     }
+    cudaError_t e = cudaMemcpyAsync(s + oT64, up.data(), 6 * nk * 8 + N * csz, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return set_error(FDF_ECUDA, (std::string("table upload: ") + cudaGetErrorString(e)).c_str());
+    a.ia = 0;
+    a.na = 2;
+    a.slot7 = kSlot7Zero;
+    a.grids = 5;
+    // as fdf_build_fields: slots 0-6 with phi_dot transformed alone, slot 7 (psi) from the
+    // fifth packed grid
+    e = launch_modes_once(st, gp, a, (const double*)(s + oT64), s + oA, s + oR);
+    if (e == cudaSuccess) e = launch_fields_z(st, gp, a, s + oA, s + oR, s + oTw, s);
+    if (e == cudaSuccess) e = launch_fields_y(st, gp, p->n_grid, 5, s + oTw, s);
+    if (e == cudaSuccess) e = launch_fields_x_planar(st, gp, p->n_grid, s + oTw, s, out);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess)
         return set_error(FDF_ECUDA, (std::string("fdf_build_fields_noalloc: ") + cudaGetErrorString(e)).c_str());

@@ -258,15 +258,22 @@ __device__ __forceinline__ V mode_unit(const FieldArgs& a, int jx, int jy, int j
     return mk<V>(re, im);
 }
 
+// The N^3 mode array, drawn by `blocks` blocks of which this is number `block`.
 template <typename V>
-__global__ void __launch_bounds__(256) k_noise(FieldArgs a, V* __restrict__ R)
+__device__ __forceinline__ void noise_part(const FieldArgs& a, V* __restrict__ R, unsigned block, unsigned blocks)
 {
     const int N = a.N;
     const size_t N3 = (size_t)N * N * N;
-    for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < N3; c += (size_t)gridDim.x * blockDim.x) {
+    for (size_t c = block * (size_t)blockDim.x + threadIdx.x; c < N3; c += (size_t)blocks * blockDim.x) {
         const int jx = (int)(c % N), jy = (int)((c / N) % N), jz = (int)(c / ((size_t)N * N));
         R[c] = mode_unit<V>(a, jx, jy, jz);
     }
+}
+
+template <typename V>
+__global__ void __launch_bounds__(256) k_noise(FieldArgs a, V* __restrict__ R)
+{
+    noise_part<V>(a, R, blockIdx.x, gridDim.x);
 }
 
 // Packed spectrum p of a mode with unit Gaussian R and amplitudes (Apsi, Aphi, Adot):
@@ -292,28 +299,52 @@ __device__ __forceinline__ V packed(int p, V R, typename Real<V>::T Apsi, typena
 // sqrt(2 pi^2 A_s / V) k^-3/2 (k/k_pivot)^((n_s-1)/2) and k's place in the transfer tables'
 // uniform ln k grid (clamped): what no step changes.  Once per run: its chain of a root, a
 // logarithm, an exponential and a division takes 10 us however small the grid is.
+__device__ __forceinline__ ModeKey mode_key(const FieldArgs& a, int m)
+{
+    ModeKey key{0.0, 0.0, 0, 0};
+    if (m > 0) {
+        const double k = a.kf * sqrt((double)m);
+        const double lnk = log(k);
+        key.amp = a.amp0 / (k * sqrt(k)) * exp(a.half_nsm1 * (lnk - a.lnkp));
+        const double pos = (lnk - a.lnk0) * a.inv_dlnk;
+        if (pos <= 0.0) {
+            key.ik = 0;
+            key.fk = 0.0;
+        } else if (pos >= a.nk - 1) {
+            key.ik = a.nk - 2;
+            key.fk = 1.0;
+        } else {
+            key.ik = (int)pos;
+            key.fk = pos - key.ik;
+        }
+    }
+    return key;
+}
+
 __global__ void __launch_bounds__(256) k_mode_keys(FieldArgs a, int M, ModeKey* __restrict__ keys)
 {
-    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
-        ModeKey key{0.0, 0.0, 0, 0};
-        if (m > 0) {
-            const double k = a.kf * sqrt((double)m);
-            const double lnk = log(k);
-            key.amp = a.amp0 / (k * sqrt(k)) * exp(a.half_nsm1 * (lnk - a.lnkp));
-            const double pos = (lnk - a.lnk0) * a.inv_dlnk;
-            if (pos <= 0.0) {
-                key.ik = 0;
-                key.fk = 0.0;
-            } else if (pos >= a.nk - 1) {
-                key.ik = a.nk - 2;
-                key.fk = 1.0;
-            } else {
-                key.ik = (int)pos;
-                key.fk = pos - key.ik;
-            }
-        }
-        keys[m] = key;
+    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) keys[m] = mode_key(a, m);
+}
+
+// A mode's four table values from rows ia and ia + 1 of the FP64 tables [3][na][nk].
+template <typename T>
+__device__ __forceinline__ void mode_values(const ModeKey& key, int ia, double fa, double aH, int na, int nk,
+                                            const double* __restrict__ tabs, T* __restrict__ out)
+{
+    double v[3];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        const double* r0 = tabs + ((size_t)t * na + ia) * nk;
+        const double* r1 = r0 + nk;
+        const double v0 = (1.0 - key.fk) * r0[key.ik] + key.fk * r0[key.ik + 1];
+        const double v1 = (1.0 - key.fk) * r1[key.ik] + key.fk * r1[key.ik + 1];
+        v[t] = key.amp * ((1.0 - fa) * v0 + fa * v1);
     }
+    v[2] *= aH;
+    out[0] = (T)v[0];
+    out[1] = (T)v[1];
+    out[2] = (T)v[2];
+    out[3] = T(0);
 }
 
 // Per scale factor and m: the amplitude times T_psi, T_phi and a H dT_phi/dln a, read
@@ -325,25 +356,24 @@ __global__ void __launch_bounds__(256) k_mode_tables(const __grid_constant__ Mod
                                                      T* __restrict__ A)
 {
     const int b = blockIdx.y;
-    const double fa = st.fa[b], aH = st.aH[b];
     T* out = A + (size_t)b * 4 * M;
-    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
-        const ModeKey key = keys[m];
-        double v[3];
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-            const double* r0 = tabs + ((size_t)t * na + st.ia[b]) * nk;
-            const double* r1 = r0 + nk;
-            const double v0 = (1.0 - key.fk) * r0[key.ik] + key.fk * r0[key.ik + 1];
-            const double v1 = (1.0 - key.fk) * r1[key.ik] + key.fk * r1[key.ik + 1];
-            v[t] = key.amp * ((1.0 - fa) * v0 + fa * v1);
-        }
-        v[2] *= aH;
-        out[4 * m] = (T)v[0];
-        out[4 * m + 1] = (T)v[1];
-        out[4 * m + 2] = (T)v[2];
-        out[4 * m + 3] = T(0);
+    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x)
+        mode_values<T>(keys[m], st.ia[b], st.fa[b], st.aH[b], na, nk, tabs, out + 4 * (size_t)m);
+}
+
+// Both parts of a build that keeps nothing, in one launch: the first blocks make the
+// amplitude table of one scale factor, the others draw the mode array.
+template <typename V>
+__global__ void __launch_bounds__(256) k_modes_once(FieldArgs a, int M, const double* __restrict__ tabs,
+                                                    typename Real<V>::T* __restrict__ A, V* __restrict__ R)
+{
+    const unsigned nm = (unsigned)((M + 255) / 256);
+    if (blockIdx.x >= nm) {
+        noise_part<V>(a, R, blockIdx.x - nm, gridDim.x - nm);
+        return;
     }
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m < M) mode_values(mode_key(a, m), a.ia, a.fa, a.aH, a.na, a.nk, tabs, A + 4 * (size_t)m);
 }
 
 // One entry of the amplitude table (4 values per |n|^2, 16- or 32-byte aligned) in
@@ -416,8 +446,8 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, sizeof(V) == 8 ? 4 : 2) k
     }
     __syncthreads();
     const size_t N3 = NN * N;
-    // this block's packed grids: all four, or one of gridDim.z
-    const int p0 = gridDim.z == 1 ? 0 : blockIdx.z, p1 = gridDim.z == 1 ? 4 : p0 + 1;
+    // this block's packed grids: all of them, or one of gridDim.z
+    const int p0 = gridDim.z == 1 ? 0 : blockIdx.z, p1 = gridDim.z == 1 ? a.grids : p0 + 1;
 #pragma unroll 1
     for (int p = p0; p < p1; ++p) {
         // one branch per packed grid, so that each reads only the amplitudes it uses
@@ -440,6 +470,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, sizeof(V) == 8 ? 4 : 2) k
             case 0: form(Idx<0>{}); break;
             case 1: form(Idx<1>{}); break;
             case 2: form(Idx<2>{}); break;
+            case 4: form(Idx<3>{}); break;
             default:
                 if (a.slot7 == kSlot7Sum) form(Idx<4>{});
                 else if (a.slot7 == kSlot7Zero) form(Idx<5>{});
@@ -562,22 +593,40 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_X) k_fields_x(const V* __res
     }
 }
 
-// ---- conversions between G and [8][N^3] FP64 (test hooks) -------------------
-template <typename Gt>
-__device__ __forceinline__ double gval(const Gt* G, size_t cell, int s)
+// The x pass of a build for inspection: five packed grids (the fifth is phi_dot + i psi), the
+// values as a gather grid of type Gt would hold them, straight into out[8][N^3] (slots 0-5
+// from grids 0-2, phi_dot from grid 3, psi from grid 4).
+template <typename V, typename Gt, int N>
+__global__ void __launch_bounds__(Shape<N>::THREADS) k_fields_x_planar(const V* __restrict__ tw, const V* __restrict__ W,
+                                                                       double* __restrict__ out)
 {
-    if constexpr (sizeof(Gt) == 2) return (double)__bfloat162float(G[cell * 8 + s]);
-    else return (double)G[cell * 8 + s];
+    using S = Shape<N>;
+    constexpr int N1 = S::N1, N2 = S::N2, T = S::T, LPB = S::THREADS / T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    V* s_tw = reinterpret_cast<V*>(smem_raw);
+    V* tr = s_tw + S::TWS;
+    const int t = threadIdx.x % T, lo = threadIdx.x / T, p = blockIdx.y;
+    const size_t N3 = (size_t)N * N * N;
+    const size_t line = (size_t)blockIdx.x * LPB + lo;
+    V v[N1];
+    const V* src = W + p * N3 + line * N;
+    sfor<N1>([&](auto N1i) { v[N1i] = src[N2 * N1i + t]; });
+    load_line_twiddles<V, N>(s_tw, tw);
+    __syncthreads();
+    line_first<V, N>(v, t, s_tw, tr + lo * S::TSX);
+    __syncthreads();
+    line_second<V, N>(t, tr + lo * S::TSX, [&](int x, V val) {
+        double re = val.x, im = val.y;
+        if constexpr (sizeof(Gt) == 2) {
+            re = (double)__bfloat162float(__float2bfloat16_rn(val.x));
+            im = (double)__bfloat162float(__float2bfloat16_rn(val.y));
+        }
+        if (p < 4) out[(size_t)(2 * p) * N3 + line * N + x] = re;
+        if (p != 3) out[(size_t)(p == 4 ? 7 : 2 * p + 1) * N3 + line * N + x] = im;
+    });
 }
 
-template <typename Gt>
-__global__ void k_fields_to_f64(size_t N3, const Gt* __restrict__ G, double* __restrict__ out, unsigned mask)
-{
-    for (size_t c = blockIdx.x * (size_t)blockDim.x + threadIdx.x; c < N3; c += (size_t)gridDim.x * blockDim.x)
-        for (int s = 0; s < 8; ++s)
-            if (mask & (1u << s)) out[s * N3 + c] = gval(G, c, s);
-}
-
+// ---- [8][N^3] FP64 into a gather grid (test hook) ---------------------------
 template <typename Gt>
 __global__ void k_fields_from_f64(size_t N3, const double* __restrict__ in, Gt* __restrict__ G)
 {
@@ -603,19 +652,19 @@ cudaError_t run_z(cudaStream_t s, const FieldArgs& a, const void* A, const void*
     const size_t sm = (size_t)(S::TWS + S::TZ * TSZ) * sizeof(V) + (size_t)3 * S::N1 * S::THREADS_Z * sizeof(T);
     cudaError_t e = set_smem(k_fields_z<V, N>, sm);
     if (e != cudaSuccess) return e;
-    k_fields_z<V, N><<<dim3(N / S::TZ, N, S::kSplitGrids ? 4 : 1), S::THREADS_Z, sm, s>>>(a, (const T*)A, (const V*)R, (const V*)tw, (V*)W0);
+    k_fields_z<V, N><<<dim3(N / S::TZ, N, S::kSplitGrids ? a.grids : 1), S::THREADS_Z, sm, s>>>(a, (const T*)A, (const V*)R, (const V*)tw, (V*)W0);
     return cudaGetLastError();
 }
 
 template <typename V, int N>
-cudaError_t run_y(cudaStream_t s, const void* tw, void* W)
+cudaError_t run_y(cudaStream_t s, int grids, const void* tw, void* W)
 {
     using S = Shape<N>;
     constexpr int TS = S::template line_stride<sizeof(V), S::TX>();
     const size_t sm = (size_t)(S::TWS + S::TX * TS) * sizeof(V);
     cudaError_t e = set_smem(k_fields_y<V, N>, sm);
     if (e != cudaSuccess) return e;
-    k_fields_y<V, N><<<dim3(N / S::TX, N, 4), S::THREADS, sm, s>>>((const V*)tw, (V*)W);
+    k_fields_y<V, N><<<dim3(N / S::TX, N, grids), S::THREADS, sm, s>>>((const V*)tw, (V*)W);
     return cudaGetLastError();
 }
 
@@ -627,6 +676,19 @@ cudaError_t run_x(cudaStream_t s, const void* tw, const void* W, void* G)
     cudaError_t e = set_smem(k_fields_x<V, Gt, N>, sm);
     if (e != cudaSuccess) return e;
     k_fields_x<V, Gt, N><<<(unsigned)((size_t)N * N / S::XL), S::THREADS_X, sm, s>>>((const V*)tw, (const V*)W, (Gt*)G);
+    return cudaGetLastError();
+}
+
+template <typename V, typename Gt, int N>
+cudaError_t run_x_planar(cudaStream_t s, const void* tw, const void* W, double* out)
+{
+    using S = Shape<N>;
+    constexpr int LPB = S::THREADS / S::T;
+    const size_t sm = (size_t)(S::TWS + LPB * S::TSX) * sizeof(V);
+    cudaError_t e = set_smem(k_fields_x_planar<V, Gt, N>, sm);
+    if (e != cudaSuccess) return e;
+    k_fields_x_planar<V, Gt, N><<<dim3((unsigned)((size_t)N * N / LPB), 5), S::THREADS, sm, s>>>((const V*)tw,
+                                                                                              (const V*)W, out);
     return cudaGetLastError();
 }
 
@@ -723,6 +785,16 @@ cudaError_t launch_mode_tables(cudaStream_t s, int precision, const FieldArgs& a
     return cudaGetLastError();
 }
 
+cudaError_t launch_modes_once(cudaStream_t s, int precision, const FieldArgs& a, const double* tabs64, void* A, void* R)
+{
+    const int M = mode_table_size(a.N);
+    const size_t N3 = (size_t)a.N * a.N * a.N;
+    const unsigned nb = (unsigned)((M + 255) / 256 + ((N3 + 255) / 256 < 152 * 32 ? (N3 + 255) / 256 : 152 * 32));
+    if (precision == FDF_PREC_F64) k_modes_once<double2><<<nb, 256, 0, s>>>(a, M, tabs64, (double*)A, (double2*)R);
+    else k_modes_once<float2><<<nb, 256, 0, s>>>(a, M, tabs64, (float*)A, (float2*)R);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_noise(cudaStream_t s, int precision, const FieldArgs& a, void* R)
 {
     const size_t N3 = (size_t)a.N * a.N * a.N;
@@ -743,10 +815,10 @@ cudaError_t launch_fields_z(cudaStream_t s, int precision, const FieldArgs& a, c
 #undef Z32
 }
 
-cudaError_t launch_fields_y(cudaStream_t s, int precision, int N, const void* tw, void* W)
+cudaError_t launch_fields_y(cudaStream_t s, int precision, int N, int grids, const void* tw, void* W)
 {
-#define Y64(n) run_y<double2, n>(s, tw, W)
-#define Y32(n) run_y<float2, n>(s, tw, W)
+#define Y64(n) run_y<double2, n>(s, grids, tw, W)
+#define Y32(n) run_y<float2, n>(s, grids, tw, W)
     if (precision == FDF_PREC_F64) FDF_DISPATCH_N(N, Y64)
     FDF_DISPATCH_N(N, Y32)
 #undef Y64
@@ -766,15 +838,17 @@ cudaError_t launch_fields_x(cudaStream_t s, int precision, int N, const void* tw
 #undef X16
 }
 
-cudaError_t launch_fields_to_f64(cudaStream_t s, int precision, int N, const void* G, double* out, unsigned mask)
+cudaError_t launch_fields_x_planar(cudaStream_t s, int precision, int N, const void* tw, const void* W, double* out)
 {
-    const size_t N3 = (size_t)N * N * N;
-    const unsigned blocks = (unsigned)((N3 + 255) / 256 < 152 * 32 ? (N3 + 255) / 256 : 152 * 32);
-    if (precision == FDF_PREC_F64) k_fields_to_f64<double><<<blocks, 256, 0, s>>>(N3, (const double*)G, out, mask);
-    else if (precision == FDF_PREC_F32)
-        k_fields_to_f64<float><<<blocks, 256, 0, s>>>(N3, (const float*)G, out, mask);
-    else k_fields_to_f64<__nv_bfloat16><<<blocks, 256, 0, s>>>(N3, (const __nv_bfloat16*)G, out, mask);
-    return cudaGetLastError();
+#define P64(n) run_x_planar<double2, double, n>(s, tw, W, out)
+#define P32(n) run_x_planar<float2, float, n>(s, tw, W, out)
+#define P16(n) run_x_planar<float2, __nv_bfloat16, n>(s, tw, W, out)
+    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(N, P64)
+    if (precision == FDF_PREC_F32) FDF_DISPATCH_N(N, P32)
+    FDF_DISPATCH_N(N, P16)
+#undef P64
+#undef P32
+#undef P16
 }
 
 cudaError_t launch_fields_from_f64(cudaStream_t s, int precision, int N, const double* in, void* G)
