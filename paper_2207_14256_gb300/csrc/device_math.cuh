@@ -164,11 +164,37 @@ __device__ __forceinline__ void fixed_cell(uint32_t X, uint32_t N, uint32_t& i0,
     i1 = (i0 + 1u == N) ? 0u : i0 + 1u;
 }
 
+// FP64 fallbacks of the integer forms, as calls: inlined, the compiler would run their
+// FP64 instructions for every argument and select afterwards.
+static __device__ __noinline__ double rsqrt_slow(double u) { return rsqrt_fp64(u); }
+static __device__ __noinline__ double square_slow(double r) { return r * r; }
+static __device__ __noinline__ double add_slow(double q, float d) { return q + f2d_bits(d); }
+static __device__ __noinline__ double sqrt_slow(double u) { return __dsqrt_rn(u); }
+static __device__ __noinline__ double div_slow(double a, double b) { return __ddiv_rn(a, b); }
+
+// sqrt(u), correctly rounded (__dsqrt_rn's bits from the integer pipe, but for the few
+// arguments that w_sqrt53 leaves to it).
+__device__ __forceinline__ double sqrt_rn(double u)
+{
+    double r;
+    if (!w_sqrt53(u, rsqrtf(d2f_bits(u)), r)) r = sqrt_slow(u);
+    return r;
+}
+
+// a 32-bit fraction X / 2^32 as a double, from its bits
+__device__ __forceinline__ double frac32(uint32_t X)
+{
+    const int z = __clz((int)X);                 // the leading one is worth 2^(-1 - z)
+    const uint32_t m = (X << z) << 1;            // the bits below it
+    const uint32_t hi = (uint32_t)(1022 - z) << 20;
+    return __hiloint2double(X ? (int)(hi | (m >> 12)) : 0, (int)(m << 20));
+}
+
 // |q| with the sampler's exactly rounded evaluation order, so that an
 // untouched momentum reproduces p = |q_sampled| bit for bit.
 __device__ __forceinline__ double norm3_rn(const double q[3])
 {
-    return __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(q[0], q[0]), __dmul_rn(q[1], q[1])), __dmul_rn(q[2], q[2])));
+    return sqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(q[0], q[0]), __dmul_rn(q[1], q[1])), __dmul_rn(q[2], q[2])));
 }
 
 // delta-f weight (Sec. 2.2), w = 1 - fbar(|q|)/fbar(p), in the cancellation-free form
@@ -181,10 +207,14 @@ __device__ __forceinline__ double dfweight(double qm, double p, double T)
 // The same weight as the FP32/BF16-grid forms compute it: the small difference p - |q| in
 // FP64 (|q| from norm3_rn), the rest in FP32 (their momenta carry FP32 rounding
 // already, and GB300's FP64 transcendental functions are slow).
-__device__ __forceinline__ float dfweight_split(double qm, double p, double T)
+// (p - |q|)/T, as FP32, is the product with invT = 1/T unless that lies within 8 FP64 last
+// places of a tie (the product and the quotient differ by two): then the quotient is taken.
+__device__ __forceinline__ float dfweight_split(double qm, double p, double T, double invT)
 {
-    const float arg = (float)((p - qm) / T);
-    return -expm1f(arg) / (1.f + expf(-(float)qm / (float)T));
+    const double d = p - qm;
+    double a = d * invT;
+    if (((uint32_t)__double2loint(a) & 0x1FFFFFFFu) - (0x10000000u - 8u) <= 16u) a = div_slow(d, T);
+    return -expm1f(w_d2f(a)) / (1.f + expf(-w_d2f(qm) / (float)T));
 }
 
 }  // namespace fdf

@@ -399,39 +399,56 @@ __device__ __forceinline__ uint32_t round_mod32(FF d)
     return (uint32_t)i + (uint32_t)i2;
 }
 
+// 1/sqrt(u) for any u >= 0
+__device__ __forceinline__ double rsqrt_any(double u)
+{
+    double r;
+    if (!w_rsqrt53(u, rsqrtf(d2f_bits(u)), r)) r = u > 1.2e-38 && u < 3.4e38 ? rsqrt_slow(u) : div_slow(1.0, sqrt_slow(u));
+    return r;
+}
+
 struct Masses {
     double m[kMaxSpecies];
 };
+
+// the mass of particle i, n_part per species (comparisons instead of a 64-bit division, and
+// no indexed copy of the parameter)
+__device__ __forceinline__ double mass_at(const Masses& ms, int64_t i, int64_t n_part)
+{
+    double m = ms.m[0];
+    m = i >= n_part ? ms.m[1] : m;
+    m = i >= 2 * n_part ? ms.m[2] : m;
+    return i >= 3 * n_part ? ms.m[3] : m;
+}
 
 // ---- initial transform -----------------------------------------------------
 // q_i <- q_i (1 - psi/2) - (eps tau_0 / 6) d_i psi  (eq:transform with delta = -2 psi,
 // theta = k^2 tau psi / 2, nu = 4, omega = 4/3), eps = sqrt(p^2 + m^2 a_0^2).
 // F: the state form (kPlain, kWide, kFixed).  The transform reads the fields at the
-// sampled fixed-point positions in every form.
+// sampled fixed-point positions in every form.  ms: m^2 a_0^2 per species.
 template <int F, typename Gt>
 __global__ void __launch_bounds__(kThreads) k_initial(ParticleState st, int64_t n, int64_t n_part, Masses ms,
-                                                      double a0, double tau0, int order, int N, double L,
+                                                      double tau0, int order, int N, double L,
                                                       const Gt* __restrict__ G)
 {
     const double tau0_6 = tau0 / 6.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double m = ms.m[i / n_part];
+        const double m2a2 = mass_at(ms, i, n_part);
         const uint32_t X0 = st.X[i], X1 = st.X[n + i], X2 = st.X[2 * n + i];
         double g[8];
-        double x[3];
-        x[0] = L * ((double)X0 * 2.3283064365386963e-10);
-        x[1] = L * ((double)X1 * 2.3283064365386963e-10);
-        x[2] = L * ((double)X2 * 2.3283064365386963e-10);
+        const double x[3] = {L * frac32(X0), L * frac32(X1), L * frac32(X2)};
         if constexpr (F == kPlain) {
             gather_f64_order<8>(order, reinterpret_cast<const double*>(G), N, (double)N / L, x, g);
         } else {
             float gf[8];
             gather_order<Gt>(order, G, (uint32_t)N, X0, X1, X2, gf);
 #pragma unroll
-            for (int s = 0; s < 8; ++s) g[s] = (double)gf[s];
+            for (int s = 0; s < 8; ++s) g[s] = f2d_bits(gf[s]);
         }
+        // eps scales a term of ~1e-9 of q: a root through rsqrt_any serves it
         const double p = st.pmag[i];
-        const double eps = sqrt(p * p + m * m * a0 * a0);
+        const double e2 = p * p + m2a2;
+        const double eps = __double_as_longlong(e2) > 0 ? e2 * rsqrt_any(e2) : 0.0;
         const double c = eps * tau0_6;          // eps tau0 / 6 (tau0/6 formed once)
         const double r = 1.0 - 0.5 * g[7];
 #pragma unroll
@@ -811,7 +828,7 @@ __device__ __forceinline__ double wide_poly(const WidePoly& P, double t, float t
 __device__ __forceinline__ double rsqrt_int(double u)
 {
     double r;
-    if (!w_rsqrt53(u, rsqrtf(d2f_bits(u)), r)) r = rsqrt_fp64(u);
+    if (!w_rsqrt53(u, rsqrtf(d2f_bits(u)), r)) r = rsqrt_slow(u);
     return r;
 }
 
@@ -824,8 +841,8 @@ __device__ __forceinline__ double rsqrt_int(double u, double& t)
     const bool ok = w_rsqrt53(u, rsqrtf(d2f_bits(u)), r, R, k);
     t = w_square53(R, k);
     if (!ok) {
-        r = rsqrt_fp64(u);
-        t = r * r;
+        r = rsqrt_slow(u);
+        t = square_slow(r);
     }
     return r;
 }
@@ -840,7 +857,7 @@ __device__ __forceinline__ void add_small(double q[3], const float d[3])
     if (!(ok[0] && ok[1] && ok[2])) {
 #pragma unroll
         for (int c = 0; c < 3; ++c)
-            if (!ok[c]) r[c] = q[c] + f2d_bits(d[c]);
+            if (!ok[c]) r[c] = add_slow(q[c], d[c]);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) q[c] = r[c];
@@ -1053,14 +1070,6 @@ void push_wide(cudaStream_t s, unsigned b, const PushArgs& a, const ParticleStat
 // roots and divisions, of which the trilinear read of seven FP64 slots takes 71.  128^3
 // particles, one step: 1224 -> 525 us.
 
-// 1/sqrt(u) for any u >= 0
-__device__ __forceinline__ double rsqrt_any(double u)
-{
-    double r;
-    if (!w_rsqrt53(u, rsqrtf(d2f_bits(u)), r)) r = u > 1.2e-38 && u < 3.4e38 ? rsqrt_fp64(u) : 1.0 / sqrt(u);
-    return r;
-}
-
 template <bool EXACT>
 __global__ void __launch_bounds__(kThreads) k_push_f64(const __grid_constant__ PushArgs a, double* __restrict__ xd,
                                                        double* __restrict__ qd, const double* __restrict__ q0d,
@@ -1141,8 +1150,8 @@ __device__ __forceinline__ void load_state(const ParticleState& st, int64_t n, i
             x[d] = st.xd[d * n + i];
             q[d] = st.qd[d * n + i];
         } else {
-            x[d] = L * ((double)st.X[d * n + i] * 2.3283064365386963e-10);
-            q[d] = (double)st.q0f[d * n + i] + (double)st.dqf[d * n + i];
+            x[d] = L * frac32(st.X[d * n + i]);
+            q[d] = f2d_bits(st.q0f[d * n + i]) + f2d_bits(st.dqf[d * n + i]);
         }
     }
 }
@@ -1152,6 +1161,7 @@ __global__ void __launch_bounds__(kThreads) k_export(ParticleState st, int64_t n
                                                      double L, double T, double* __restrict__ xo,
                                                      double* __restrict__ qo, double* __restrict__ wo)
 {
+    const double invT = 1.0 / T;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < count;
          j += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = begin + j;
@@ -1170,7 +1180,7 @@ __global__ void __launch_bounds__(kThreads) k_export(ParticleState st, int64_t n
         }
         if (wo) {
             if constexpr (F == kPlain) wo[o] = dfweight(norm3_rn(q), st.pmag[i], T);
-            else wo[o] = (double)dfweight_split(norm3_rn(q), st.pmag[i], T);
+            else wo[o] = (double)dfweight_split(norm3_rn(q), st.pmag[i], T, invT);
         }
     }
 }
@@ -1221,7 +1231,7 @@ __global__ void __launch_bounds__(kThreads) k_accel_terms(ParticleState st, int6
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < count;
          j += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = begin + j;
-        const double m = ms.m[i / n_part];
+        const double m = mass_at(ms, i, n_part);
         double x[3], q[3], g[8];
         load_state<F>(st, n, i, L, x, q);
         if constexpr (F == kPlain) {
@@ -1286,13 +1296,16 @@ __device__ __forceinline__ void peer_sum(T (&v)[K], unsigned peers)
     }
 }
 
+// Bound: the FP64 pipe as long as |q| and the weight's quotient ran there; with their bits
+// from the integer pipe and no FP64 conversions, 3 x 200^3 particles take 0.99 ms against
+// 2.21 ms (the L2 atomics and the state's 60 bytes per particle share what is left).
 template <int F, bool PRESUM>
 __global__ void __launch_bounds__(kThreads) k_deposit(ParticleState st, int64_t n, int64_t begin, int64_t count,
                                                       int64_t n_part, Masses ms, double a, double T, int quantity,
                                                       int parity, int order, int N, double L,
                                                       double* __restrict__ grid)
 {
-    const double invh = (double)N / L;
+    const double invh = (double)N / L, invT = 1.0 / T;
     // Warp-uniform trips: the lanes of a warp take 32 consecutive particles (neighbours in
     // the bucket order of the last sort) and stay converged for the pre-sum.
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1302,11 +1315,12 @@ __global__ void __launch_bounds__(kThreads) k_deposit(ParticleState st, int64_t 
         const int64_t i = begin + (live ? j : 0);
         if (live && parity >= 0 && (int)(st.id[i] & 1u) != parity) live = false;
         if (!PRESUM && !live) continue;
-        const double m = ms.m[i / n_part];
+        const double m = mass_at(ms, i, n_part);
         double x[3], q[3];
         load_state<F>(st, n, i, L, x, q);
         const double qm = norm3_rn(q);
         double v = 1.0;
+        float vf = 1.f;
         if constexpr (F == kPlain) {
             const double eps = sqrt(qm * qm + m * m * a * a);
             if (quantity == FDF_Q_W_EPS) v = dfweight(qm, st.pmag[i], T) * eps;
@@ -1317,14 +1331,14 @@ __global__ void __launch_bounds__(kThreads) k_deposit(ParticleState st, int64_t 
             // The FP32-grid forms deposit in FP32 arithmetic (FP64 sums): the weight's
             // argument p - |q| (a small difference) is formed in FP64 first, and the
             // kernel weights of an FP64 position take its fraction from FP64.
-            const float qf = (float)qm;
-            const float ma = (float)(m * a);
+            const float qf = w_d2f(qm);
+            const float ma = w_d2f(m * a);
             const float eps = sqrtf(fmaf(qf, qf, ma * ma));
-            const float w = dfweight_split(qm, st.pmag[i], T);
-            if (quantity == FDF_Q_W_EPS) v = (double)(w * eps);
-            else if (quantity == FDF_Q_W) v = (double)w;
-            else if (quantity == FDF_Q_EPS) v = (double)eps;
-            else if (quantity >= FDF_Q_W_QX) v = (double)(w * (float)q[quantity - FDF_Q_W_QX]);
+            const float w = dfweight_split(qm, st.pmag[i], T, invT);
+            if (quantity == FDF_Q_W_EPS) vf = w * eps;
+            else if (quantity == FDF_Q_W) vf = w;
+            else if (quantity == FDF_Q_EPS) vf = eps;
+            else if (quantity >= FDF_Q_W_QX) vf = w * w_d2f(q[quantity - FDF_Q_W_QX]);
         }
         // per axis: the kernel's nodes and weights (order 1: 2 nodes, order 2: 3), in the
         // form's deposit precision
@@ -1337,14 +1351,19 @@ __global__ void __launch_bounds__(kThreads) k_deposit(ParticleState st, int64_t 
             if constexpr (F != kFixed) {
                 u = x[d] * invh;
             } else {
+                // the cell, and the fraction from the low product word
                 const uint32_t Xd = st.X[d * n + i];
-                u = (double)__umulhi(Xd, (uint32_t)N) + (double)(Xd * (uint32_t)N) * 2.3283064365386963e-10;
+                u = (double)__umulhi(Xd, (uint32_t)N) + frac32(Xd * (uint32_t)N);
             }
-            const double c = order == 2 ? floor(u + 0.5) : floor(u);
-            const Wt e = (Wt)(u - c);
-            int ii = (int)c;
+            // floor(u) as u + 2^52 rounded down: the sum's low word is the integer
+            const double c52 = __dadd_rd(order == 2 ? u + 0.5 : u, 4503599627370496.0);
+            const double frac = u - (c52 - 4503599627370496.0);
+            Wt e;
+            if constexpr (F == kPlain) e = frac;
+            else e = w_d2f(frac);
+            int ii = __double2loint(c52);
             if (ii >= N) ii -= N;
-            if (ii < 0) ii += N;
+            ii = ii < 0 || ii >= N ? 0 : ii;       // (never taken for x in [0, L); keeps writes in the grid)
             if (order == 2) {
                 idx[d][0] = ii == 0 ? N - 1 : ii - 1;
                 idx[d][1] = ii;
@@ -1361,7 +1380,14 @@ __global__ void __launch_bounds__(kThreads) k_deposit(ParticleState st, int64_t 
                 w[d][2] = Wt(0);
             }
         }
-        const Wt vw = (Wt)v;
+        Wt vw;
+        if constexpr (F == kPlain) vw = v;
+        else vw = vf;
+        // (an FP64 conversion costs an FP64 slot)
+        auto to64 = [](Wt t) {
+            if constexpr (F == kPlain) return t;
+            else return f2d_bits(t);
+        };
         if constexpr (PRESUM) {
             // Particles sharing the base cell share every node: one match on it, sums
             // over the set by shuffles, and one atomic per set and node.
@@ -1371,7 +1397,7 @@ __global__ void __launch_bounds__(kThreads) k_deposit(ParticleState st, int64_t 
             if (order == 2) {
                 double c[27];
 #pragma unroll
-                for (int k = 0; k < 27; ++k) c[k] = live ? (double)(w[0][k % 3] * w[1][(k / 3) % 3] * w[2][k / 9] * vw) : 0.0;
+                for (int k = 0; k < 27; ++k) c[k] = live ? to64(w[0][k % 3] * w[1][(k / 3) % 3] * w[2][k / 9] * vw) : 0.0;
                 peer_sum<27>(c, peers);
                 if (lead) {
 #pragma unroll
@@ -1381,7 +1407,7 @@ __global__ void __launch_bounds__(kThreads) k_deposit(ParticleState st, int64_t 
             } else {
                 double c[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) c[k] = live ? (double)(w[0][k & 1] * w[1][(k >> 1) & 1] * w[2][k >> 2] * vw) : 0.0;
+                for (int k = 0; k < 8; ++k) c[k] = live ? to64(w[0][k & 1] * w[1][(k >> 1) & 1] * w[2][k >> 2] * vw) : 0.0;
                 peer_sum<8>(c, peers);
                 if (lead) {
 #pragma unroll
@@ -1396,7 +1422,7 @@ __global__ void __launch_bounds__(kThreads) k_deposit(ParticleState st, int64_t 
                     for (int cx = 0; cx < m3; ++cx) {
                         const Wt wt = w[0][cx] * w[1][cy] * w[2][cz];
                         const size_t cell = ((size_t)idx[2][cz] * N + idx[1][cy]) * N + idx[0][cx];
-                        atomicAdd(grid + cell, (double)(wt * vw));
+                        atomicAdd(grid + cell, to64(wt * vw));
                     }
         }
     }
@@ -1416,10 +1442,11 @@ cudaError_t launch_initial(cudaStream_t s, int precision, const ParticleState& s
 {
     if (n <= 0) return cudaSuccess;
     const unsigned b = grid_for(n);
-    const Masses ms = masses_of(m_ev);
+    Masses ms = masses_of(m_ev);
+    for (double& m : ms.m) m = m * m * a0 * a0;
     const int f = form_of(precision), gp = grid_prec(precision);
 #define FDF_INITIAL(F_, Gt_) \
-    k_initial<F_, Gt_><<<b, kThreads, 0, s>>>(st, n, n_part, ms, a0, tau0, order, N, L, (const Gt_*)G)
+    k_initial<F_, Gt_><<<b, kThreads, 0, s>>>(st, n, n_part, ms, tau0, order, N, L, (const Gt_*)G)
     if (f == kPlain) FDF_INITIAL(kPlain, double);
     else if (f == kWide && gp == FDF_PREC_F32) FDF_INITIAL(kWide, float);
     else if (f == kWide) FDF_INITIAL(kWide, __nv_bfloat16);

@@ -16,23 +16,31 @@
 
 namespace fdf {
 
-// u = m 2^-53 with the 53-bit integer m = (w0 >> 5) 2^26 + (w1 >> 6): the integer is
-// formed exactly in 64 bits and converted exactly (m < 2^53), so only one FP64
-// conversion and one exact power-of-two scaling are spent (the GPU's FP64 rate is low).
+// The 53-bit integer m = (w0 >> 5) 2^26 + (w1 >> 6) of two words, exact in 64 bits.
 __device__ __forceinline__ uint64_t m53(uint32_t w0, uint32_t w1)
 {
     return ((uint64_t)(w0 >> 5) << 26) | (uint64_t)(w1 >> 6);
 }
 
-__device__ __forceinline__ double u53(uint32_t w0, uint32_t w1)
+// 1 + (m mod 2^52) 2^-52, a bit pattern (no FP64 conversion, which costs an FP64 slot)
+__device__ __forceinline__ double one_plus(uint64_t m)
 {
-    return __dmul_rn(__ull2double_rn(m53(w0, w1)), 1.1102230246251565404e-16);  // 2^-53
+    return __longlong_as_double((long long)((m & 0xFFFFFFFFFFFFFull) | 0x3FF0000000000000ull));
 }
 
-// v = 2u - 1 = (m - 2^52) 2^-52, exact (|m - 2^52| <= 2^52)
+// u = m 2^-53, exact
+__device__ __forceinline__ double u53(uint32_t w0, uint32_t w1)
+{
+    const uint64_t m = m53(w0, w1);
+    const double x = (m >> 52) ? one_plus(m) : __dsub_rn(one_plus(m), 1.0);    // m 2^-52
+    return __dmul_rn(x, 0.5);
+}
+
+// v = 2u - 1 = (m - 2^52) 2^-52, exact
 __device__ __forceinline__ double v53(uint32_t w0, uint32_t w1)
 {
-    return __dmul_rn(__ll2double_rn((long long)m53(w0, w1) - (1ll << 52)), 2.220446049250313080847e-16);  // 2^-52
+    const uint64_t m = m53(w0, w1);
+    return __dsub_rn(one_plus(m), (m >> 52) ? 1.0 : 2.0);
 }
 
 __device__ __forceinline__ double fd_inverse(const double* __restrict__ t, const double* __restrict__ F, int n,
@@ -55,18 +63,28 @@ __device__ __forceinline__ double fd_inverse(const double* __restrict__ t, const
     return __dadd_rn(t[lo], __ddiv_rn(__dmul_rn(du, dt), dF));
 }
 
-// Attempt `att` of the direction of particle (g0, g1): v from streams 2 and 3;
-// accepted when 1e-300 < |v|^2 <= 1.
+// Attempt `att` of the direction of particle (g0, g1): the words of v from streams 2 and 3;
+// accepted when 1e-300 < |v|^2 <= 1 in FP64.  FP32 settles that (the top 32 bits of each
+// component, |v|^2 to 3e-7) unless |v|^2 is within 1e-6 of 1 or of 0.
 __device__ __forceinline__ bool direction_attempt(uint32_t g0, uint32_t g1, uint32_t att, uint32_t key0, uint32_t key1,
-                                                  double& v0, double& v1, double& v2, double& r2)
+                                                  uint32_t w[6])
 {
     const uint4 a = philox4x32_10(make_uint4(g0, g1, 2u, att), key0, key1);
     const uint4 b = philox4x32_10(make_uint4(g0, g1, 3u, att), key0, key1);
-    v0 = v53(a.x, a.y);
-    v1 = v53(a.z, a.w);
-    v2 = v53(b.x, b.y);
-    r2 = __dadd_rn(__dadd_rn(__dmul_rn(v0, v0), __dmul_rn(v1, v1)), __dmul_rn(v2, v2));
-    return (r2 > 1e-300) && (r2 <= 1.0);
+    w[0] = a.x;
+    w[1] = a.y;
+    w[2] = a.z;
+    w[3] = a.w;
+    w[4] = b.x;
+    w[5] = b.y;
+    // m >> 21 is the first word: (w0 - 2^31) 2^-31 is v to 2^-31
+    const float f0 = (float)(int)(a.x - 0x80000000u), f1 = (float)(int)(a.z - 0x80000000u);
+    const float f2 = (float)(int)(b.x - 0x80000000u);
+    const float r2 = (f0 * f0 + f1 * f1 + f2 * f2) * 2.168404344971009e-19f;   // 2^-62
+    if (fabsf(r2 - 1.f) > 1e-6f && r2 > 1e-6f) return r2 < 1.f;
+    const double v0 = v53(w[0], w[1]), v1 = v53(w[2], w[3]), v2 = v53(w[4], w[5]);
+    const double s = __dadd_rn(__dadd_rn(__dmul_rn(v0, v0), __dmul_rn(v1, v1)), __dmul_rn(v2, v2));
+    return (s > 1e-300) && (s <= 1.0);
 }
 
 constexpr uint32_t kMaxAttempts = 64;
@@ -78,8 +96,7 @@ constexpr uint32_t kMaxAttempts = 64;
 // still pending over all 32 lanes: with np pending, lane l tries attempt
 // next + l / np of the (l mod np)-th pending particle.  Lanes without a particle
 // (live = false) only help.  Returns whether this lane's particle got a direction.
-__device__ bool warp_direction(bool live, uint32_t g0, uint32_t g1, uint32_t key0, uint32_t key1, double& v0,
-                               double& v1, double& v2, double& r2)
+__device__ bool warp_direction(bool live, uint32_t g0, uint32_t g1, uint32_t key0, uint32_t key1, uint32_t v[6])
 {
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -94,8 +111,8 @@ __device__ bool warp_direction(bool live, uint32_t g0, uint32_t g1, uint32_t key
         const int owner = __ffs(m) - 1;
         const uint32_t og0 = __shfl_sync(full, g0, owner), og1 = __shfl_sync(full, g1, owner);
         const uint32_t att = __shfl_sync(full, next, owner) + (uint32_t)rep;
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, ar2 = 0.0;
-        const bool acc = att < kMaxAttempts && direction_attempt(og0, og1, att, key0, key1, a0, a1, a2, ar2);
+        uint32_t a[6] = {0u, 0u, 0u, 0u, 0u, 0u};
+        const bool acc = att < kMaxAttempts && direction_attempt(og0, og1, att, key0, key1, a);
         const unsigned accepted = __ballot_sync(full, acc);
         // an owner's lanes are its rank r + j np, j = 0, 1, ...: the lowest accepted one wins
         const bool mine = (pending >> lane) & 1u;
@@ -105,15 +122,14 @@ __device__ bool warp_direction(bool live, uint32_t g0, uint32_t g1, uint32_t key
             for (int l = r; l < 32; l += np) lanes |= 1u << l;
         const int win = mine ? __ffs(accepted & lanes) - 1 : -1;
         const int src = win >= 0 ? win : lane;
-        const double w0 = __shfl_sync(full, a0, src), w1 = __shfl_sync(full, a1, src);
-        const double w2 = __shfl_sync(full, a2, src), wr2 = __shfl_sync(full, ar2, src);
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const uint32_t w = __shfl_sync(full, a[j], src);
+            if (win >= 0) v[j] = w;
+        }
         bool done = false;
         if (mine) {
             if (win >= 0) {
-                v0 = w0;
-                v1 = w1;
-                v2 = w2;
-                r2 = wr2;
                 ok = true;
                 done = true;
             } else {
@@ -126,40 +142,57 @@ __device__ bool warp_direction(bool live, uint32_t g0, uint32_t g1, uint32_t key
     return ok;
 }
 
-__global__ void __launch_bounds__(256) k_sample(int64_t n, uint32_t key0, uint32_t key1, double T_ev,
+// a / b, correctly rounded (__ddiv_rn's bits), with inv within a few last places of 1/b
+__device__ __forceinline__ double div_rn(double a, double b, double inv)
+{
+    double r;
+    if (!w_div53(a, b, a * inv, r)) r = div_slow(a, b);
+    return r;
+}
+
+// Bound: the FP64 pipe.  The roots and quotients have their correctly rounded bits from the
+// integer pipe, and attempts are settled in FP32: 36 FP64 instructions per particle
+// against 105 (3 x 200^3 particles: 4.63 -> 1.71 ms).  The FP64 fallbacks are calls
+// (sqrt_slow and its kin): inlined, they ran for every particle (3.54 ms).
+__global__ void __launch_bounds__(256) k_sample(int64_t N, uint32_t key0, uint32_t key1, double T_ev,
                                                 const double* __restrict__ cdf_t, const double* __restrict__ cdf_F,
                                                 int ncdf, uint32_t* __restrict__ X, double* __restrict__ qs,
                                                 double* __restrict__ pmag, uint32_t* __restrict__ id, int* flag)
 {
     // warp-uniform trip count: every lane takes part in the warp's direction rounds
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x; i0 < n; i0 += stride) {
+    for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x; i0 < N; i0 += stride) {
         const int64_t i = i0 + threadIdx.x;
-        const bool live = i < n;
+        const bool live = i < N;
         const uint32_t g0 = (uint32_t)i, g1 = (uint32_t)((uint64_t)i >> 32);
-        double v0 = 0.0, v1 = 0.0, v2 = 0.0, r2 = 0.0;
-        bool ok = warp_direction(live, g0, g1, key0, key1, v0, v1, v2, r2);
+        uint32_t v[6] = {0u, 0u, 0u, 0u, 0u, 0u};
+        const bool ok = warp_direction(live, g0, g1, key0, key1, v);
         if (!live) continue;
         uint4 w = philox4x32_10(make_uint4(g0, g1, 0u, 0u), key0, key1);
         X[i] = w.x;
-        X[n + i] = w.y;
-        X[2 * n + i] = w.z;
+        X[N + i] = w.y;
+        X[2 * N + i] = w.z;
         w = philox4x32_10(make_uint4(g0, g1, 1u, 0u), key0, key1);
         const double qmag = __dmul_rn(T_ev, fd_inverse(cdf_t, cdf_F, ncdf, u53(w.x, w.y)));
+        double v0 = v53(v[0], v[1]), v1 = v53(v[2], v[3]), v2 = v53(v[4], v[5]);
+        double r2 = __dadd_rn(__dadd_rn(__dmul_rn(v0, v0), __dmul_rn(v1, v1)), __dmul_rn(v2, v2));
         if (!ok) {
             atomicOr(flag, 1);
             r2 = 1.0;
             v0 = 1.0;
             v1 = v2 = 0.0;
         }
-        const double s = __dsqrt_rn(r2);
-        const double q0 = __dmul_rn(qmag, __ddiv_rn(v0, s));
-        const double q1 = __dmul_rn(qmag, __ddiv_rn(v1, s));
-        const double q2 = __dmul_rn(qmag, __ddiv_rn(v2, s));
-        qs[i] = q0;
-        qs[n + i] = q1;
-        qs[2 * n + i] = q2;
-        pmag[i] = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(q0, q0), __dmul_rn(q1, q1)), __dmul_rn(q2, q2)));
+        // v / sqrt(r2): the quotients' estimates from 1/sqrt(r2)
+        const float y = rsqrtf(d2f_bits(r2));
+        double s, inv;
+        if (!w_sqrt53(r2, y, s)) s = sqrt_slow(r2);
+        if (!w_rsqrt53(r2, y, inv)) inv = div_slow(1.0, s);
+        const double n[3] = {div_rn(v0, s, inv), div_rn(v1, s, inv), div_rn(v2, s, inv)};
+        const double q[3] = {__dmul_rn(qmag, n[0]), __dmul_rn(qmag, n[1]), __dmul_rn(qmag, n[2])};
+        qs[i] = q[0];
+        qs[N + i] = q[1];
+        qs[2 * N + i] = q[2];
+        pmag[i] = norm3_rn(q);
         id[i] = (uint32_t)i;
     }
 }

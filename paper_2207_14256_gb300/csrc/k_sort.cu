@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_keys(ParticleState st, int64_
         const bool live = i < n;
         const unsigned active = __ballot_sync(0xffffffffu, live);
         if (!live) continue;
-        const uint32_t s = (uint32_t)(i / n_part);
+        const uint32_t s = (uint32_t)(i >= n_part) + (uint32_t)(i >= 2 * n_part) + (uint32_t)(i >= 3 * n_part);
         uint32_t c[3];
         if constexpr (F == kPlain) {
 #pragma unroll
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_keys(ParticleState st, int64_
             float q[3], q2 = 0.f;
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                q[d] = (float)st.qd[d * n + i];
+                q[d] = d2f_bits(st.qd[d * n + i]);      // (an FP64 conversion costs an FP64 slot)
                 q2 = fmaf(q[d], q[d], q2);
             }
             const float k = lead.on ? lead.dtau_q32[s] * ((float)N * 2.3283064365386963e-10f) *
@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_keys(ParticleState st, int64_
                                     : 0.f;
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                float u = (float)st.xd[d * n + i] * (float)invh + q[d] * k;
+                float u = d2f_bits(st.xd[d * n + i]) * (float)invh + q[d] * k;
                 u = fminf(fmaxf(u, -1.0e6f), 1.0e6f);      // a saturated lead is only a poor guess
                 int ci = (int)floorf(u) % (int)N;
                 ci = ci < 0 ? ci + (int)N : ci;
@@ -437,6 +437,7 @@ __global__ void __launch_bounds__(kThreads) k_export_unpack(const void* __restri
                                                             double T, double* __restrict__ xo,
                                                             double* __restrict__ qo, double* __restrict__ wo)
 {
+    const double invT = 1.0 / T;
     for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < count;
          o += (int64_t)gridDim.x * blockDim.x) {
         double x[3], q[3], pm;
@@ -457,8 +458,8 @@ __global__ void __launch_bounds__(kThreads) k_export_unpack(const void* __restri
         } else {
             const SplitRec r = load_split(recs, o);
             for (int d = 0; d < 3; ++d) {
-                x[d] = L * ((double)r.X[d] * 2.3283064365386963e-10);
-                q[d] = (double)r.q0[d] + (double)r.dq[d];
+                x[d] = L * frac32(r.X[d]);
+                q[d] = f2d_bits(r.q0[d]) + f2d_bits(r.dq[d]);
             }
             pm = r.pmag;
         }
@@ -474,7 +475,7 @@ __global__ void __launch_bounds__(kThreads) k_export_unpack(const void* __restri
         }
         if (wo) {
             if constexpr (F == kPlain) wo[o] = dfweight(norm3_rn(q), pm, T);
-            else wo[o] = (double)dfweight_split(norm3_rn(q), pm, T);
+            else wo[o] = (double)dfweight_split(norm3_rn(q), pm, T, invT);
         }
     }
 }

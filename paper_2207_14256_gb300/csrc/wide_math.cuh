@@ -10,7 +10,8 @@
 //   w_rsqrt53: rsqrt_fp64's four FP64 instructions (~50 others), w_square53 its square (~20);
 //   w_add:     the sum of a double and a much smaller float (~25, and no conversion);
 //   w_kick:    the kick's integrals as the FP32 values their user reads (9 FP64
-//              instructions as polynomials, 8 per node as sums).
+//              instructions as polynomials, 8 per node as sums);
+//   w_sqrt53, w_div53: correctly rounded roots and quotients (the sampler, |q|, the weights).
 // tests/test_wide_math.py compares both with the FP64 formulas, bit for bit.
 //
 // Plain C++ besides the intrinsics, so that the test compiles it for the host.
@@ -115,6 +116,84 @@ FDF_DEV bool w_add(double q, float d, double& r)
     r = __hiloint2double((int)bh, (int)(uint32_t)b);
     return L <= 27 && ed != 255 && (uint32_t)(eq - 1) < 0x7FEu && ((bh ^ hi) >> 20) == 0u &&
            ((bh & 0xFFFFFu) | (uint32_t)b) != 0u;
+}
+
+// ---- correctly rounded root and quotient ------------------------------------------------
+// An estimate within a few last places, its exact remainder modulo 2^64 (the remainder is
+// small, so the low 64 bits hold it), the correction that the remainder asks for, and a test
+// of the corrected remainder that no other 53-bit number is nearer: the IEEE result
+// whatever the estimate's error, or false.
+
+// sqrt(u) from the FP32 estimate yf = rsqrtf(d2f_bits(u)): u = M 2^-52 4^k and the root
+// S 2^(k-52), 2^52 <= S < 2^53, where S^2 is nearest M 2^52.
+FDF_DEV bool w_sqrt53(double u, float yf, double& root)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(u), lo = (uint32_t)__double2loint(u);
+    const int ex = (int)(hi >> 20) - 1023, k = ex >> 1, odd = ex & 1;
+    const uint32_t m1 = (hi & 0xFFFFFu) | 0x100000u;
+    const uint32_t Mh = odd ? (m1 << 1) | (lo >> 31) : m1, Ml = lo << odd;
+    const uint32_t yb = __float_as_uint(yf);
+    const uint32_t Y = (yb & 0x7FFFFFu) | 0x800000u;
+    bool ok = hi - 0x38100000u < 0x0FE00000u && (int)(yb >> 23) + k == 126;
+    // V = m h and E = (1 - V h) / 2 as in w_rsqrt53; the root is V (1 + 2 E / 2 ...): V + V E
+    const uint64_t a = (uint64_t)Ml * Y;
+    const uint64_t b = (uint64_t)Mh * Y + (a >> 32);
+    const uint32_t al = (uint32_t)a, bl = (uint32_t)b, bh = (uint32_t)(b >> 32);
+    const uint64_t V = ((uint64_t)__funnelshift_l(bl, bh, 8) << 32) | __funnelshift_l(al, bl, 8);
+    const uint32_t Vh = (uint32_t)(V >> 32), Vl = (uint32_t)V;
+    const int64_t E = -(int64_t)((uint64_t)Vl * Y + ((uint64_t)(Vh * Y) << 32));     // units of 2^-77
+    // V (E + 3 E^2 / 2) in units of 2^-52
+    const float eh = __fmul_rn(__int2float_rn((int)(E >> 25)), 2.220446049250313081e-16f);     // 2^-52
+    const float kap = __fmul_rn(__fmul_rn(1.5f, eh), eh);
+    const int64_t step = (((int64_t)(int)(V >> 22) * (int)(E >> 25)) >> 30) +
+                         __float2int_rn(__fmul_rn(__fmul_rn(kap, __uint2float_rn(Vh)), 4294967296.f));
+    const uint64_t S0 = V + (uint64_t)step;
+    const uint32_t Sl = (uint32_t)S0, Sh = (uint32_t)(S0 >> 32);
+    int64_t rem = (int64_t)(((uint64_t)Ml << 52) - ((uint64_t)Sl * Sl + ((uint64_t)(2u * Sl * Sh) << 32)));
+    // n = rem / (2 S), 1 / (2 S) = h 2^-53
+    const int n = __float2int_rn(__fmul_rn(__fmul_rn(__int2float_rn((int)(rem >> 32)), __uint2float_rn(Y)),
+                                           2.842170943040401e-14f));                           // 2^(32 - 53 - 24)
+    const int64_t S = (int64_t)S0 + n;
+    rem -= n * ((int64_t)S0 + S);
+    ok = ok && rem <= S && rem > -S && (uint32_t)((uint64_t)S >> 52) == 1u;
+    root = __hiloint2double((int)((uint32_t)((uint64_t)S >> 32) + ((uint32_t)(1022 + k) << 20)), (int)(uint32_t)S);
+    return ok;
+}
+
+// a / b from an estimate q within a few last places.
+FDF_DEV bool w_div53(double a, double b, double q, double& r)
+{
+    const uint32_t ah = (uint32_t)__double2hiint(a), bh = (uint32_t)__double2hiint(b), qh = (uint32_t)__double2hiint(q);
+    const int ea = (int)((ah >> 20) & 0x7FFu), eb = (int)((bh >> 20) & 0x7FFu), eq = (int)((qh >> 20) & 0x7FFu);
+    const uint64_t A = ((uint64_t)((ah & 0xFFFFFu) | 0x100000u) << 32) | (uint32_t)__double2loint(a);
+    const uint32_t Bh = (bh & 0xFFFFFu) | 0x100000u, Bl = (uint32_t)__double2loint(b);
+    const uint64_t B = ((uint64_t)Bh << 32) | Bl;
+    const uint32_t Qh = (qh & 0xFFFFFu) | 0x100000u, Ql = (uint32_t)__double2loint(q);
+    // the remainder A 2^s - Q B, s = 52 or 53
+    const int sft = ea - eb - eq + 1075;
+    bool ok = (unsigned)(ea - 1) < 0x7FEu && (unsigned)(eb - 1) < 0x7FEu && (unsigned)(eq - 1) < 0x7FEu &&
+              (sft == 52 || sft == 53) && (int)(ah ^ bh ^ qh) >= 0;
+    int64_t rem = (int64_t)((A << (sft & 63)) - ((uint64_t)Ql * Bl + ((uint64_t)(Qh * Bl + Ql * Bh) << 32)));
+    // n = rem / B, B = f 2^52
+    const float f = __uint_as_float(0x3F800000u | ((Bh & 0xFFFFFu) << 3) | (Bl >> 29));
+    const int n = __float2int_rn(__fmul_rn(__fmul_rn(__int2float_rn((int)(rem >> 32)), 9.5367431640625e-7f), w_rcp(f)));
+    rem -= (int64_t)n * (int64_t)B;
+    const uint64_t bits = (((uint64_t)qh << 32) | Ql) + (uint64_t)(int64_t)n;
+    ok = ok && 2 * rem <= (int64_t)B && 2 * rem >= -(int64_t)B && (((uint32_t)(bits >> 32) ^ qh) >> 20) == 0u &&
+         (((uint32_t)(bits >> 32) << 12) | (uint32_t)bits) != 0u;
+    r = __hiloint2double((int)(uint32_t)(bits >> 32), (int)(uint32_t)bits);
+    return ok;
+}
+
+// The nearest float of a double in the FP32 normal range, ties to even (magnitudes below it
+// become zero, as d2f_bits takes them).
+FDF_DEV float w_d2f(double d)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    const uint32_t mag = hi & 0x7FFFFFFFu;
+    uint32_t f = ((mag - 0x38000000u) << 3) | (lo >> 29);
+    f += (lo & 0x1FFFFFFFu) > 0x10000000u - (f & 1u);
+    return __uint_as_float((hi & 0x80000000u) | (mag < 0x38100000u ? 0u : f));
 }
 
 // ---- pairs of floats (value = hi + lo, 48 bits) -----------------------------------------

@@ -29,6 +29,7 @@ static inline float __fmul_rn(float a, float b) { return a * b; }
 static inline float __fmaf_rn(float a, float b, float c) { return std::fma(a, b, c); }
 template <class T, class S> static inline T bits(S s) { T t; std::memcpy(&t, &s, sizeof(t)); return t; }
 static inline uint32_t __float_as_uint(float f) { return bits<uint32_t>(f); }
+static inline float __uint_as_float(uint32_t u) { return bits<float>(u); }
 static inline int __double2hiint(double d) { return (int)(bits<uint64_t>(d) >> 32); }
 static inline int __double2loint(double d) { return (int)bits<uint64_t>(d); }
 static inline double __hiloint2double(int h, int l) { return bits<double>(((uint64_t)(uint32_t)h << 32) | (uint32_t)l); }
@@ -38,6 +39,7 @@ static inline float __int2float_rn(int i) { return (float)i; }
 static inline float __uint2float_rn(uint32_t i) { return (float)i; }
 static inline int __float2int_rn(float f) { return (int)std::nearbyint(f); }
 static inline float w_rsqrt(float f) { return (float)(1.0 / std::sqrt((double)f) * (1.0 + g_skew)); }
+static inline float w_rcp(float f) { return (float)(1.0 / f * (1.0 + g_skew)); }
 #include "wide_math.cuh"
 #include "wide_poly.cuh"
 using namespace fdf;
@@ -76,6 +78,28 @@ extern "C" void check_add(int n, const double* q, const float* d, long* counts)
         const double x = std::fabs(d[i]) < 1.1754943508222875e-38f ? 0.0 : (double)d[i];
         if (!w_add(q[i], d[i], r)) ++counts[0];
         else if (bits<uint64_t>(r) != bits<uint64_t>(q[i] + x)) ++counts[1];
+    }
+}
+extern "C" void check_sqrt(int n, const double* v, long* counts)
+{
+    for (int i = 0; i < n; ++i) {
+        skew(i);
+        double r;
+        if (!w_sqrt53(v[i], w_rsqrt(d2f(v[i])), r)) ++counts[0];
+        else if (r != std::sqrt(v[i])) ++counts[1];
+        const float f = w_d2f(v[i]);
+        if (v[i] > 1.2e-38 && v[i] < 3.4e38 && f != (float)v[i]) ++counts[1];
+    }
+}
+// estimates off by up to `off` last places
+extern "C" void check_div(int n, const double* a, const double* b, int off, long* counts)
+{
+    for (int i = 0; i < n; ++i) {
+        const double q = a[i] / b[i];
+        double r;
+        const double est = bits<double>(bits<uint64_t>(q) + (uint64_t)(int64_t)(i % (2 * off + 1) - off));
+        if (!w_div53(a[i], b[i], est, r)) ++counts[0];
+        else if (r != q) ++counts[1];
     }
 }
 extern "C" void check_square(int n, const long* R, long* counts)
@@ -158,6 +182,39 @@ def test_rsqrt_bits(lib, lo, hi):
     assert counts[1] == 0
     if hi - lo > 1e-3:
         assert counts[0] <= 4 * 33 / 65536 * n
+
+
+@pytest.mark.parametrize("lo,hi", [(1.0, 4.0), (1.0, 1.0 + 2e-6), (4.0 - 4e-6, 4.0), (1e-30, 1e30)])
+def test_sqrt_bits(lib, lo, hi):
+    rng = np.random.default_rng(13)
+    n = 1000000
+    v = np.exp(rng.uniform(math.log(lo), math.log(hi), n)) if hi > 8 else rng.uniform(lo, hi, n)
+    v[::3] = (v[::3] * 2.0 ** 20).round() * 2.0 ** -20          # short, and squares among them
+    v[1::3] = np.sqrt(v[1::3]).astype(np.float32).astype(np.float64) ** 2
+    v = np.concatenate([v, [0.0, -1.0, 5e-324, np.inf, np.nan, 1e300, 1e-300]])
+    counts = np.zeros(2, np.int64)
+    lib.check_sqrt(len(v), _ptr(v), _ptr(counts))
+    assert counts[1] == 0
+    if hi - lo > 1e-3:
+        # refused: zeros, estimates outside [1/2, 1), mantissas within 2^-20 of a power of 4
+        v = np.ascontiguousarray(v[v > 0])
+        counts[:] = 0
+        lib.check_sqrt(len(v), _ptr(v), _ptr(counts))
+        assert counts[0] <= 2e-3 * n
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-4, 1e30])
+def test_div_bits(lib, scale):
+    rng = np.random.default_rng(17)
+    n = 1000000
+    a = scale * rng.normal(size=n)
+    b = rng.uniform(1e-3, 2.0, n)
+    a[::5] = (b[::5] * rng.integers(1, 100, len(b[::5])))         # exact and nearly exact quotients
+    a[-3:] = 0.0, np.inf, np.nan
+    counts = np.zeros(2, np.int64)
+    lib.check_div(n, _ptr(a), _ptr(b), 3, _ptr(counts))
+    assert counts[1] == 0
+    assert counts[0] <= 2e-3 * n + len(a[::5]) / 10               # powers of two among the exact ones
 
 
 def test_square_bits(lib):
