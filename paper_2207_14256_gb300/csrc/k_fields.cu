@@ -91,10 +91,48 @@ __host__ __device__ constexpr int bitrev(int i, int R)
 }
 __host__ __device__ constexpr int ilog2c(int R) { return R <= 1 ? 0 : 1 + ilog2c(R / 2); }
 
-// In-place inverse DFT of R <= 32 values in registers, X_k = sum_n v_n e^{+2 pi i n k / R}:
-// iterative radix-2 Cooley-Tukey on a bit-reversed copy.
+// One butterfly, (u, t) -> (u + w t, u - w t), w = e^{2 pi i k / len}.  In FP64, whose pipe the
+// FP64 transforms are bound by, a general w takes six fused multiply-adds (u + w t, then
+// 2 u - (u + w t)) instead of a product and two sums, eight; in FP32, bound by memory, the
+// product form.  With the twiddles between the levels taken the same way (line_part), the
+// FP64 passes of 128^3 take 405, 290 and 302 us (z, y, x) against 460, 344 and 358.
+template <int k, int len, typename V>
+__device__ __forceinline__ void butterfly(V& a, V& b)
+{
+    const V u = a;
+    V t = b;
+    if constexpr (k != 0 && 4 * k != len && sizeof(V) == 16) {
+        const V w = tw32<V>(k * (32 / len));
+        a = mk<V>(fma(-w.y, t.y, fma(w.x, t.x, u.x)), fma(w.y, t.x, fma(w.x, t.y, u.y)));
+        b = mk<V>(fma(2.0, u.x, -a.x), fma(2.0, u.y, -a.y));
+    } else {
+        if constexpr (k != 0) {
+            if constexpr (4 * k == len) t = cmuli(t);
+            else t = cmul(t, tw32<V>(k * (32 / len)));
+        }
+        a = cadd(u, t);
+        b = csub(u, t);
+    }
+}
+
+// The stages of dft_reg from butterflies of length 2 << S0 on, on bit-reversed values.
+template <int R, int S0, typename V>
+__device__ __forceinline__ void dft_stages(V* v)
+{
+    sfor<ilog2c(R) - S0>([&](auto S) {
+        constexpr int len = 2 << (S + S0);
+        sfor<R / len>([&](auto B) {
+            constexpr int i = B * len;
+            sfor<len / 2>([&](auto K) {
+                constexpr int k = K;
+                butterfly<k, len>(v[i + k], v[i + k + len / 2]);
+            });
+        });
+    });
+}
+
 template <int R, typename V>
-__device__ __forceinline__ void dft_reg(V* v)
+__device__ __forceinline__ void bit_reverse(V* v)
 {
     sfor<R>([&](auto I) {
         constexpr int i = I, j = bitrev(I, R);
@@ -104,23 +142,15 @@ __device__ __forceinline__ void dft_reg(V* v)
             v[j] = t;
         }
     });
-    sfor<ilog2c(R)>([&](auto S) {
-        constexpr int len = 2 << S;
-        sfor<R / len>([&](auto B) {
-            constexpr int i = B * len;
-            sfor<len / 2>([&](auto K) {
-                constexpr int k = K;
-                const V u = v[i + k];
-                V t = v[i + k + len / 2];
-                if constexpr (k != 0) {
-                    if constexpr (4 * k == len) t = cmuli(t);
-                    else t = cmul(t, tw32<V>(k * (32 / len)));
-                }
-                v[i + k] = cadd(u, t);
-                v[i + k + len / 2] = csub(u, t);
-            });
-        });
-    });
+}
+
+// In-place inverse DFT of R <= 32 values in registers, X_k = sum_n v_n e^{+2 pi i n k / R}:
+// iterative radix-2 Cooley-Tukey on a bit-reversed copy.
+template <int R, typename V>
+__device__ __forceinline__ void dft_reg(V* v)
+{
+    bit_reverse<R>(v);
+    dft_stages<R, 0>(v);
 }
 
 // ---- the line transform: N = N1 N2, two levels ----------------------------------
@@ -197,20 +227,48 @@ __device__ __forceinline__ void line_first(V* v, int n2, const V* __restrict__ s
 {
     constexpr int N1 = Shape<N>::N1;
     dft_reg<N1>(v);
-    const V* row = s_tw + n2 * (N1 + 1);
-    sfor<N1>([&](auto K1) { tr[n2 * (N1 + 1) + K1] = cmul(v[K1], row[K1]); });
+    if constexpr (sizeof(V) == 16) {
+        // the twiddles go into the second level's first butterflies (line_part)
+        sfor<N1>([&](auto K1) { tr[n2 * (N1 + 1) + K1] = v[K1]; });
+    } else {
+        const V* row = s_tw + n2 * (N1 + 1);
+        sfor<N1>([&](auto K1) { tr[n2 * (N1 + 1) + K1] = cmul(v[K1], row[K1]); });
+    }
+}
+
+// The second level of one k1: u[k2] = X[k1 + N1 k2].
+template <typename V, int N>
+__device__ __forceinline__ void line_part(int k1, const V* tr, const V* __restrict__ s_tw, V* u)
+{
+    constexpr int N1 = Shape<N>::N1, N2 = Shape<N>::N2;
+    sfor<N2>([&](auto N2i) { u[N2i] = tr[N2i * (N1 + 1) + k1]; });
+    if constexpr (sizeof(V) == 16) {
+        // a w_a +- b w_b: ten fused multiply-adds (six for n2 = 0, where w_a = 1) instead of two
+        // products and two sums, twelve
+        sfor<N2 / 2>([&](auto J) {
+            constexpr int j = J, h = J + N2 / 2;
+            const V wb = s_tw[h * (N1 + 1) + k1], b = u[h];
+            V a = u[j];
+            if constexpr (j != 0) a = cmul(a, s_tw[j * (N1 + 1) + k1]);
+            u[j] = mk<V>(fma(-wb.y, b.y, fma(wb.x, b.x, a.x)), fma(wb.y, b.x, fma(wb.x, b.y, a.y)));
+            u[h] = mk<V>(fma(2.0, a.x, -u[j].x), fma(2.0, a.y, -u[j].y));
+        });
+        bit_reverse<N2>(u);
+        dft_stages<N2, 1>(u);
+    } else {
+        dft_reg<N2>(u);
+    }
 }
 
 // Second level for k1 = t + g N2; out(k2, value) receives X[k1 + N1 k2].
 template <typename V, int N, typename Out>
-__device__ __forceinline__ void line_second(int t, const V* tr, Out&& out)
+__device__ __forceinline__ void line_second(int t, const V* tr, const V* __restrict__ s_tw, Out&& out)
 {
     constexpr int N1 = Shape<N>::N1, N2 = Shape<N>::N2, G = Shape<N>::G;
     sfor<G>([&](auto Gi) {
         const int k1 = t + Gi * N2;
         V u[N2];
-        sfor<N2>([&](auto N2i) { u[N2i] = tr[N2i * (N1 + 1) + k1]; });
-        dft_reg<N2>(u);
+        line_part<V, N>(k1, tr, s_tw, u);
         sfor<N2>([&](auto K2) { out(k1 + N1 * K2, u[K2]); });
     });
 }
@@ -287,6 +345,7 @@ __device__ __forceinline__ V packed(int p, V R, typename Real<V>::T Apsi, typena
                                     typename Real<V>::T kz)
 {
     const V iR = cmuli(R);
+    if (sizeof(V) == 16 && p == 5) return mk<V>(Adot * R.x, Adot * R.y);     // (a product with 0 costs an FP64 slot)
     switch (p) {
         case 0: return mk<V>(Apsi * (kx * iR.x - ky * R.x), Apsi * (kx * iR.y - ky * R.y));
         case 1: return mk<V>(kz * Apsi * iR.x - kx * Aphi * R.x, kz * Apsi * iR.y - kx * Aphi * R.y);
@@ -463,7 +522,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, sizeof(V) == 8 ? 4 : 2) k
                 const T apsi = (P == 2 || Q == 5) ? T(0) : As[0 * N1 * NT + o];
                 const T aphi = (P == 1 || P == 2 || Q == 4) ? As[1 * N1 * NT + o] : T(0);
                 const T adot = (P == 3) ? As[2 * N1 * NT + o] : T(0);
-                v[I] = packed<V>(P, Rv[I], Q == 4 ? apsi + aphi : apsi, aphi, adot, kx, ky, kz);
+                v[I] = packed<V>(Q == 5 ? 5 : P, Rv[I], Q == 4 ? apsi + aphi : apsi, aphi, adot, kx, ky, kz);
             });
         };
         switch (p) {
@@ -480,7 +539,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, sizeof(V) == 8 ? 4 : 2) k
         line_first<V, N>(v, t, s_tw, tr + xo * TSZ);
         __syncthreads();
         V* dst = W0 + p * N3 + (size_t)jy * N + x0 + xo;
-        line_second<V, N>(t, tr + xo * TSZ, [&](int z, V val) { dst[(size_t)z * NN] = val; });
+        line_second<V, N>(t, tr + xo * TSZ, s_tw, [&](int z, V val) { dst[(size_t)z * NN] = val; });
         __syncthreads();
     }
 }
@@ -507,7 +566,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS) k_fields_y(const V* __restr
     __syncthreads();
     line_first<V, N>(v, t, s_tw, tr + xo * TS);
     __syncthreads();
-    line_second<V, N>(t, tr + xo * TS, [&](int y, V val) { dst[(size_t)y * N] = val; });
+    line_second<V, N>(t, tr + xo * TS, s_tw, [&](int y, V val) { dst[(size_t)y * N] = val; });
 }
 
 // ---- pass x: inverse DFT along x, interleave into G[cell][8] ----------------
@@ -577,8 +636,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_X) k_fields_x(const V* __res
     V r[N1];
     sfor<S::G>([&](auto Gi) {
         V u[N2];
-        sfor<N2>([&](auto N2i) { u[N2i] = tr[lp * S::TSX + N2i * (N1 + 1) + t + Gi * N2]; });
-        dft_reg<N2>(u);
+        line_part<V, N>(t + Gi * N2, tr + lp * S::TSX, s_tw, u);
         sfor<N2>([&](auto K2) { r[Gi * N2 + K2] = u[K2]; });
     });
     __syncthreads();
@@ -615,7 +673,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS) k_fields_x_planar(const V* 
     __syncthreads();
     line_first<V, N>(v, t, s_tw, tr + lo * S::TSX);
     __syncthreads();
-    line_second<V, N>(t, tr + lo * S::TSX, [&](int x, V val) {
+    line_second<V, N>(t, tr + lo * S::TSX, s_tw, [&](int x, V val) {
         double re = val.x, im = val.y;
         if constexpr (sizeof(Gt) == 2) {
             re = (double)__bfloat162float(__float2bfloat16_rn(val.x));

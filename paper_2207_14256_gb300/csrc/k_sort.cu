@@ -193,26 +193,29 @@ template <int F> struct RecOf { using T = SplitRec; };
 template <> struct RecOf<kPlain> { using T = PlainRec; };
 template <> struct RecOf<kWide> { using T = WideRec; };
 
-// A wide record moves as three 32-byte vector accesses (records are 32-byte aligned).
-__device__ __forceinline__ void store_wide(void* recs, int64_t j, const WideRec& r)
+// Wide and plain records move as three and four 32-byte vector accesses (records are 32-byte
+// aligned; a plain record copied as a struct moved in 16-byte pieces).
+template <typename Rec>
+__device__ __forceinline__ void store_words(void* recs, int64_t j, const Rec& r)
 {
     const uint32_t* w = reinterpret_cast<const uint32_t*>(&r);
-    uint32_t* p = reinterpret_cast<uint32_t*>(recs) + 24 * j;
+    uint32_t* p = reinterpret_cast<uint32_t*>(recs) + sizeof(Rec) / 4 * j;
 #pragma unroll
-    for (int h = 0; h < 3; ++h)
+    for (int h = 0; h < (int)sizeof(Rec) / 32; ++h)
         asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p + 8 * h), "r"(w[8 * h]),
                      "r"(w[8 * h + 1]), "r"(w[8 * h + 2]), "r"(w[8 * h + 3]), "r"(w[8 * h + 4]), "r"(w[8 * h + 5]),
                      "r"(w[8 * h + 6]), "r"(w[8 * h + 7])
                      : "memory");
 }
 
-__device__ __forceinline__ WideRec load_wide(const void* recs, int64_t j)
+template <typename Rec>
+__device__ __forceinline__ Rec load_words(const void* recs, int64_t j)
 {
-    WideRec r;
+    Rec r;
     uint32_t* w = reinterpret_cast<uint32_t*>(&r);
-    const uint32_t* p = reinterpret_cast<const uint32_t*>(recs) + 24 * j;
+    const uint32_t* p = reinterpret_cast<const uint32_t*>(recs) + sizeof(Rec) / 4 * j;
 #pragma unroll
-    for (int h = 0; h < 3; ++h)
+    for (int h = 0; h < (int)sizeof(Rec) / 32; ++h)
         asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                      : "=r"(w[8 * h]), "=r"(w[8 * h + 1]), "=r"(w[8 * h + 2]), "=r"(w[8 * h + 3]), "=r"(w[8 * h + 4]),
                        "=r"(w[8 * h + 5]), "=r"(w[8 * h + 6]), "=r"(w[8 * h + 7])
@@ -354,9 +357,8 @@ __global__ void __launch_bounds__(kThreads) k_sort_pack(ParticleState a, int64_t
             if (!live[u]) continue;
             const uint32_t b = __shfl_sync(peers[u], base[u], leader[u]);
             const int64_t j = (int64_t)b + __popc(peers[u] & ((1u << lane) - 1u));
-            if constexpr (F == kPlain) reinterpret_cast<Rec*>(recs)[j] = r[u];
-            else if constexpr (F == kWide) store_wide(recs, j, r[u]);
-            else store_split(recs, j, r[u]);
+            if constexpr (F == kFixed) store_split(recs, j, r[u]);
+            else store_words(recs, j, r[u]);
         }
     }
 }
@@ -367,7 +369,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_unpack(ParticleState b, int64
 {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
         if constexpr (F == kWide) {
-            const WideRec r = load_wide(recs, j);
+            const WideRec r = load_words<WideRec>(recs, j);
             for (int d = 0; d < 3; ++d) {
                 b.xd[d * n + j] = r.x[d];
                 b.qd[d * n + j] = r.q[d];
@@ -376,7 +378,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_unpack(ParticleState b, int64
             b.pmag[j] = r.pmag;
             b.id[j] = r.id;
         } else if constexpr (F == kPlain) {
-            const PlainRec r = reinterpret_cast<const PlainRec*>(recs)[j];
+            const PlainRec r = load_words<PlainRec>(recs, j);
             for (int d = 0; d < 3; ++d) {
                 b.xd[d * n + j] = r.x[d];
                 b.qd[d * n + j] = r.q[d];
@@ -426,9 +428,8 @@ __global__ void __launch_bounds__(kThreads) k_export_pack(ParticleState a, int64
         const int64_t o = (int64_t)a.id[i] - begin;
         Rec r;
         make_rec<F>(a, n, i, r);
-        if constexpr (F == kPlain) reinterpret_cast<Rec*>(recs)[o] = r;
-        else if constexpr (F == kWide) store_wide(recs, o, r);
-        else store_split(recs, o, r);
+        if constexpr (F == kFixed) store_split(recs, o, r);
+        else store_words(recs, o, r);
     }
 }
 
@@ -442,14 +443,14 @@ __global__ void __launch_bounds__(kThreads) k_export_unpack(const void* __restri
          o += (int64_t)gridDim.x * blockDim.x) {
         double x[3], q[3], pm;
         if constexpr (F == kWide) {
-            const WideRec r = load_wide(recs, o);
+            const WideRec r = load_words<WideRec>(recs, o);
             for (int d = 0; d < 3; ++d) {
                 x[d] = r.x[d];
                 q[d] = r.q[d];
             }
             pm = r.pmag;
         } else if constexpr (F == kPlain) {
-            const PlainRec r = reinterpret_cast<const PlainRec*>(recs)[o];
+            const PlainRec r = load_words<PlainRec>(recs, o);
             for (int d = 0; d < 3; ++d) {
                 x[d] = r.x[d];
                 q[d] = r.q[d];
