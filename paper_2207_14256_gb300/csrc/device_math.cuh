@@ -167,7 +167,7 @@ __device__ __forceinline__ void fixed_cell(uint32_t X, uint32_t N, uint32_t& i0,
 // FP64 fallbacks of the integer forms, as calls: inlined, the compiler would run their
 // FP64 instructions for every argument and select afterwards.
 static __device__ __noinline__ double rsqrt_slow(double u) { return rsqrt_fp64(u); }
-static __device__ __noinline__ double square_slow(double r) { return r * r; }
+static __device__ __noinline__ double mul_slow(double a, double b) { return a * b; }
 static __device__ __noinline__ double add_slow(double q, float d) { return q + f2d_bits(d); }
 static __device__ __noinline__ double sqrt_slow(double u) { return __dsqrt_rn(u); }
 static __device__ __noinline__ double div_slow(double a, double b) { return __ddiv_rn(a, b); }

@@ -832,21 +832,6 @@ __device__ __forceinline__ double rsqrt_int(double u)
     return r;
 }
 
-// The same with t = r * r.
-__device__ __forceinline__ double rsqrt_int(double u, double& t)
-{
-    double r;
-    int64_t R;
-    int k;
-    const bool ok = w_rsqrt53(u, rsqrtf(d2f_bits(u)), r, R, k);
-    t = w_square53(R, k);
-    if (!ok) {
-        r = rsqrt_slow(u);
-        t = square_slow(r);
-    }
-    return r;
-}
-
 // q += d, one branch for the few sums that w_add leaves to FP64.
 __device__ __forceinline__ void add_small(double q[3], const float d[3])
 {
@@ -872,10 +857,22 @@ __device__ __forceinline__ double drift_integral(const SubStep& st, int s, int n
         // v = 1 + |q|^2 / (m^2 a_c^2), t = 1/v, D = v^(-1/2) gm(t) / (m a_c); a massless
         // species takes D = |q|^-1 sum_j W_j
         const bool massless = st.wide.massless[s];
-        double t;
-        const double r = rsqrt_int(massless ? qq : fma(qq, st.wide.inv_muc[s], 1.0), t);
-        const double g = wide_poly<kWideD64>(st.wide.drift[s], t, d2f_bits(t));
-        return r * (massless ? st.wide.wsum[s] : g);
+        const double v = massless ? qq : fma(qq, st.wide.inv_muc[s], 1.0);
+        // r = v^(-1/2), t = r r and D = r g in integers; all three in FP64 for the few v (or g)
+        // that they leave to it
+        double r, D;
+        int64_t R;
+        int k;
+        const bool ok = w_rsqrt53(v, rsqrtf(d2f_bits(v)), r, R, k);
+        double t = w_square53(R, k);
+        if (!ok) {
+            r = rsqrt_slow(v);
+            t = mul_slow(r, r);
+        }
+        double g = wide_poly<kWideD64>(st.wide.drift[s], t, d2f_bits(t));
+        if (massless) g = st.wide.wsum[s];
+        if (!(w_mul53(R, k, g, D) && ok)) D = mul_slow(r, g);
+        return D;
     } else {
         const SpeciesCoef& sc = st.sp[s];
         double D = 0.0;

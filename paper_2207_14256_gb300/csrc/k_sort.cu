@@ -414,22 +414,37 @@ __global__ void __launch_bounds__(kThreads) k_sort_unpack(ParticleState b, int64
 // ---- export in id order through the record buffer -------------------------------
 // A sorted state holds particle i's outputs at slot id[i] - begin of the caller's
 // arrays.  Writing them there directly scatters seven 8-byte values per particle;
-// instead each particle's record goes whole to that slot (one scattered 64-byte
-// write), and a streaming pass turns the records into positions, momenta and
-// weights.
+// instead a record goes whole to that slot (one scattered 64-byte write), and a streaming
+// pass turns the records into positions, momenta and weights.  The record holds what the
+// outputs need and no more: DRAM's random writes bound the pack (8e6 particles with the
+// 96-byte records of the sort: 446 us, and 178 us for the streaming pass).
+struct alignas(64) ExportRec {
+    double x[3], q[3], pmag, pad;
+};
+
 template <int F>
 __global__ void __launch_bounds__(kThreads) k_export_pack(ParticleState a, int64_t n, int64_t begin, int64_t count,
                                                           void* __restrict__ recs)
 {
-    using Rec = typename RecOf<F>::T;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < count;
          j += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = begin + j;
         const int64_t o = (int64_t)a.id[i] - begin;
-        Rec r;
-        make_rec<F>(a, n, i, r);
-        if constexpr (F == kFixed) store_split(recs, o, r);
-        else store_words(recs, o, r);
+        if constexpr (F == kFixed) {
+            SplitRec r;
+            make_rec<F>(a, n, i, r);
+            store_split(recs, o, r);
+        } else {
+            ExportRec r;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                r.x[d] = a.xd[d * n + i];
+                r.q[d] = a.qd[d * n + i];
+            }
+            r.pmag = a.pmag[i];
+            r.pad = 0.0;
+            store_words(recs, o, r);
+        }
     }
 }
 
@@ -442,15 +457,8 @@ __global__ void __launch_bounds__(kThreads) k_export_unpack(const void* __restri
     for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < count;
          o += (int64_t)gridDim.x * blockDim.x) {
         double x[3], q[3], pm;
-        if constexpr (F == kWide) {
-            const WideRec r = load_words<WideRec>(recs, o);
-            for (int d = 0; d < 3; ++d) {
-                x[d] = r.x[d];
-                q[d] = r.q[d];
-            }
-            pm = r.pmag;
-        } else if constexpr (F == kPlain) {
-            const PlainRec r = load_words<PlainRec>(recs, o);
+        if constexpr (F != kFixed) {
+            const ExportRec r = load_words<ExportRec>(recs, o);
             for (int d = 0; d < 3; ++d) {
                 x[d] = r.x[d];
                 q[d] = r.q[d];

@@ -94,6 +94,30 @@ FDF_DEV double w_square53(int64_t R, int k)
     return __hiloint2double((int)((uint32_t)(q >> 32) + ((1020u + big - 2u * (uint32_t)k) << 20)), (int)(uint32_t)q);
 }
 
+// The bits of r * g for r as above, rounded to nearest, ties to even, from the 106-bit product;
+// false unless g and the product are finite normal numbers.
+FDF_DEV bool w_mul53(int64_t R, int k, double g, double& x)
+{
+    const uint32_t Rh = (uint32_t)((uint64_t)R >> 32), Rl = (uint32_t)R;
+    const uint32_t gh = (uint32_t)__double2hiint(g), Gl = (uint32_t)__double2loint(g);
+    const uint32_t Gh = (gh & 0xFFFFFu) | 0x100000u;
+    const int eg = (int)((gh >> 20) & 0x7FFu);
+    const uint64_t ll = (uint64_t)Rl * Gl;
+    const uint64_t m1 = (uint64_t)Rh * Gl + (ll >> 32);
+    const uint64_t m2 = (uint64_t)Rl * Gh + (uint32_t)m1;
+    const uint64_t top = (uint64_t)Rh * Gh + (m1 >> 32) + (m2 >> 32);
+    const uint32_t m = (uint32_t)m2, th = (uint32_t)(top >> 32), tl = (uint32_t)top;
+    const uint32_t big = th >> 9;                               // the product of significands >= 2^105
+    const uint32_t sh = 12u - big;
+    const uint32_t ql = __funnelshift_l(m, tl, sh), rem = m << sh;
+    const uint32_t sticky = ((uint32_t)ll != 0u) | (ql & 1u);
+    const uint64_t q = (((uint64_t)__funnelshift_l(tl, th, sh) << 32) | ql) + (rem > 0x80000000u - sticky);
+    // r's exponent is -1 - k, so the product's is eg - 1 - k, or one less
+    const int e = eg - 2 + (int)big - k;
+    x = __hiloint2double((int)(((uint32_t)(q >> 32) + ((uint32_t)e << 20)) | (gh & 0x80000000u)), (int)(uint32_t)q);
+    return (unsigned)(eg - 1) < 0x7FEu && e >= 0 && e < 0x7FD;
+}
+
 // The bits of q + (double)d in integers (a subnormal d counts as zero, as f2d_bits takes it):
 // d's 24-bit significand in units of q's last place, rounded to nearest, ties to even, is
 // added to q's bit pattern.  False where that may not be the sum's pattern: the sum leaves q's

@@ -80,6 +80,15 @@ extern "C" void check_add(int n, const double* q, const float* d, long* counts)
         else if (bits<uint64_t>(r) != bits<uint64_t>(q[i] + x)) ++counts[1];
     }
 }
+extern "C" void check_mul(int n, const long* R, const int* k, const double* g, long* counts)
+{
+    for (int i = 0; i < n; ++i) {
+        double x;
+        const double r = std::ldexp((double)R[i], -53 - k[i]);
+        if (!w_mul53(R[i], k[i], g[i], x)) ++counts[0];
+        else if (bits<uint64_t>(x) != bits<uint64_t>(r * g[i])) ++counts[1];
+    }
+}
 extern "C" void check_sqrt(int n, const double* v, long* counts)
 {
     for (int i = 0; i < n; ++i) {
@@ -226,6 +235,24 @@ def test_square_bits(lib):
                         2 ** 53 - 1 - np.arange(999), root2 + np.arange(-999, 999)])
     counts = np.zeros(2, np.int64)
     lib.check_square(len(R), _ptr(R), _ptr(counts))
+    assert counts[1] == 0
+
+
+def test_mul_bits(lib):
+    rng = np.random.default_rng(19)
+    n = 1000000
+    R = rng.integers(2 ** 52, 2 ** 53, n)
+    R[::5] = (R[::5] >> 30) << 30                    # short significands: ties and exact products
+    k = rng.integers(-60, 60, n).astype(np.int32)
+    g = rng.normal(size=n) * np.exp2(rng.integers(-40, 40, n))
+    g[::7] = np.float32(g[::7])
+    g[::11] = np.exp2(rng.integers(-40, 40, len(g[::11])))
+    counts = np.zeros(2, np.int64)
+    lib.check_mul(n, _ptr(R), _ptr(k), _ptr(g), _ptr(counts))
+    assert counts[1] == 0 and counts[0] == 0
+    g = np.tile(np.array([0.0, -0.0, np.inf, np.nan, 5e-324, 1e-300, 1e300, -1e308]), 100)
+    R, k = R[:len(g)].copy(), rng.integers(-60, 60, len(g)).astype(np.int32)
+    lib.check_mul(len(g), _ptr(R), _ptr(k), _ptr(g), _ptr(counts))
     assert counts[1] == 0
 
 
