@@ -279,8 +279,8 @@ Layout make_layout(const fdf_params& p, int nk, int na, int ncdf)
         return o;
     };
     L.tabs = take(3 * (size_t)na * nk * 8);
-    // an amplitude table per grid of a pass (its steps and the opening half kick)
-    L.modeA = take((steps_per_pass(p) + 1) * 4 * (size_t)mode_table_size(p.n_grid) * real_bytes(prec));
+    // amplitude tables of kMaxSub steps (a pass of 8 steps and its opening half kick)
+    L.modeA = take(kMaxSub * 4 * (size_t)mode_table_size(p.n_grid) * real_bytes(prec));
     L.keys = take((size_t)mode_table_size(p.n_grid) * sizeof(ModeKey));
     L.noise = take(N3 * complex_bytes(prec));
     L.cdf_t = take((size_t)ncdf * 8);
@@ -1380,12 +1380,20 @@ int slice_prepare(fdf_ctx* c, int j, std::vector<int>& bufs, std::vector<const v
     if (j == 0) ks.push_back(sl.k_start);                       // the opening half kick
     for (int i = 0; i < pass_len(c, j); ++i) ks.push_back(sl.k_start + sl.dir * (pass_first(c, j) + i + 1));
     if (!c->frozen && !c->supersteps && c->noise_ready) {
-        // the amplitude tables of all grids to build, in one launch
+        // the amplitude tables of all grids to build, and as many of the steps after them as
+        // there are slots, in one launch (5 us a launch, which passes of one step on a small
+        // grid would pay for every step)
         double lna[kMaxSub];
-        int count = 0;
+        int count = 0, missing = 0;
+        auto held = [&](double l) { return std::find(c->mode_lna, c->mode_lna + c->mode_count, l) != c->mode_lna + c->mode_count; };
         for (int kk : ks)
-            if (find_grid(c, kk) < 0) lna[count++] = c->lna(kk);
-        int rc = count > 1 ? mode_tables(c, lna, count, c->sf) : FDF_OK;
+            if (find_grid(c, kk) < 0) {
+                lna[count++] = c->lna(kk);
+                missing += !held(lna[count - 1]);
+            }
+        for (int i = pass_first(c, j) + pass_len(c, j) + 1; i <= sl.steps && count < kMaxSub; ++i)
+            lna[count++] = c->lna(sl.k_start + sl.dir * i);
+        int rc = missing ? mode_tables(c, lna, count, c->sf) : FDF_OK;
         if (rc) return rc;
     }
     for (int kk : ks) {
