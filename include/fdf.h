@@ -144,7 +144,10 @@ typedef struct fdf_params {
                                   are held (0 = 4 for the FP32/BF16-grid forms, 1 for the plain
                                   FP64 form) */
     int32_t  sort_tile;        /* sort buckets are cubes of 2^sort_tile cells per axis, 0..3
-                                  (0 = single cells) */
+                                  (0 = single cells), or larger cubes of up to 4^3 cells while a
+                                  bucket would hold only a few particles (fewer than 3 of a
+                                  species on average, or than 32 in the FP64-state forms with
+                                  interp_order 1) */
     int32_t  sort_cells;       /* with sort_every = 0: re-bucket when the typical particle has
                                   moved this many cells since the last sort (0 = 4) */
     int32_t  interp_order;     /* interpolation order r of the force read and the deposit

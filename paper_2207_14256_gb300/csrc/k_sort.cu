@@ -4,7 +4,7 @@
 // computed beforehand in linear theory, Sec. 2.1), so the particle arrays may
 // be permuted freely; results are read back by particle id.  Particles are
 // ordered by key = species * B + Morton(bucket), a bucket being a cube of
-// 2^sort_tile cells per axis (B buckets per species) around the particle's
+// sort_tile_shift's cells (B buckets per species) around the particle's
 // predicted position halfway through the next pass, with a counting sort:
 //   keys:    key of every particle and a histogram of keys;
 //   scan:    exclusive prefix sum of the histogram (recursive, any bin count);
