@@ -794,8 +794,9 @@ int mode_tables(fdf_ctx* c, const double* lna, int count, cudaStream_t s)
 }
 
 // The transforms of the eight fields at ln a up to their y pass, into c->W on stream s;
-// slot 7 as `slot7` says (kSlot7*), `grids` packed grids.
-int build_lines(fdf_ctx* c, double lna, cudaStream_t s, int slot7, int grids)
+// slot 7 as `slot7` says (kSlot7*), `grids` packed grids (FP32).  `a` receives the build's
+// arguments, which the x pass reads too.
+int build_lines(fdf_ctx* c, double lna, cudaStream_t s, int slot7, int grids, FieldArgs& a)
 {
     if (!c->noise_ready) {
         if (s != c->sf) FDF_CUDA(cudaStreamSynchronize(c->stream), "sync");
@@ -810,25 +811,26 @@ int build_lines(fdf_ctx* c, double lna, cudaStream_t s, int slot7, int grids)
         if (rc0) return rc0;
         slot = 0;
     }
-    FieldArgs a = field_args(c, lna);
+    a = field_args(c, lna);
     a.slot7 = slot7;
     a.grids = grids;
-    const int prec = grid_prec(c->p.precision), N = c->p.n_grid;
-    const void* A = c->modeA + (size_t)slot * 4 * mode_table_size(N) * real_bytes(c->p.precision);
+    const int prec = grid_prec(c->p.precision);
+    const void* A = c->modeA + (size_t)slot * 4 * mode_table_size(a.N) * real_bytes(c->p.precision);
     int rc = timed_on(c, s, FDF_K_FIELDS_Z, "fields z pass",
                       [&] { return launch_fields_z(s, prec, a, A, c->noise, c->tw, c->W); });
     if (rc) return rc;
     return timed_on(c, s, FDF_K_FIELDS_Y, "fields y pass",
-                    [&] { return launch_fields_y(s, prec, N, grids, c->tw, c->W); });
+                    [&] { return launch_fields_y(s, prec, a, c->tw, c->W); });
 }
 
 // The eight fields at ln a into G, on stream s.
 int build_fields(fdf_ctx* c, double lna, void* G, cudaStream_t s, int slot7)
 {
-    int rc = build_lines(c, lna, s, slot7, 4);
+    FieldArgs a;
+    int rc = build_lines(c, lna, s, slot7, 4, a);
     if (rc) return rc;
     return timed_on(c, s, FDF_K_FIELDS_X, "fields x pass", [&] {
-        return launch_fields_x(s, grid_prec(c->p.precision), c->p.n_grid, c->tw, c->W, G);
+        return launch_fields_x(s, grid_prec(c->p.precision), a, c->tw, c->W, G);
     });
 }
 
@@ -1850,10 +1852,11 @@ int fdf_build_fields(fdf_ctx* c, double lna, double* out, int32_t out_on_device)
     // as the initial transform reads it, the fifth packed grid
     double* dst = out;
     if (!out_on_device) FDF_CUDA(cudaMalloc(&dst, 8 * N3 * 8), "allocating the field copy");
-    int rc = build_lines(c, lna, c->stream, kSlot7Zero, 5);
+    FieldArgs a;
+    int rc = build_lines(c, lna, c->stream, kSlot7Zero, 5, a);
     if (!rc)
         rc = timed(c, FDF_K_FIELDS_X, "fields x pass", [&] {
-            return launch_fields_x_planar(c->stream, grid_prec(c->p.precision), N, c->tw, c->W, dst);
+            return launch_fields_x_planar(c->stream, grid_prec(c->p.precision), a, c->tw, c->W, dst);
         });
     if (!rc && !out_on_device) {
         cudaError_t e = cudaMemcpyAsync(out, dst, 8 * N3 * 8, cudaMemcpyDeviceToHost, c->stream);

@@ -243,10 +243,11 @@ cudaError_t launch_mode_tables(cudaStream_t s, int precision, const FieldArgs& a
 cudaError_t launch_noise(cudaStream_t s, int precision, const FieldArgs& a, void* R);
 cudaError_t launch_fields_z(cudaStream_t s, int precision, const FieldArgs& a, const void* A, const void* R,
                             const void* tw, void* W0);
-cudaError_t launch_fields_y(cudaStream_t s, int precision, int N, int grids, const void* tw, void* W);
-cudaError_t launch_fields_x(cudaStream_t s, int precision, int N, const void* tw, const void* W, void* G);
+cudaError_t launch_fields_y(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, void* W);
+cudaError_t launch_fields_x(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, const void* W, void* G);
 // The x pass of five packed grids into out[8][N^3], each value as a gather grid holds it.
-cudaError_t launch_fields_x_planar(cudaStream_t s, int precision, int N, const void* tw, const void* W, double* out);
+cudaError_t launch_fields_x_planar(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, const void* W,
+                                   double* out);
 // The amplitude table at one scale factor (from two-row tables or more) and the unit
 // Gaussian field, in one launch.
 cudaError_t launch_modes_once(cudaStream_t s, int precision, const FieldArgs& a, const double* tabs64, void* A, void* R);

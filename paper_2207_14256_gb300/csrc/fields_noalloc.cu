@@ -115,8 +115,8 @@ extern "C" int fdf_build_fields_noalloc(const fdf_params* p, const fdf_tables* t
     // fifth packed grid
     e = launch_modes_once(st, gp, a, (const double*)(s + oT64), s + oA, s + oR);
     if (e == cudaSuccess) e = launch_fields_z(st, gp, a, s + oA, s + oR, s + oTw, s);
-    if (e == cudaSuccess) e = launch_fields_y(st, gp, p->n_grid, 5, s + oTw, s);
-    if (e == cudaSuccess) e = launch_fields_x_planar(st, gp, p->n_grid, s + oTw, s, out);
+    if (e == cudaSuccess) e = launch_fields_y(st, gp, a, s + oTw, s);
+    if (e == cudaSuccess) e = launch_fields_x_planar(st, gp, a, s + oTw, s, out);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess)
         return set_error(FDF_ECUDA, (std::string("fdf_build_fields_noalloc: ") + cudaGetErrorString(e)).c_str());

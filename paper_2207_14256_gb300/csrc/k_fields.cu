@@ -23,6 +23,12 @@
 //   y: transform along y;
 //   x: transform along x and write the interleaved gather grid G[cell][8] as
 //      whole 32-byte records.
+// That is the FP32 form, bound by memory.  The FP64 passes, bound by the FP64 pipe, hold half
+// spectra instead (the columns jx < N/2 of a real field's Hermitian spectrum) and take each
+// axis' gradients at that axis' pass, so that fewer columns are transformed along z and y:
+//   z: psi, d_z psi, phi, d_z phi and phi_dot (five half arrays: 2.5 N^3 of 4 N^3);
+//   y: those, d_y psi and d_y phi (seven: 3.5 N^3);
+//   x: the pairs P0..P3 formed line by line from the half spectra, d_x there.
 #include <cuda_bf16.h>
 
 #include <utility>
@@ -95,7 +101,7 @@ __host__ __device__ constexpr int ilog2c(int R) { return R <= 1 ? 0 : 1 + ilog2c
 // FP64 transforms are bound by, a general w takes six fused multiply-adds (u + w t, then
 // 2 u - (u + w t)) instead of a product and two sums, eight; in FP32, bound by memory, the
 // product form.  With the twiddles between the levels taken the same way (line_part), the
-// FP64 passes of 128^3 take 405, 290 and 302 us (z, y, x) against 460, 344 and 358.
+// packed FP64 passes of 128^3 took 405, 290 and 302 us (z, y, x) against 460, 344 and 358.
 template <int k, int len, typename V>
 __device__ __forceinline__ void butterfly(V& a, V& b)
 {
@@ -208,7 +214,15 @@ template <int N> struct Shape {
     static constexpr int TZ0 = kSplitGrids ? 8 : 128 / T;
     static constexpr int TZ = TZ0 < N ? TZ0 : N;
     static constexpr int THREADS_Z = TZ * T;
+    // the half-spectrum passes' tiles, of rows of N / 2
+    static constexpr int HX = TX0 < N / 2 ? TX0 : N / 2;
+    static constexpr int HZ = TZ0 < N / 2 ? TZ0 : N / 2;
 };
+
+// The half-spectrum work array: arrays of N^2 (N/2) values [z][y][x].  The z pass writes the
+// first five, the y pass transforms 1, 3 and 4 in place and 0 and 2 twice, into the last four.
+enum Half { kHPsi0, kHDzPsi, kHPhi0, kHDzPhi, kHDot, kHPsi, kHDyPsi, kHPhi, kHDyPhi };
+constexpr int kHalfZ = 5, kHalfY = 7;
 
 // Twiddles of the first level, w_N^(n2 k1) at [n2 (N1 + 1) + k1]: a thread reads its
 // own row, and lanes with different n2 fall in different banks.
@@ -281,6 +295,13 @@ __device__ __forceinline__ double f_sqrt(double x) { return sqrt(x); }
 __device__ __forceinline__ void f_sincospi(float x, float* s, float* c) { sincospif(x, s, c); }
 __device__ __forceinline__ void f_sincospi(double x, double* s, double* c) { sincospi(x, s, c); }
 
+// |n| < 2^20 in FP64, in integer operations: the conversion would take a slot of the FP64 pipe.
+__device__ __forceinline__ double small_int(int n)
+{
+    const uint32_t f = __float_as_uint((float)n);
+    return __hiloint2double((int)(n == 0 ? 0u : (f & 0x80000000u) | (((f & 0x7FFFFFFFu) >> 3) + 0x38000000u)), 0);
+}
+
 __device__ __forceinline__ int sidx(int j, int N) { return j < (N >> 1) ? j : j - N; }
 
 // The unit Gaussian of mode (jx, jy, jz), R/sqrt(P_R/V): zero for the mean and the
@@ -345,7 +366,6 @@ __device__ __forceinline__ V packed(int p, V R, typename Real<V>::T Apsi, typena
                                     typename Real<V>::T kz)
 {
     const V iR = cmuli(R);
-    if (sizeof(V) == 16 && p == 5) return mk<V>(Adot * R.x, Adot * R.y);     // (a product with 0 costs an FP64 slot)
     switch (p) {
         case 0: return mk<V>(Apsi * (kx * iR.x - ky * R.x), Apsi * (kx * iR.y - ky * R.y));
         case 1: return mk<V>(kz * Apsi * iR.x - kx * Aphi * R.x, kz * Apsi * iR.y - kx * Aphi * R.y);
@@ -435,8 +455,7 @@ __global__ void __launch_bounds__(256) k_modes_once(FieldArgs a, int M, const do
     if (m < M) mode_values(mode_key(a, m), a.ia, a.fa, a.aH, a.na, a.nk, tabs, A + 4 * (size_t)m);
 }
 
-// One entry of the amplitude table (4 values per |n|^2, 16- or 32-byte aligned) in
-// as few loads as the type allows.
+// One entry of the FP32 amplitude table (4 values per |n|^2) in one load.
 __device__ __forceinline__ void amp_entry(const float* A, int m, float& ap, float& af, float& ad)
 {
     const float4 v = __ldg(reinterpret_cast<const float4*>(A) + m);
@@ -444,20 +463,13 @@ __device__ __forceinline__ void amp_entry(const float* A, int m, float& ap, floa
     af = v.y;
     ad = v.z;
 }
-__device__ __forceinline__ void amp_entry(const double* A, int m, double& ap, double& af, double& ad)
-{
-    const double2 u = __ldg(reinterpret_cast<const double2*>(A) + 2 * m);
-    ap = u.x;
-    af = u.y;
-    ad = __ldg(A + 4 * m + 2);
-}
 
 // ---- pass z: spectrum + inverse DFT along z ---------------------------------
 // Block (x-tile, jy): TX columns along z.  Each thread reads the unit Gaussians of
 // its N1 modes once, with their amplitudes A[|n|^2] at this scale factor, then forms,
 // transforms and writes each of the four packed grids in turn.
 template <typename V, int N>
-__global__ void __launch_bounds__(Shape<N>::THREADS_Z, sizeof(V) == 8 ? 4 : 2) k_fields_z(FieldArgs a,
+__global__ void __launch_bounds__(Shape<N>::THREADS_Z, 4) k_fields_z(FieldArgs a,
                                                                   const typename Real<V>::T* __restrict__ A,
                                                                   const V* __restrict__ R, const V* __restrict__ tw,
                                                                   V* __restrict__ W0)
@@ -522,7 +534,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, sizeof(V) == 8 ? 4 : 2) k
                 const T apsi = (P == 2 || Q == 5) ? T(0) : As[0 * N1 * NT + o];
                 const T aphi = (P == 1 || P == 2 || Q == 4) ? As[1 * N1 * NT + o] : T(0);
                 const T adot = (P == 3) ? As[2 * N1 * NT + o] : T(0);
-                v[I] = packed<V>(Q == 5 ? 5 : P, Rv[I], Q == 4 ? apsi + aphi : apsi, aphi, adot, kx, ky, kz);
+                v[I] = packed<V>(P, Rv[I], Q == 4 ? apsi + aphi : apsi, aphi, adot, kx, ky, kz);
             });
         };
         switch (p) {
@@ -567,6 +579,159 @@ __global__ void __launch_bounds__(Shape<N>::THREADS) k_fields_y(const V* __restr
     line_first<V, N>(v, t, s_tw, tr + xo * TS);
     __syncthreads();
     line_second<V, N>(t, tr + xo * TS, s_tw, [&](int y, V val) { dst[(size_t)y * N] = val; });
+}
+
+// ---- the half-spectrum passes z and y (FP64) ----------------------------------
+// All three FP64 passes are bound by the FP64 pipe (84-85 % busy), so the transforms that half
+// spectra save are time: 128^3, a build 997 -> 857 us (z 405 -> 238, y 290 -> 280, x 302 -> 340,
+// which now forms its lines and d_x); a run of 100 steps 158 -> 145 ms, and 5.16 -> 4.2 ms at 32^3.
+// Block (array f and x tile, jy): HZ columns along z of one of the five arrays, the real
+// fields' spectra A R or i k_z A R.  The array index runs fastest, so that the five blocks
+// that read the same unit Gaussians run together.
+template <int N>
+__global__ void __launch_bounds__(Shape<N>::HZ * Shape<N>::T, Shape<N>::N1 == 32 ? 2 : 4)
+    k_half_z(FieldArgs a, const double* __restrict__ A, const double2* __restrict__ R, const double2* __restrict__ tw,
+             double2* __restrict__ W)
+{
+    using S = Shape<N>;
+    constexpr int TX = S::HZ, N1 = S::N1, N2 = S::N2, NT = TX * S::T;
+    constexpr int TSZ = S::template line_stride<16, TX>();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double2* s_tw = reinterpret_cast<double2*>(smem_raw);
+    double2* tr = s_tw + S::TWS;                            // TX * TSZ
+    double* As = reinterpret_cast<double*>(tr + TX * TSZ);  // [N1][NT]: each thread's own column
+    load_line_twiddles<double2, N>(s_tw, tw);
+    const int xo = threadIdx.x % TX, t = threadIdx.x / TX;
+    const int f = blockIdx.x % kHalfZ, x0 = blockIdx.x / kHalfZ * TX, jy = blockIdx.y;
+    const int nx = x0 + xo, ny = sidx(jy, N), h = -(N >> 1);
+    const bool dz = f == kHDzPsi || f == kHDzPhi;
+    const size_t NN = (size_t)N * N;
+    double2 v[N1];
+    sfor<N1>([&](auto I) { v[I] = R[(size_t)(N2 * I + t) * NN + (size_t)jy * N + nx]; });
+    // The amplitudes, each looked up once for the modes nz and -nz (as in k_fields_z); a z
+    // gradient's factor k_z A changes sign between them.
+    {
+        const double* row = A + (f <= kHDzPsi ? 0 : f <= kHDzPhi ? 1 : 2);
+        const int tp = t == 0 ? 0 : N2 - t;
+        const int partner = xo + TX * tp;
+        sfor<N1 / 2 + 1>([&](auto I) {
+            if (I < N1 / 2 || t == 0) {
+                const int nz = sidx(N2 * I + t, N);
+                const int Ip = t == 0 ? (N1 - I) % N1 : N1 - 1 - I;
+                double ap = 0.0;
+                if (ny != h && nz != h) ap = __ldg(row + 4 * (size_t)(nx * nx + ny * ny + nz * nz));
+                if (dz) ap *= a.kf * small_int(nz);
+                As[I * NT + threadIdx.x] = ap;
+                As[Ip * NT + partner] = dz ? -ap : ap;
+            }
+        });
+    }
+    __syncthreads();
+    sfor<N1>([&](auto I) {
+        const double ap = As[I * NT + threadIdx.x];
+        const double re = ap * v[I].x, im = ap * v[I].y;
+        v[I] = dz ? make_double2(-im, re) : make_double2(re, im);
+    });
+    line_first<double2, N>(v, t, s_tw, tr + xo * TSZ);
+    __syncthreads();
+    double2* dst = W + f * (NN * (N / 2)) + (size_t)jy * (N / 2) + nx;
+    line_second<double2, N>(t, tr + xo * TSZ, s_tw, [&](int z, double2 val) { dst[(size_t)z * (NN / 2)] = val; });
+}
+
+// Block (transform q and x tile, jz): HX lines along y of one of the seven transforms, the y
+// gradients multiplied by i k_y as they are read.
+template <int N>
+__global__ void __launch_bounds__(Shape<N>::HX * Shape<N>::T) k_half_y(double kf, const double2* __restrict__ tw,
+                                                                        double2* W)
+{
+    using S = Shape<N>;
+    constexpr int TX = S::HX, N1 = S::N1, N2 = S::N2;
+    constexpr int TS = S::template line_stride<16, TX>();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double2* s_tw = reinterpret_cast<double2*>(smem_raw);
+    double2* tr = s_tw + S::TWS;
+    load_line_twiddles<double2, N>(s_tw, tw);
+    const int xo = threadIdx.x % TX, t = threadIdx.x / TX;
+    const int q = blockIdx.x % kHalfY, x0 = blockIdx.x / kHalfY * TX, jz = blockIdx.y;
+    // psi, d_y psi, phi, d_y phi (out of place: their sources are read twice), then in place
+    const int src = q < 2 ? kHPsi0 : q < 4 ? kHPhi0 : q == 4 ? kHDzPsi : q == 5 ? kHDzPhi : kHDot;
+    const int to = q < 4 ? kHPsi + q : src;
+    const size_t NH = (size_t)N * (N / 2), N3H = NH * N;
+    const size_t at = (size_t)jz * NH + x0 + xo;
+    double2 v[N1];
+    sfor<N1>([&](auto I) { v[I] = W[src * N3H + at + (size_t)(N2 * I + t) * (N / 2)]; });
+    if (q == 1 || q == 3)
+        sfor<N1>([&](auto I) {
+            const double ky = kf * small_int(sidx(N2 * I + t, N));
+            v[I] = make_double2(-ky * v[I].y, ky * v[I].x);
+        });
+    __syncthreads();
+    line_first<double2, N>(v, t, s_tw, tr + xo * TS);
+    __syncthreads();
+    double2* dst = W + to * N3H + at;
+    line_second<double2, N>(t, tr + xo * TS, s_tw, [&](int y, double2 val) { dst[(size_t)y * (N / 2)] = val; });
+}
+
+// The x spectrum of packed grid p (4: grid 3 as kSlot7Psi has it) along one line, thread t's
+// values, from the half spectra: F(N - k) = conj F(k), F(N/2) = 0.
+//   P0 = i (k_x psi + d_y psi)    P1 = d_z psi - k_x phi    P2 = d_y phi + i d_z phi
+//   P3 = phi_dot + i psi, phi_dot + i (phi + psi) or phi_dot
+template <int N>
+__device__ __forceinline__ void half_line(double2* v, int p, int t, double kf, int slot7, size_t line,
+                                          const double2* __restrict__ W)
+{
+    constexpr int N1 = Shape<N>::N1, N2 = Shape<N>::N2;
+    const size_t N3H = (size_t)N * N * (N / 2);
+    const double2* a = W + line * (N / 2) + N3H * (p == 0 ? kHDyPsi : p == 1 ? kHDzPsi : p == 2 ? kHDyPhi : kHDot);
+    const double2* b = W + line * (N / 2) + N3H * (p == 1 ? kHPhi : p == 2 ? kHDzPhi : kHPsi);
+    auto each = [&](auto&& f) {
+        sfor<N1>([&](auto I) {
+            const int k = N2 * I + t;
+            if constexpr (I < N1 / 2) {
+                v[I] = f(k, [&](const double2* s) { return s[k]; });
+            } else {
+                if (I == N1 / 2 && t == 0) v[I] = make_double2(0.0, 0.0);
+                else
+                    v[I] = f(k - N, [&](const double2* s) {
+                        const double2 u = s[N - k];
+                        return make_double2(u.x, -u.y);
+                    });
+            }
+        });
+    };
+    if (p < 2) {
+        const double kp = p == 0 ? kf : -kf;
+        each([&](int n, auto&& get) {
+            const double2 u = get(a), w = get(b);
+            const double k = kp * small_int(n), x = fma(k, w.x, u.x), y = fma(k, w.y, u.y);
+            return p == 0 ? make_double2(-y, x) : make_double2(x, y);
+        });
+    } else if (p == 3 && slot7 == kSlot7Zero) {
+        each([&](int, auto&& get) { return get(a); });
+    } else if (p == 3 && slot7 == kSlot7Sum) {
+        const double2* c = W + line * (N / 2) + N3H * kHPhi;
+        each([&](int, auto&& get) {
+            const double2 u = get(a), w = get(b), z = get(c);
+            return make_double2(u.x - (w.y + z.y), u.y + (w.x + z.x));
+        });
+    } else {
+        each([&](int, auto&& get) {
+            const double2 u = get(a), w = get(b);
+            return make_double2(u.x - w.y, u.y + w.x);
+        });
+    }
+}
+
+// Thread t's values of a line of packed grid p: read (FP32) or formed (FP64).
+template <typename V, int N>
+__device__ __forceinline__ void x_line(V* v, int p, int t, double kf, int slot7, size_t line, const V* __restrict__ W)
+{
+    if constexpr (sizeof(V) == 16) {
+        half_line<N>(v, p, t, kf, slot7, line, W);
+    } else {
+        const V* src = W + p * ((size_t)N * N * N) + line * N;
+        sfor<Shape<N>::N1>([&](auto I) { v[I] = src[Shape<N>::N2 * I + t]; });
+    }
 }
 
 // ---- pass x: inverse DFT along x, interleave into G[cell][8] ----------------
@@ -614,8 +779,8 @@ template <> struct GRec<__nv_bfloat16, float2> {
 // Bound by DRAM at N = 256 (48 (BF16) or 64 (FP32) bytes per cell): BF16 records 164 ->
 // 120 us; N = 128 in FP32 28.9 -> 23.8 us, N = 32 in FP64 22.9 -> 12.5 us.
 template <typename V, typename Gt, int N>
-__global__ void __launch_bounds__(Shape<N>::THREADS_X) k_fields_x(const V* __restrict__ tw, const V* __restrict__ W,
-                                                                  Gt* __restrict__ G)
+__global__ void __launch_bounds__(Shape<N>::THREADS_X) k_fields_x(double kf, int slot7, const V* __restrict__ tw,
+                                                                  const V* __restrict__ W, Gt* __restrict__ G)
 {
     using S = Shape<N>;
     constexpr int XL = S::XL, N1 = S::N1, N2 = S::N2, T = S::T, PS = S::XPS;
@@ -624,11 +789,9 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_X) k_fields_x(const V* __res
     V* tr = s_tw + S::TWS;          // 4 XL TSX transpose elements, then 4 XL PS results
     const int t = threadIdx.x % T, lp = threadIdx.x / T;
     const int lo = lp % XL, p = lp / XL;
-    const size_t N3 = (size_t)N * N * N;
     const size_t line0 = (size_t)blockIdx.x * XL;
     V v[N1];
-    const V* src = W + p * N3 + (line0 + lo) * N;
-    sfor<N1>([&](auto N1i) { v[N1i] = src[N2 * N1i + t]; });
+    x_line<V, N>(v, p, t, kf, slot7, line0 + lo, W);
     load_line_twiddles<V, N>(s_tw, tw);
     __syncthreads();
     line_first<V, N>(v, t, s_tw, tr + lp * S::TSX);
@@ -655,11 +818,12 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_X) k_fields_x(const V* __res
 // values as a gather grid of type Gt would hold them, straight into out[8][N^3] (slots 0-5
 // from grids 0-2, phi_dot from grid 3, psi from grid 4).
 template <typename V, typename Gt, int N>
-__global__ void __launch_bounds__(Shape<N>::THREADS) k_fields_x_planar(const V* __restrict__ tw, const V* __restrict__ W,
+__global__ void __launch_bounds__(Shape<N>::THREADS) k_fields_x_planar(double kf, const V* __restrict__ tw,
+                                                                       const V* __restrict__ W,
                                                                        double* __restrict__ out)
 {
     using S = Shape<N>;
-    constexpr int N1 = S::N1, N2 = S::N2, T = S::T, LPB = S::THREADS / T;
+    constexpr int N1 = S::N1, T = S::T, LPB = S::THREADS / T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* s_tw = reinterpret_cast<V*>(smem_raw);
     V* tr = s_tw + S::TWS;
@@ -667,8 +831,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS) k_fields_x_planar(const V* 
     const size_t N3 = (size_t)N * N * N;
     const size_t line = (size_t)blockIdx.x * LPB + lo;
     V v[N1];
-    const V* src = W + p * N3 + line * N;
-    sfor<N1>([&](auto N1i) { v[N1i] = src[N2 * N1i + t]; });
+    x_line<V, N>(v, p, t, kf, kSlot7Zero, line, W);
     load_line_twiddles<V, N>(s_tw, tw);
     __syncthreads();
     line_first<V, N>(v, t, s_tw, tr + lo * S::TSX);
@@ -714,6 +877,30 @@ cudaError_t run_z(cudaStream_t s, const FieldArgs& a, const void* A, const void*
     return cudaGetLastError();
 }
 
+template <int N>
+cudaError_t run_half_z(cudaStream_t s, const FieldArgs& a, const void* A, const void* R, const void* tw, void* W)
+{
+    using S = Shape<N>;
+    constexpr int NT = S::HZ * S::T;
+    const size_t sm = (size_t)(S::TWS + S::HZ * S::template line_stride<16, S::HZ>()) * 16 + (size_t)S::N1 * NT * 8;
+    cudaError_t e = set_smem(k_half_z<N>, sm);
+    if (e != cudaSuccess) return e;
+    k_half_z<N><<<dim3(kHalfZ * (N / 2 / S::HZ), N), NT, sm, s>>>(a, (const double*)A, (const double2*)R,
+                                                                   (const double2*)tw, (double2*)W);
+    return cudaGetLastError();
+}
+
+template <int N>
+cudaError_t run_half_y(cudaStream_t s, double kf, const void* tw, void* W)
+{
+    using S = Shape<N>;
+    const size_t sm = (size_t)(S::TWS + S::HX * S::template line_stride<16, S::HX>()) * 16;
+    cudaError_t e = set_smem(k_half_y<N>, sm);
+    if (e != cudaSuccess) return e;
+    k_half_y<N><<<dim3(kHalfY * (N / 2 / S::HX), N), S::HX * S::T, sm, s>>>(kf, (const double2*)tw, (double2*)W);
+    return cudaGetLastError();
+}
+
 template <typename V, int N>
 cudaError_t run_y(cudaStream_t s, int grids, const void* tw, void* W)
 {
@@ -727,26 +914,27 @@ cudaError_t run_y(cudaStream_t s, int grids, const void* tw, void* W)
 }
 
 template <typename V, typename Gt, int N>
-cudaError_t run_x(cudaStream_t s, const void* tw, const void* W, void* G)
+cudaError_t run_x(cudaStream_t s, const FieldArgs& a, const void* tw, const void* W, void* G)
 {
     using S = Shape<N>;
     const size_t sm = S::template x_smem<V>();
     cudaError_t e = set_smem(k_fields_x<V, Gt, N>, sm);
     if (e != cudaSuccess) return e;
-    k_fields_x<V, Gt, N><<<(unsigned)((size_t)N * N / S::XL), S::THREADS_X, sm, s>>>((const V*)tw, (const V*)W, (Gt*)G);
+    k_fields_x<V, Gt, N><<<(unsigned)((size_t)N * N / S::XL), S::THREADS_X, sm, s>>>(a.kf, a.slot7, (const V*)tw,
+                                                                                      (const V*)W, (Gt*)G);
     return cudaGetLastError();
 }
 
 template <typename V, typename Gt, int N>
-cudaError_t run_x_planar(cudaStream_t s, const void* tw, const void* W, double* out)
+cudaError_t run_x_planar(cudaStream_t s, const FieldArgs& a, const void* tw, const void* W, double* out)
 {
     using S = Shape<N>;
     constexpr int LPB = S::THREADS / S::T;
     const size_t sm = (size_t)(S::TWS + LPB * S::TSX) * sizeof(V);
     cudaError_t e = set_smem(k_fields_x_planar<V, Gt, N>, sm);
     if (e != cudaSuccess) return e;
-    k_fields_x_planar<V, Gt, N><<<dim3((unsigned)((size_t)N * N / LPB), 5), S::THREADS, sm, s>>>((const V*)tw,
-                                                                                              (const V*)W, out);
+    k_fields_x_planar<V, Gt, N><<<dim3((unsigned)((size_t)N * N / LPB), 5), S::THREADS, sm, s>>>(
+        a.kf, (const V*)tw, (const V*)W, out);
     return cudaGetLastError();
 }
 
@@ -865,7 +1053,7 @@ cudaError_t launch_noise(cudaStream_t s, int precision, const FieldArgs& a, void
 cudaError_t launch_fields_z(cudaStream_t s, int precision, const FieldArgs& a, const void* A, const void* R,
                             const void* tw, void* W0)
 {
-#define Z64(n) run_z<double2, n>(s, a, A, R, tw, W0)
+#define Z64(n) run_half_z<n>(s, a, A, R, tw, W0)
 #define Z32(n) run_z<float2, n>(s, a, A, R, tw, W0)
     if (precision == FDF_PREC_F64) FDF_DISPATCH_N(a.N, Z64)
     FDF_DISPATCH_N(a.N, Z32)
@@ -873,37 +1061,38 @@ cudaError_t launch_fields_z(cudaStream_t s, int precision, const FieldArgs& a, c
 #undef Z32
 }
 
-cudaError_t launch_fields_y(cudaStream_t s, int precision, int N, int grids, const void* tw, void* W)
+cudaError_t launch_fields_y(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, void* W)
 {
-#define Y64(n) run_y<double2, n>(s, grids, tw, W)
-#define Y32(n) run_y<float2, n>(s, grids, tw, W)
-    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(N, Y64)
-    FDF_DISPATCH_N(N, Y32)
+#define Y64(n) run_half_y<n>(s, a.kf, tw, W)
+#define Y32(n) run_y<float2, n>(s, a.grids, tw, W)
+    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(a.N, Y64)
+    FDF_DISPATCH_N(a.N, Y32)
 #undef Y64
 #undef Y32
 }
 
-cudaError_t launch_fields_x(cudaStream_t s, int precision, int N, const void* tw, const void* W, void* G)
+cudaError_t launch_fields_x(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, const void* W, void* G)
 {
-#define X64(n) run_x<double2, double, n>(s, tw, W, G)
-#define X32(n) run_x<float2, float, n>(s, tw, W, G)
-#define X16(n) run_x<float2, __nv_bfloat16, n>(s, tw, W, G)
-    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(N, X64)
-    if (precision == FDF_PREC_F32) FDF_DISPATCH_N(N, X32)
-    FDF_DISPATCH_N(N, X16)
+#define X64(n) run_x<double2, double, n>(s, a, tw, W, G)
+#define X32(n) run_x<float2, float, n>(s, a, tw, W, G)
+#define X16(n) run_x<float2, __nv_bfloat16, n>(s, a, tw, W, G)
+    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(a.N, X64)
+    if (precision == FDF_PREC_F32) FDF_DISPATCH_N(a.N, X32)
+    FDF_DISPATCH_N(a.N, X16)
 #undef X64
 #undef X32
 #undef X16
 }
 
-cudaError_t launch_fields_x_planar(cudaStream_t s, int precision, int N, const void* tw, const void* W, double* out)
+cudaError_t launch_fields_x_planar(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, const void* W,
+                                   double* out)
 {
-#define P64(n) run_x_planar<double2, double, n>(s, tw, W, out)
-#define P32(n) run_x_planar<float2, float, n>(s, tw, W, out)
-#define P16(n) run_x_planar<float2, __nv_bfloat16, n>(s, tw, W, out)
-    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(N, P64)
-    if (precision == FDF_PREC_F32) FDF_DISPATCH_N(N, P32)
-    FDF_DISPATCH_N(N, P16)
+#define P64(n) run_x_planar<double2, double, n>(s, a, tw, W, out)
+#define P32(n) run_x_planar<float2, float, n>(s, a, tw, W, out)
+#define P16(n) run_x_planar<float2, __nv_bfloat16, n>(s, a, tw, W, out)
+    if (precision == FDF_PREC_F64) FDF_DISPATCH_N(a.N, P64)
+    if (precision == FDF_PREC_F32) FDF_DISPATCH_N(a.N, P32)
+    FDF_DISPATCH_N(a.N, P16)
 #undef P64
 #undef P32
 #undef P16
