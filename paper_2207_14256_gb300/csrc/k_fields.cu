@@ -467,9 +467,13 @@ __device__ __forceinline__ void amp_entry(const float* A, int m, float& ap, floa
 // ---- pass z: spectrum + inverse DFT along z ---------------------------------
 // Block (x-tile, jy): TX columns along z.  Each thread reads the unit Gaussians of
 // its N1 modes once, with their amplitudes A[|n|^2] at this scale factor, then forms,
-// transforms and writes each of the four packed grids in turn.
+// transforms and writes each of the four packed grids in turn.  Its shared-memory traffic (two
+// transposes per grid, the amplitudes) needs warps to hide it: with the amplitudes of half the
+// modes in shared memory (44 -> 32 KB a block) and 96 registers, five blocks per SM instead of
+// four; N = 256: a build 493 -> 478 us (FP32), 458 -> 443 us (BF16); six blocks of 80 registers:
+// 487 and 452; N = 128: 67.0, 66.7 and 66.2 us.
 template <typename V, int N>
-__global__ void __launch_bounds__(Shape<N>::THREADS_Z, 4) k_fields_z(FieldArgs a,
+__global__ void __launch_bounds__(Shape<N>::THREADS_Z, N >= 512 ? 4 : 5) k_fields_z(FieldArgs a,
                                                                   const typename Real<V>::T* __restrict__ A,
                                                                   const V* __restrict__ R, const V* __restrict__ tw,
                                                                   V* __restrict__ W0)
@@ -481,7 +485,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, 4) k_fields_z(FieldArgs a
     extern __shared__ __align__(16) unsigned char smem_raw[];
     V* s_tw = reinterpret_cast<V*>(smem_raw);
     V* tr = s_tw + S::TWS;                                  // TX * TSZ
-    T* As = reinterpret_cast<T*>(tr + TX * TSZ);            // [3][N1][NT]: each thread's own column
+    T* As = reinterpret_cast<T*>(tr + TX * TSZ);            // [3][N1 / 2][NT]: each thread's own column
     load_line_twiddles<V, N>(s_tw, tw);
     const int xo = threadIdx.x % TX, t = threadIdx.x / TX;
     const int x0 = blockIdx.x * TX, jy = blockIdx.y;
@@ -492,29 +496,24 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, 4) k_fields_z(FieldArgs a
     V Rv[N1];
     sfor<N1>([&](auto I) { Rv[I] = R[(size_t)(N2 * I + t) * NN + (size_t)jy * N + x0 + xo]; });
     // The amplitudes depend on |n|^2 only, so the modes nz and -nz of a column share
-    // them.  Mode z = N2 I + t mirrors to z' = N - z: for t > 0 that is thread N2 - t,
-    // index N1 - 1 - I; for t = 0 it is thread 0, index (N1 - I) mod N1.  Each thread
-    // looks up the first half of its modes (t = 0 also I = N1/2) and writes the
-    // amplitudes into its own column and into its mirror partner's.
-    {
-        const int tp = t == 0 ? 0 : N2 - t;
-        const int partner = xo + TX * tp;
-        sfor<N1 / 2 + 1>([&](auto I) {
-            if (I < N1 / 2 || t == 0) {
-                const int z = N2 * I + t;
-                const int nz = sidx(z, N);
-                const int Ip = t == 0 ? (N1 - I) % N1 : N1 - 1 - I;
-                T ap = T(0), af = T(0), ad = T(0);
-                if (nx != h && ny != h && nz != h) amp_entry(A, nx * nx + ny * ny + nz * nz, ap, af, ad);
-                As[(0 * N1 + I) * NT + threadIdx.x] = ap;
-                As[(1 * N1 + I) * NT + threadIdx.x] = af;
-                As[(2 * N1 + I) * NT + threadIdx.x] = ad;
-                As[(0 * N1 + Ip) * NT + partner] = ap;
-                As[(1 * N1 + Ip) * NT + partner] = af;
-                As[(2 * N1 + Ip) * NT + partner] = ad;
-            }
-        });
-    }
+    // them: each thread looks up the first half of its modes, nz >= 0.  Mode z = N2 I + t
+    // mirrors to z' = N - z: for t > 0 that is thread N2 - t, index N1 - 1 - I; for t = 0 it
+    // is thread 0, index N1 - I (I = N1 / 2: the Nyquist mode, zero).
+    constexpr int NH = N1 / 2;
+    sfor<NH>([&](auto I) {
+        const int nz = N2 * I + t;
+        T ap = T(0), af = T(0), ad = T(0);
+        if (nx != h && ny != h) amp_entry(A, nx * nx + ny * ny + nz * nz, ap, af, ad);
+        As[(0 * NH + I) * NT + threadIdx.x] = ap;
+        As[(1 * NH + I) * NT + threadIdx.x] = af;
+        As[(2 * NH + I) * NT + threadIdx.x] = ad;
+    });
+    const int mirror = t == 0 ? (int)threadIdx.x + NT : xo + TX * (N2 - t);
+    auto amp = [&](int slot, auto I) {
+        const T* Aq = As + slot * NH * NT;
+        if constexpr (I < NH) return Aq[I * NT + threadIdx.x];
+        else return I == NH && t == 0 ? T(0) : Aq[(N1 - 1 - I) * NT + mirror];
+    };
     __syncthreads();
     const size_t N3 = NN * N;
     // this block's packed grids: all of them, or one of gridDim.z
@@ -530,10 +529,9 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, 4) k_fields_z(FieldArgs a
             constexpr int P = Q < 4 ? (int)Q : 3;
             sfor<N1>([&](auto I) {
                 const T kz = kf * (T)sidx(N2 * I + t, N);
-                const int o = I * NT + threadIdx.x;
-                const T apsi = (P == 2 || Q == 5) ? T(0) : As[0 * N1 * NT + o];
-                const T aphi = (P == 1 || P == 2 || Q == 4) ? As[1 * N1 * NT + o] : T(0);
-                const T adot = (P == 3) ? As[2 * N1 * NT + o] : T(0);
+                const T apsi = (P == 2 || Q == 5) ? T(0) : amp(0, I);
+                const T aphi = (P == 1 || P == 2 || Q == 4) ? amp(1, I) : T(0);
+                const T adot = (P == 3) ? amp(2, I) : T(0);
                 v[I] = packed<V>(P, Rv[I], Q == 4 ? apsi + aphi : apsi, aphi, adot, kx, ky, kz);
             });
         };
@@ -870,7 +868,7 @@ cudaError_t run_z(cudaStream_t s, const FieldArgs& a, const void* A, const void*
     using S = Shape<N>;
     using T = typename Real<V>::T;
     constexpr int TSZ = S::template line_stride<sizeof(V), S::TZ>();
-    const size_t sm = (size_t)(S::TWS + S::TZ * TSZ) * sizeof(V) + (size_t)3 * S::N1 * S::THREADS_Z * sizeof(T);
+    const size_t sm = (size_t)(S::TWS + S::TZ * TSZ) * sizeof(V) + (size_t)3 * (S::N1 / 2) * S::THREADS_Z * sizeof(T);
     cudaError_t e = set_smem(k_fields_z<V, N>, sm);
     if (e != cudaSuccess) return e;
     k_fields_z<V, N><<<dim3(N / S::TZ, N, S::kSplitGrids ? a.grids : 1), S::THREADS_Z, sm, s>>>(a, (const T*)A, (const V*)R, (const V*)tw, (V*)W0);
