@@ -608,6 +608,7 @@ void fill_pass(const fdf_ctx* c, PushArgs& a)
     a.L = c->p.box_mpc;
     a.invL = 1.0 / c->p.box_mpc;
     a.invh = c->p.n_grid / c->p.box_mpc;
+    a.invh32 = (float)a.invh;
     a.fx_scale = split_ff(4294967296.0 / c->p.box_mpc);
 }
 

@@ -788,11 +788,11 @@ void push_split(cudaStream_t s, unsigned b, const PushArgs& a, const ParticleSta
 //
 // GB300 runs FP64 arithmetic and FP64 <-> FP32 conversions at 1/64 of its FP32 rate, so
 // conversions are bit operations (d2f_bits, f2d_bits), and the inverse square roots, their
-// squares, the kick's integrals and q's sums get the bits of their FP64 formulas from the
-// integer and FP32 pipes (wide_math.cuh): 13 FP64 instructions per particle-step (|q|^2 3,
-// v 1, polynomial 5, D 1, x 3), 30 with everything in FP64.  3 x 256^3 particles, 200
-// steps, passes of 8: 563 -> 341 ms in the pass; node sums, 160^3 particles, 100 steps:
-// 61.4 -> 19.7 ms.
+// squares and products, the kick's integrals and q's sums get the bits of their FP64 formulas
+// from the integer and FP32 pipes (wide_math.cuh): 12 FP64 instructions per particle-step
+// (|q|^2 3, v 1, polynomial 5, x 3), 30 with everything in FP64.  3 x 256^3 particles, 200
+// steps, passes of 8: 563 -> 337 ms in the pass; node sums, 160^3 particles, 100 steps:
+// 61.4 -> 19.5 ms.
 
 // Periodic wrap into [0, L) (wrap_f64, a result equal to L mapping to 0), taken only
 // when x left the box.  The test runs on the bit patterns (IEEE doubles order like
@@ -927,7 +927,7 @@ __device__ __forceinline__ Norm0 norm0(const PushArgs& a, float qa, float qb, fl
     q02 = d2f_bits(n.s);
     n.h = q02 * a.q_unit2;
     // in the unit first: the low part of a tiny |q_0|^2 would leave FP32's exponents
-    n.l = d2f_bits((n.s - f2d_bits(q02)) * (double)a.q_unit2);
+    n.l = d2f_bits((n.s - f2d_bits(q02)) * f2d_bits(a.q_unit2));
     return n;
 }
 
@@ -951,7 +951,6 @@ __device__ __forceinline__ void wide_particle(const PushArgs& a, double* __restr
 {
     const int64_t n = a.n;
     const uint32_t N = (uint32_t)a.N;
-    const float invh = (float)a.invh;
     const int s = UNI ? 0 : species_of(a, i);
     double x[3] = {__ldcs(xd + i), __ldcs(xd + n + i), __ldcs(xd + 2 * n + i)};
     double q[3] = {__ldcs(qd + i), __ldcs(qd + n + i), __ldcs(qd + 2 * n + i)};
@@ -971,7 +970,7 @@ __device__ __forceinline__ void wide_particle(const PushArgs& a, double* __restr
         if (st.do_kick) {
             float Kpsif, Kphif, g[8];
             kick_integrals<SERIES>(a, st, s, n0, Kpsif, Kphif);
-            gather_wide<Gt>(a.order, reinterpret_cast<const Gt*>(a.G[u]), N, invh, x, g);
+            gather_wide<Gt>(a.order, reinterpret_cast<const Gt*>(a.G[u]), N, a.invh32, x, g);
             const float qdphi = qa * g[3] + qb * g[4] + qc * g[5];
             const float b = qdphi * Kphif + g[6] * st.wide.dtau_k;
             const float a2 = q02 * Kphif;

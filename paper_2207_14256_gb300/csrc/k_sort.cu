@@ -8,7 +8,7 @@
 // predicted position halfway through the next pass, with a counting sort:
 //   keys:    key of every particle and a histogram of keys;
 //   scan:    exclusive prefix sum of the histogram (recursive, any bin count);
-//   pack:    every particle's state, as one 64-byte record, goes to
+//   pack:    every particle's state, as one record of 64, 96 or 128 bytes, goes to
 //            offset[key]++ (warp-aggregated atomics, two particles in flight
 //            per thread);
 //   unpack:  the records go back to the arrays of the other half of the

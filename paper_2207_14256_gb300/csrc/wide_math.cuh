@@ -2,17 +2,18 @@
 // integer pipes, bit for bit.
 //
 // GB300 issues two FP64 instructions per clock and SM against 128 FP32 or integer ones, so
-// an FP64 instruction costs as much as 64 others.  The two functions here give the bits of
+// an FP64 instruction costs as much as 64 others.  The functions here give the bits of
 // an FP64 formula without its FP64 instructions: each forms the formula's last, rounded
 // value with some bits to spare and a bound on its distance from what FP64 arithmetic
 // gets; where that value lies so near a rounding boundary that the bound could cross it
 // (one evaluation in 2^11 or rarer), it says so and the caller runs the FP64 formula.
-//   w_rsqrt53: rsqrt_fp64's four FP64 instructions (~50 others), w_square53 its square (~20);
+//   w_rsqrt53: rsqrt_fp64's four FP64 instructions (~50 others), w_square53 its square (~20),
+//              w_mul53 its product with a double;
 //   w_add:     the sum of a double and a much smaller float (~25, and no conversion);
 //   w_kick:    the kick's integrals as the FP32 values their user reads (9 FP64
 //              instructions as polynomials, 8 per node as sums);
 //   w_sqrt53, w_div53: correctly rounded roots and quotients (the sampler, |q|, the weights).
-// tests/test_wide_math.py compares both with the FP64 formulas, bit for bit.
+// tests/test_wide_math.py compares them with the FP64 formulas, bit for bit.
 //
 // Plain C++ besides the intrinsics, so that the test compiles it for the host.
 #pragma once
