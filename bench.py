@@ -43,19 +43,18 @@ FORM_NAMES = {0: "FP64 grids and state", 1: "FP32 grids, FP64 state", 2: "BF16 g
               3: "FP32 grids, split state (fixed-point x, FP32 q0 + dq)",
               4: "BF16 grids, split state (fixed-point x, FP32 q0 + dq)"}
 # FP64-pipe instructions of the FP64-state pass (k_push_wide), counted in its source: a drift
-# takes 18 (|q|^2 3, v = 1 + |q|^2 / (m a_c)^2 1, the inverse square root 4, t 1, five FP64
-# terms of the polynomial 5, D 1, x += q D 3) and a kick 12 (argument 1, first-order inverse
-# square root 3, one FP64 term of each of two polynomials 2, K_phi 1, K_psi 2, q += dq 3);
-# |q0|^2 takes 3 per particle and pass.  Conversions run on the integer pipe.  ncu's count of
-# FP64-pipe instructions (profiles/) checks these figures.
-WIDE_FP64_PER_STEP = 30
-WIDE_FP64_PER_PASS = 3
+# takes 12 (|q|^2 3, v = 1 + |q|^2 / (m a_c)^2 1, five FP64 terms of the polynomial 5, x += q D 3);
+# the inverse square root, its square and product, the kick's integrals, q += dq and the
+# conversions run on the integer and FP32 pipes.  |q0|^2 and its low part take 5 per particle
+# and pass.  ncu's count of FP64-pipe instructions (profiles/) checks these figures.
+WIDE_FP64_PER_STEP = 12
+WIDE_FP64_PER_PASS = 5
 
 # FP64-pipe instructions per particle-step of the plain FP64 pass (k_push_f64), from ncu
 # (sm__inst_executed_pipe_fp64.sum x 32 / particle-steps of the launch, 128^3 particles, one step
 # per pass; profiles/), for its FP64-pipe roofline.  Dropped if the sources changed.
-PLAIN_FP64 = {"per_particle_step": 19136512 * 32 / 128 ** 3,
-              "sources_sha256": "a61bc5ef3323c092:256bffcc5979e4f1:55a2ba5a6a8ebd0f"}
+PLAIN_FP64 = {"per_particle_step": 8831492 * 32 / 128 ** 3,
+              "sources_sha256": "80ae3655c29e4f3f:80f9684a0189b685:d5c895147bbe2b3b:2a492a4e0bbb3fee"}
 
 # DRAM bytes per particle-step of the pass, from ncu (dram__bytes_read.sum + dram__bytes_write.sum,
 # mean over the 50 passes of a one-species 256^3 run of the bench's schedule;
@@ -67,7 +66,7 @@ PUSH_TRAFFIC = {1: {"bytes_per_particle_step": (10.827e9 + 0.795e9) / (256 ** 3 
                     "sources_sha256": "a61bc5ef3323c092:256bffcc5979e4f1:55a2ba5a6a8ebd0f"},
                 3: {"bytes_per_particle_step": (3.433e9 + 0.402e9) / (256 ** 3 * 4),
                     "sources_sha256": "a61bc5ef3323c092:256bffcc5979e4f1:55a2ba5a6a8ebd0f"}}
-PUSH_SOURCES = ("k_particles.cu", "fdf_internal.cuh", "device_math.cuh")
+PUSH_SOURCES = ("k_particles.cu", "fdf_internal.cuh", "device_math.cuh", "wide_math.cuh")
 
 
 def push_sources_hash():
