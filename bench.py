@@ -57,15 +57,15 @@ PLAIN_FP64 = {"per_particle_step": 8831492 * 32 / 128 ** 3,
               "sources_sha256": "80ae3655c29e4f3f:80f9684a0189b685:d5c895147bbe2b3b:2a492a4e0bbb3fee"}
 
 # DRAM bytes per particle-step of the pass, from ncu (dram__bytes_read.sum + dram__bytes_write.sum,
-# mean over the 50 passes of a one-species 256^3 run of the bench's schedule;
+# mean over the 50 passes of a one-species 256^3 run with the schedule named in
 # profiles/), by precision setting.  A launch's traffic is this times the particle-steps it
 # processes (the species are sorted one after the other, so each reads the grid on its own).
 # Valid only for the kernel sources they were measured on: their hash is checked and the figure
 # dropped if they changed.
-PUSH_TRAFFIC = {1: {"bytes_per_particle_step": (10.827e9 + 0.795e9) / (256 ** 3 * 8),
-                    "sources_sha256": "a61bc5ef3323c092:256bffcc5979e4f1:55a2ba5a6a8ebd0f"},
-                3: {"bytes_per_particle_step": (3.433e9 + 0.402e9) / (256 ** 3 * 4),
-                    "sources_sha256": "a61bc5ef3323c092:256bffcc5979e4f1:55a2ba5a6a8ebd0f"}}
+PUSH_TRAFFIC = {1: {"bytes_per_particle_step": (10.646e9 + 0.802e9) / (256 ** 3 * 8),
+                    "sources_sha256": "80ae3655c29e4f3f:80f9684a0189b685:d5c895147bbe2b3b:2a492a4e0bbb3fee"},
+                3: {"bytes_per_particle_step": (3.435e9 + 0.401e9) / (256 ** 3 * 4),
+                    "sources_sha256": "80ae3655c29e4f3f:80f9684a0189b685:d5c895147bbe2b3b:2a492a4e0bbb3fee"}}
 PUSH_SOURCES = ("k_particles.cu", "fdf_internal.cuh", "device_math.cuh", "wide_math.cuh")
 
 
@@ -237,8 +237,8 @@ def hbm_roofline(p, ktimes, hbm):
             "frac": achieved / hbm if hbm else None,
             "traffic": (tr["bytes_per_particle_step"] * n_total * p["n_steps"] / max(push_n, 1)
                         if tr and push_sources_hash() == tr["sources_sha256"] else None),
-            "traffic_note": "ncu DRAM bytes per particle-step of the pass (one-species 256^3 run, the headline's "
-                            "schedule; profiles/) times the launch's particle-steps; null when the kernel sources "
+            "traffic_note": "ncu DRAM bytes per particle-step of the pass (one-species 256^3 run with the "
+                            "schedule named in profiles/) times the launch's particle-steps; null when the kernel sources "
                             "changed since the capture",
             "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if hbm else "fallback 6800",
             "algorithmic_bytes_per_launch": alg, "avg_launch_ms": push_avg,

@@ -209,7 +209,7 @@ template <int N> struct Shape {
     // z pass: 128 threads (its per-thread amplitudes live in shared memory) that form all four
     // packed grids in turn.  Up to N = 64 that would be N^2 T / 128 <= 256 blocks of a long
     // chain for 152 SMs: there a block is 8 columns of one grid (N = 32 in FP64: 512 blocks of
-    // 32 threads for 32 of 128, 28 -> 13 us a pass).
+    // 32 threads for 32 of 128, 28 -> 13 us a pass when FP64 took this path).
     static constexpr bool kSplitGrids = N <= 64;
     static constexpr int TZ0 = kSplitGrids ? 8 : 128 / T;
     static constexpr int TZ = TZ0 < N ? TZ0 : N;
