@@ -81,6 +81,9 @@ __device__ __forceinline__ FF ff_rsqrt(FF s)
 // rate of its FMAs), so the FP64-state particle pass converts with bit operations,
 // which run on the integer pipe.  Both follow the IEEE-754 binary64 and binary32
 // layouts (sign, biased exponent, fraction; the biases differ by 1023 - 127 = 896).
+// They are for the pass's inner loops and know no NaN, infinity or subnormal; what is read
+// or written once (gradients of the transform, weights, densities, positions) goes through
+// w_d2f and w_f2d, which are plain casts for every value.
 //
 // d2f_bits: a double in the FP32 normal range (or a value below 2^-126 in
 // magnitude, returned as a signed zero) to the nearest float, ties away from zero.
@@ -168,7 +171,7 @@ __device__ __forceinline__ void fixed_cell(uint32_t X, uint32_t N, uint32_t& i0,
 // FP64 instructions for every argument and select afterwards.
 static __device__ __noinline__ double rsqrt_slow(double u) { return rsqrt_fp64(u); }
 static __device__ __noinline__ double mul_slow(double a, double b) { return a * b; }
-static __device__ __noinline__ double add_slow(double q, float d) { return q + f2d_bits(d); }
+static __device__ __noinline__ double add_slow(double q, float d) { return q + w_f2d(d); }
 static __device__ __noinline__ double sqrt_slow(double u) { return __dsqrt_rn(u); }
 static __device__ __noinline__ double div_slow(double a, double b) { return __ddiv_rn(a, b); }
 

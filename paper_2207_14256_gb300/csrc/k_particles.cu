@@ -445,12 +445,12 @@ __global__ void __launch_bounds__(kThreads) k_initial(ParticleState st, int64_t 
             float gf[8];
             gather_order<Gt>(order, G, (uint32_t)N, X0, X1, X2, gf);
 #pragma unroll
-            for (int s = 0; s < 8; ++s) g[s] = f2d_bits(gf[s]);
+            for (int s = 0; s < 8; ++s) g[s] = w_f2d(gf[s]);
         }
         // eps scales a term of ~1e-9 of q: a root through rsqrt_any serves it
         const double p = st.pmag[i];
         const double e2 = p * p + m2a2;
-        const double eps = __double_as_longlong(e2) > 0 ? e2 * rsqrt_any(e2) : 0.0;
+        const double eps = __double_as_longlong(e2) != 0 ? e2 * rsqrt_any(e2) : 0.0;
         const double c = eps * tau0_6;          // eps tau0 / 6 (tau0/6 formed once)
         const double r = 1.0 - 0.5 * g[7];
 #pragma unroll
@@ -1149,7 +1149,7 @@ __device__ __forceinline__ void load_state(const ParticleState& st, int64_t n, i
             q[d] = st.qd[d * n + i];
         } else {
             x[d] = L * frac32(st.X[d * n + i]);
-            q[d] = f2d_bits(st.q0f[d * n + i]) + f2d_bits(st.dqf[d * n + i]);
+            q[d] = w_f2d(st.q0f[d * n + i]) + w_f2d(st.dqf[d * n + i]);
         }
     }
 }
@@ -1384,7 +1384,7 @@ __global__ void __launch_bounds__(kThreads) k_deposit(ParticleState st, int64_t 
         // (an FP64 conversion costs an FP64 slot)
         auto to64 = [](Wt t) {
             if constexpr (F == kPlain) return t;
-            else return f2d_bits(t);
+            else return w_f2d(t);
         };
         if constexpr (PRESUM) {
             // Particles sharing the base cell share every node: one match on it, sums

@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(kThreads) k_export_unpack(const void* __restri
             const SplitRec r = load_split(recs, o);
             for (int d = 0; d < 3; ++d) {
                 x[d] = L * frac32(r.X[d]);
-                q[d] = f2d_bits(r.q0[d]) + f2d_bits(r.dq[d]);
+                q[d] = w_f2d(r.q0[d]) + w_f2d(r.dq[d]);
             }
             pm = r.pmag;
         }

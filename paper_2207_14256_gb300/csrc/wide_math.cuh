@@ -210,15 +210,29 @@ FDF_DEV bool w_div53(double a, double b, double q, double& r)
     return ok;
 }
 
-// The nearest float of a double in the FP32 normal range, ties to even (magnitudes below it
-// become zero, as d2f_bits takes them).
+// (float)d and (double)f in integers: the bits of the plain casts for every value.  What lies
+// outside FP32's normal range (zeros, subnormals, overflows, infinities, NaN) is left to the
+// cast itself, as a call: inlined, every argument would run its FP64 instruction.
+static __device__ __attribute__((noinline)) float w_d2f_rest(double d) { return (float)d; }
+static __device__ __attribute__((noinline)) double w_f2d_rest(float f) { return (double)f; }
+
 FDF_DEV float w_d2f(double d)
 {
     const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
     const uint32_t mag = hi & 0x7FFFFFFFu;
     uint32_t f = ((mag - 0x38000000u) << 3) | (lo >> 29);
     f += (lo & 0x1FFFFFFFu) > 0x10000000u - (f & 1u);
-    return __uint_as_float((hi & 0x80000000u) | (mag < 0x38100000u ? 0u : f));
+    float r = __uint_as_float((hi & 0x80000000u) | f);
+    if (mag - 0x38100000u >= 0x0FE00000u) r = w_d2f_rest(d);
+    return r;
+}
+
+FDF_DEV double w_f2d(float f)
+{
+    const uint32_t b = __float_as_uint(f), mag = b & 0x7FFFFFFFu;
+    double r = __hiloint2double((int)(((mag >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
+    if (mag - 0x00800000u >= 0x7F000000u) r = w_f2d_rest(f);
+    return r;
 }
 
 // ---- pairs of floats (value = hi + lo, 48 bits) -----------------------------------------
