@@ -143,9 +143,9 @@ typedef struct fdf_params {
                                   read and written once per pass, and 2 steps_per_pass + 1 grids
                                   are held (0 = 4 for the FP32/BF16-grid forms, 1 for the plain
                                   FP64 form) */
-    int32_t  sort_tile;        /* sort buckets are cubes of 2^sort_tile cells per axis, 0..3
-                                  (0 = single cells), or larger cubes of up to 4^3 cells while a
-                                  bucket would hold only a few particles (fewer than 3 of a
+    int32_t  sort_tile;        /* sort buckets are cubes of 2^sort_tile cells per axis, 1..3;
+                                  0 = automatic: single cells, or cubes of 2^3 or 4^3 cells while
+                                  a bucket would hold only a few particles (fewer than 3 of a
                                   species on average, or than 32 in the FP64-state forms with
                                   interp_order 1) */
     int32_t  sort_cells;       /* with sort_every = 0: re-bucket when the typical particle has

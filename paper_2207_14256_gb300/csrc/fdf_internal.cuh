@@ -312,20 +312,22 @@ struct SortLead {
     // use the positions alone and the sampled momenta qs travel with the particles
     int pre_transform;
 };
-// The bucket size: sort_tile's, or the smallest larger one (up to 4^3 cells) whose buckets hold
-// 3 particles of a species on average, 32 in the FP64-state form's trilinear passes.  Smaller
-// buckets order nothing that a warp of 32 would gain from, while the histogram of more bins
-// than particles costs the sort its atomics and scans: single cells against the size taken,
-// 256^3 particles on 256^3 (300 steps, BF16) 336.2 -> 326.6 ms, 2 x 150^3 on 128^3 (split
-// state) 38.3 -> 36.5 ms (38.1 with 4^3 cells: its gather is bound by L1), initial
-// conditions of 3 x 200^3 on 256^3 8.1 -> 7.2 ms.
+// The bucket size: sort_tile's cubes if it names a size (1..3), else (0) the smallest of up to
+// 4^3 cells whose buckets hold 3 particles of a species on average, 32 in the FP64-state
+// form's trilinear passes.  Smaller buckets order nothing that a warp of 32 would gain from,
+// while the histogram of more bins than particles costs the sort its atomics and scans: single
+// cells against the size taken, 256^3 particles on 256^3 (300 steps, BF16) 336.2 -> 326.6 ms,
+// 2 x 150^3 on 128^3 (split state) 38.3 -> 36.5 ms (38.1 with 4^3 cells: its gather is bound
+// by L1), initial conditions of 3 x 200^3 on 256^3 8.1 -> 7.2 ms.  These have 0.5 to 1.6
+// particles per cell and species; no density between 2 and 32 was measured.
 inline int sort_tile_shift(const fdf_params& p)
 {
+    if (p.sort_tile > 0) return p.sort_tile;
     const double per_cell = (double)p.n_part / ((double)p.n_grid * p.n_grid * p.n_grid);
     const double want = form_of(p.precision) == kWide && p.interp_order != 2 ? 32.0 : 3.0;
     int s = 0;
     while (s < 2 && per_cell * (double)(1 << (3 * s)) < want) ++s;
-    return s > p.sort_tile ? s : p.sort_tile;
+    return s;
 }
 size_t sort_record_bytes(int precision);
 cudaError_t launch_sort(cudaStream_t s, int precision, const ParticleState& a, const ParticleState& b, int64_t n,
