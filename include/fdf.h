@@ -389,10 +389,11 @@ FDF_API const char* fdf_last_error(void);
 FDF_API void fdf_destroy(fdf_ctx* c);
 
 /* Autotuner of the schedule knobs that change speed only (no result beyond the
- * stated tolerances): sort_cells, sort_tile and steps_per_pass.  It times whole runs (fdf_sample + fdf_step(n_steps)) of p on the
- * device, one knob at a time (coordinate descent over sort_cells in {2, 4, 8, 16, 32, 64},
- * sort_tile in {0, 1, 2, 3}, steps_per_pass in {2, 3, 4, 6, 8}, gather_tile in {-1, 1}
- * (split-state forms), then sort_cells again in {3, 5, 6, 12, 24, 48}), starting from the automatic choices, and writes
+ * stated tolerances): sort_cells, sort_tile and steps_per_pass.  It times whole runs
+ * (fdf_sample + fdf_step(n_steps)) of p on the device, one knob at a time (coordinate
+ * descent over sort_cells in {2, 4, 8, 16, 32, 64}, sort_tile in {0, 1, 2, 3} without the size
+ * that 0 stands for, steps_per_pass in {2, 3, 4, 6, 8}, gather_tile in {-1, 1} (split-state
+ * forms), then sort_cells again in {3, 5, 6, 12, 24, 48}), starting from the automatic choices, and writes
  * the fastest parameter set to *out (p with the knobs set).  The paper
  * has no counterpart.  stream: a cudaStream_t or NULL; every trial allocates
  * and frees its own context.  ms (may be NULL) receives the best run time;

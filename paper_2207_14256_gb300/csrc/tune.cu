@@ -90,11 +90,14 @@ extern "C" int fdf_tune(const fdf_params* p, const fdf_tables* t, void* stream, 
     for (const Knob& k : knobs) {
         if (k.field == &fdf_params::gather_tile && wide) continue;
         const int32_t start = best.*(k.field);
+        const int start_shift = sort_tile_shift(best);
         for (int32_t v : k.values) {
             if (v == start) continue;
             fdf_params q = best;
             q.*(k.field) = v;
             if (q.sort_tile > 0 && (q.n_grid >> q.sort_tile) < 1) continue;
+            // the automatic bucket size is one of the others: a second run of it would decide by noise
+            if (k.field == &fdf_params::sort_tile && sort_tile_shift(q) == start_shift) continue;
             double m = 0;
             rc = timed_run(q, t, s, &m);
             if (rc) return rc;
