@@ -20,6 +20,9 @@ def load(tmp):
     fdf._lib, fdf.LIB_PATH = None, so
     L = fdf.lib()
     L.fdf_check_grid.argtypes = [C.c_void_p, C.c_int32, C.c_void_p, C.c_size_t]
+    L.fdf_check_kick_fp64.argtypes = [C.c_int32, C.POINTER(C.c_int32)]
+    L.fdf_check_kick_fp64.restype = None
+    L.fdf_check_bits.argtypes = [C.c_int64] + [C.c_void_p] * 4
     return fdf
 
 
