@@ -225,7 +225,7 @@ typedef struct fdf_tables {
 FDF_API int fdf_footprint(const fdf_params* p, size_t* bytes);
 
 /* Validate p and t, copy the tables to the device, allocate (or carve from
- * arena, a device pointer with arena_bytes >= fdf_footprint) every buffer,
+ * arena, a device pointer of any alignment with arena_bytes >= fdf_footprint) every buffer,
  * and precompute the background.  stream is a cudaStream_t (may be NULL).
  * On success *out holds a new context; on failure *out is NULL. */
 FDF_API int fdf_create(const fdf_params* p, const fdf_tables* t, void* stream, void* arena, size_t arena_bytes,

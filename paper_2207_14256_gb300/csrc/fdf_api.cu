@@ -1124,7 +1124,7 @@ int fdf_footprint(const fdf_params* p, size_t* bytes)
     int rc = validate(p);
     if (rc) return rc;
     if (!bytes) return fail(FDF_EINVAL, "bytes is NULL");
-    *bytes = make_layout(*p, 1024, 256, 8192).total;
+    *bytes = make_layout(*p, 1024, 256, 8192).total + kAlign;      // an arena of any alignment
     return FDF_OK;
 }
 
@@ -1189,11 +1189,12 @@ int fdf_create(const fdf_params* p, const fdf_tables* t, void* stream, void* are
     c->lay = make_layout(c->p, t->nk, t->na, t->ncdf);
     const Layout& L = c->lay;
     if (arena) {
-        if (arena_bytes < L.total) {
+        // the kernels' widest accesses (32 bytes) want their buffers aligned; an arena need not be
+        c->block = (char*)align_up((size_t)arena);
+        if (arena_bytes < L.total + (size_t)(c->block - (char*)arena)) {
             delete c;
             return fail(FDF_ENOMEM, "arena smaller than the footprint");
         }
-        c->block = (char*)arena;
     } else {
         cudaError_t e = cudaMalloc(&c->block, L.total);
         if (e != cudaSuccess) {
