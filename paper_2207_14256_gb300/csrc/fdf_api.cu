@@ -663,7 +663,13 @@ void fill_wide(fdf_ctx* c, bool drift, double d1, double d2, const double* Wd, c
 }
 
 // The kick's integrals for the FP32 pipe (w_kick), once it is known whether the pass uses
-// the fits (series) or sums the nodes: u.wide.kick_fast says whether they serve it.
+// the fits (series) or sums the nodes: u.wide.kick_fast says whether they serve it.  They do
+// not for fits longer than KickLen<true>::kDeg, which some passes of about 140 to 153 steps
+// from z = 1e9 to 31 have, nor for nodes farther apart than kick_node_poly takes (fewer than about
+// 90 steps); such a pass takes its kicks from FP64, 12 more FP64-pipe instructions per
+// particle-step with a fit, or its nodes' sums.  The pass per step, 160^3 particles in passes
+// of 4: 0.135 ms at 155 to 200 steps, 0.155 at 152, 0.163 at 150, 0.178 at 120 to 145 (node sums
+// on the FP32 pipe), 0.194 at 92 and 100, 0.440 at 60 to 88 (node sums in FP64).
 void fill_kick_fast(const fdf_ctx* c, bool series, SubStep& u)
 {
     WideCoef& w = u.wide;
@@ -732,8 +738,8 @@ void fill_substep(fdf_ctx* c, bool drift, double d1, double d2, bool kick, doubl
                 e[j] = sc.mud[jc] > 0 ? (sc.mud[j] - sc.mud[jc]) / sc.mud[jc] : 0.0;
                 u.emax = std::max(u.emax, std::fabs(e[j]));
             }
-            // Cd_k = c_k sum_j Wd_j e_j^k (the split-state form's series) with c_k the binomial coefficients of
-            // (1 + d)^(-1/2) - 1 = sum_k c_k d^k: c_1 = -1/2, c_k = c_(k-1) (1 - 2k)/(2k)
+            // Cd_k = c_k sum_j Wd_j e_j^k (the split-state form's series) with c_k the binomial
+            // coefficients of (1 + d)^(-1/2) - 1 = sum_k c_k d^k: c_1 = -1/2, c_k = c_(k-1) (1 - 2k)/(2k)
             double ck = 1.0;
             for (int k = 1; k <= kTaylor && form_of(c->p.precision) == kFixed; ++k) {
                 ck *= (1.0 - 2.0 * k) / (2.0 * k);
@@ -1389,7 +1395,10 @@ int slice_prepare(fdf_ctx* c, int j, std::vector<int>& bufs, std::vector<const v
         // grid would pay for every step)
         double lna[kMaxSub];
         int count = 0, missing = 0;
-        auto held = [&](double l) { return std::find(c->mode_lna, c->mode_lna + c->mode_count, l) != c->mode_lna + c->mode_count; };
+        auto held = [&](double l) {
+            const double *begin = c->mode_lna, *end = begin + c->mode_count;
+            return std::find(begin, end, l) != end;
+        };
         for (int kk : ks)
             if (find_grid(c, kk) < 0) {
                 lna[count++] = c->lna(kk);

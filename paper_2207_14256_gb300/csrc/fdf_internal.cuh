@@ -247,7 +247,7 @@ cudaError_t launch_mode_tables(cudaStream_t s, int precision, const FieldArgs& a
 // The unit Gaussian field R_n / sqrt(P_R/V) on the N^3 mode array (drawn once per run).
 cudaError_t launch_noise(cudaStream_t s, int precision, const FieldArgs& a, void* R);
 cudaError_t launch_fields_z(cudaStream_t s, int precision, const FieldArgs& a, const void* A, const void* R,
-                            const void* tw, void* W0);
+                            const void* tw, void* W);
 cudaError_t launch_fields_y(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, void* W);
 cudaError_t launch_fields_x(cudaStream_t s, int precision, const FieldArgs& a, const void* tw, const void* W, void* G);
 // The x pass of five packed grids into out[8][N^3], each value as a gather grid holds it.

@@ -476,7 +476,7 @@ template <typename V, int N>
 __global__ void __launch_bounds__(Shape<N>::THREADS_Z, N >= 512 ? 4 : 5) k_fields_z(FieldArgs a,
                                                                   const typename Real<V>::T* __restrict__ A,
                                                                   const V* __restrict__ R, const V* __restrict__ tw,
-                                                                  V* __restrict__ W0)
+                                                                  V* __restrict__ W)
 {
     using T = typename Real<V>::T;
     using S = Shape<N>;
@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(Shape<N>::THREADS_Z, N >= 512 ? 4 : 5) k_field
         }
         line_first<V, N>(v, t, s_tw, tr + xo * TSZ);
         __syncthreads();
-        V* dst = W0 + p * N3 + (size_t)jy * N + x0 + xo;
+        V* dst = W + p * N3 + (size_t)jy * N + x0 + xo;
         line_second<V, N>(t, tr + xo * TSZ, s_tw, [&](int z, V val) { dst[(size_t)z * NN] = val; });
         __syncthreads();
     }
@@ -863,7 +863,7 @@ cudaError_t set_smem(K kernel, size_t bytes)
 }
 
 template <typename V, int N>
-cudaError_t run_z(cudaStream_t s, const FieldArgs& a, const void* A, const void* R, const void* tw, void* W0)
+cudaError_t run_z(cudaStream_t s, const FieldArgs& a, const void* A, const void* R, const void* tw, void* W)
 {
     using S = Shape<N>;
     using T = typename Real<V>::T;
@@ -871,7 +871,8 @@ cudaError_t run_z(cudaStream_t s, const FieldArgs& a, const void* A, const void*
     const size_t sm = (size_t)(S::TWS + S::TZ * TSZ) * sizeof(V) + (size_t)3 * (S::N1 / 2) * S::THREADS_Z * sizeof(T);
     cudaError_t e = set_smem(k_fields_z<V, N>, sm);
     if (e != cudaSuccess) return e;
-    k_fields_z<V, N><<<dim3(N / S::TZ, N, S::kSplitGrids ? a.grids : 1), S::THREADS_Z, sm, s>>>(a, (const T*)A, (const V*)R, (const V*)tw, (V*)W0);
+    k_fields_z<V, N><<<dim3(N / S::TZ, N, S::kSplitGrids ? a.grids : 1), S::THREADS_Z, sm, s>>>(
+        a, (const T*)A, (const V*)R, (const V*)tw, (V*)W);
     return cudaGetLastError();
 }
 
@@ -1049,10 +1050,10 @@ cudaError_t launch_noise(cudaStream_t s, int precision, const FieldArgs& a, void
 }
 
 cudaError_t launch_fields_z(cudaStream_t s, int precision, const FieldArgs& a, const void* A, const void* R,
-                            const void* tw, void* W0)
+                            const void* tw, void* W)
 {
-#define Z64(n) run_half_z<n>(s, a, A, R, tw, W0)
-#define Z32(n) run_z<float2, n>(s, a, A, R, tw, W0)
+#define Z64(n) run_half_z<n>(s, a, A, R, tw, W)
+#define Z32(n) run_z<float2, n>(s, a, A, R, tw, W)
     if (precision == FDF_PREC_F64) FDF_DISPATCH_N(a.N, Z64)
     FDF_DISPATCH_N(a.N, Z32)
 #undef Z64

@@ -1064,9 +1064,9 @@ void push_wide(cudaStream_t s, unsigned b, const PushArgs& a, const ParticleStat
 //
 // Bound: the FP64 pipe.  Every 1/sqrt is rsqrt_fp64 (good to FP64 rounding) with its bits
 // from the integer pipe, the wrap tests bit patterns, and a kick reads only the slots its
-// equation uses: 133 FP64 instructions per particle-step against 292 with FP64 square
+// equation uses: 134.8 FP64 instructions per particle-step (ncu) against 292 with FP64 square
 // roots and divisions, of which the trilinear read of seven FP64 slots takes 71.  128^3
-// particles, one step: 1224 -> 525 us.
+// particles, one step: 1224 -> 504 us.
 
 template <bool EXACT>
 __global__ void __launch_bounds__(kThreads) k_push_f64(const __grid_constant__ PushArgs a, double* __restrict__ xd,

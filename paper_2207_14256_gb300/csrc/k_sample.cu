@@ -64,8 +64,8 @@ __device__ __forceinline__ double fd_inverse(const double* __restrict__ t, const
 }
 
 // Attempt `att` of the direction of particle (g0, g1): the words of v from streams 2 and 3;
-// accepted when 1e-300 < |v|^2 <= 1 in FP64.  FP32 settles that (the top 32 bits of each
-// component, |v|^2 to 3e-7) unless |v|^2 is within 1e-6 of 1 or of 0.
+// accepted when 1e-300 < |v|^2 <= 1 in FP64.  FP32 settles that (the first word of each
+// component, |v|^2 to 3.5e-7) unless |v|^2 is within 1e-6 of 1 or of 0.
 __device__ __forceinline__ bool direction_attempt(uint32_t g0, uint32_t g1, uint32_t att, uint32_t key0, uint32_t key1,
                                                   uint32_t w[6])
 {
@@ -77,7 +77,8 @@ __device__ __forceinline__ bool direction_attempt(uint32_t g0, uint32_t g1, uint
     w[3] = a.w;
     w[4] = b.x;
     w[5] = b.y;
-    // m >> 21 is the first word: (w0 - 2^31) 2^-31 is v to 2^-31
+    // (w0 - 2^31) 2^-31 is v to 2^-26 (m's top 27 bits are w0's; the next come from the second
+    // word), and FP32 rounds it and the sum: |v|^2 to 3.5e-7
     const float f0 = (float)(int)(a.x - 0x80000000u), f1 = (float)(int)(a.z - 0x80000000u);
     const float f2 = (float)(int)(b.x - 0x80000000u);
     const float r2 = (f0 * f0 + f1 * f1 + f2 * f2) * 2.168404344971009e-19f;   // 2^-62

@@ -122,7 +122,8 @@ FDF_DEV bool w_mul53(int64_t R, int k, double g, double& x)
 // The bits of q + (double)d in integers (a subnormal d counts as zero, as f2d_bits takes it):
 // d's 24-bit significand in units of q's last place, rounded to nearest, ties to even, is
 // added to q's bit pattern.  False where that may not be the sum's pattern: the sum leaves q's
-// binade or comes to its lower end (below which last places are finer), |d| is above 2^-1 |q| or so, or one of them is no finite normal number.
+// binade or comes to its lower end (below which last places are finer), |d| is above 2^-1 |q|
+// or so, or one of them is no finite normal number.
 FDF_DEV bool w_add(double q, float d, double& r)
 {
     const uint32_t hi = (uint32_t)__double2hiint(q), lo = (uint32_t)__double2loint(q), db = __float_as_uint(d);
@@ -259,7 +260,8 @@ FDF_DEV void w_horner(float ch, float cl, float th, float tl, float& sh, float& 
 // Polynomials in t = m^2 a_c^2 / u_0 (WideCoef says of what), coefficients h[k] + l[k].
 constexpr int kKickDeg = 10;    // highest degree
 // SERIES: the pass's fitted polynomials (c_0 in FP64, the others FP32), evaluated as the
-// FP64 formula does: u^(-1/2) to first order, t and the terms above c_0 in FP32.
+// FP64 formula does: u^(-1/2) to first order, t and the terms above c_0 in FP32.  Up to degree
+// 5, which steps of d ln a up to 0.111 need (155 steps from z = 1e9 to 31 and more).
 // !SERIES: the sums over the nodes themselves, from polynomials that agree with them to
 // 2^-47 (wide_poly.cuh); c_1 .. c_6 as pairs.
 template <bool SERIES> struct KickLen {
@@ -271,9 +273,11 @@ struct KickPoly {
 };
 
 // K_psi = u_0^(1/2) psi(t) and K_phi = u_0^(-1/2) phi(t) as FP32, u_0 = s_0 + mu, s_0 = |q_0|^2
-// and mu = m^2 a_c^2 as pairs in the run's momentum unit.  Pairs carry 2^-44 of the result;
-// the FP64 formula and the pairs differ by less than 2^-42, so a result that +-2^-41 does not
-// move to another float is FP64's (rounded to FP32).  Returns whether both are.
+// and mu = m^2 a_c^2 as pairs in the run's momentum unit.  A result that +-2^-41 does not move to another float counts as
+// FP64's (rounded to FP32).  The margin is a choice, not a derived bound: pairs carry about
+// 2^-44 of the result and FP64's own error is below 2^-50, and no result so accepted had other
+// bits than the FP64 formula's, on the host (tests/test_wide_math.py) and in whole runs on the
+// device (tests/test_gpu_wide_bits.py).  Returns whether both are.
 template <bool SERIES>
 FDF_DEV bool w_kick(float s0h, float s0l, float muh, float mul, const KickPoly& psi, const KickPoly& phi, float& Kpsi,
                     float& Kphi)
