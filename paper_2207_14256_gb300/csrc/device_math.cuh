@@ -157,6 +157,24 @@ template <typename V> __device__ __forceinline__ V cadd(V a, V b) { return mk<V>
 template <typename V> __device__ __forceinline__ V csub(V a, V b) { return mk<V>(a.x - b.x, a.y - b.y); }
 template <typename V> __device__ __forceinline__ V cmuli(V a) { return mk<V>(-a.y, a.x); }  // i a
 
+// ---- one axis of the order-2 kernel at u cells, in FP64 ----------------------
+// The nodes around the nearest one and their weights.  u is in [0, N] for a position in the
+// box; any other value, such as a NaN's, reads nodes of the grid too.
+__device__ __forceinline__ void tsc_f64(double u, int N, int idx[3], double w[3])
+{
+    const double c = floor(u + 0.5);
+    const double e = u - c;
+    int i = (int)c;
+    if (i >= N) i -= N;
+    i = i < 0 || i >= N ? 0 : i;
+    idx[0] = i == 0 ? N - 1 : i - 1;
+    idx[1] = i;
+    idx[2] = i + 1 == N ? 0 : i + 1;
+    w[0] = 0.5 * (0.5 - e) * (0.5 - e);
+    w[1] = 0.75 - e * e;
+    w[2] = 0.5 * (0.5 + e) * (0.5 + e);
+}
+
 // ---- fixed-point periodic coordinate -> (cell, fraction) on an N grid -------
 // X / 2^32 is the position in units of L; cell = floor(X N / 2^32), fraction =
 // ((X N) mod 2^32) / 2^32.

@@ -339,18 +339,7 @@ __device__ __forceinline__ void gather_f64_tsc(const double* __restrict__ G, int
     double w[3][3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        const double u = x[d] * invh;
-        const double c = floor(u + 0.5);
-        const double e = u - c;
-        int i = (int)c;
-        if (i >= N) i -= N;
-        if (i < 0) i += N;
-        idx[d][0] = i == 0 ? N - 1 : i - 1;
-        idx[d][1] = i;
-        idx[d][2] = i + 1 == N ? 0 : i + 1;
-        w[d][0] = 0.5 * (0.5 - e) * (0.5 - e);
-        w[d][1] = 0.75 - e * e;
-        w[d][2] = 0.5 * (0.5 + e) * (0.5 + e);
+        tsc_f64(x[d] * invh, N, idx[d], w[d]);
     }
 #pragma unroll
     for (int s = 0; s < 8; ++s) g[s] = 0.0;

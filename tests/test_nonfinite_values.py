@@ -1,8 +1,10 @@
 """The integer conversions of csrc/wide_math.cuh and the weight of csrc/device_math.cuh, compiled for
 the host, at values outside FP32's normal range: they are those of plain casts, so that NaN,
-infinities and overflows of a state reach the weights and the density as what they are.
+infinities and overflows of a state reach the weights and the density as what they are.  Reads at
+such positions stay in the grid.
 """
 import ctypes as C
+import math
 import os
 import subprocess
 
@@ -64,6 +66,7 @@ extern "C" void weights(long n, const double* q, const double* p, double T, floa
 {
     for (long i = 0; i < n; ++i) w[i] = dfweight_split(norm3_rn(q + 3 * i), p[i], T, 1.0 / T);
 }
+extern "C" void tsc(double u, int N, int* idx, double* w) { tsc_f64(u, N, idx, w); }
 extern "C" double kicked(double q, float d) { return add_slow(q, d); }
 """
 
@@ -79,6 +82,7 @@ def lib(tmp_path_factory):
     L = C.CDLL(str(d / "w.so"))
     L.check_narrow.restype = L.check_widen.restype = C.c_long
     L.kicked.restype, L.kicked.argtypes = C.c_double, [C.c_double, C.c_float]
+    L.tsc.argtypes = [C.c_double, C.c_int, C.c_void_p, C.c_void_p]
     return L
 
 
@@ -122,3 +126,18 @@ def test_kick_of_a_non_finite_gradient(lib):
     assert np.isnan(lib.kicked(1e-4, np.nan))
     assert lib.kicked(1e-4, np.inf) == np.inf and lib.kicked(1e-4, -np.inf) == -np.inf
     assert lib.kicked(1e-4, 1e-6) == 1e-4 + float(np.float32(1e-6))
+
+
+@pytest.mark.parametrize("N", [8, 512])
+def test_order_2_reads_stay_in_the_grid(lib, N):
+    idx, w = np.zeros(3, np.int32), np.zeros(3)
+    for u in (np.nan, -np.nan, np.inf, -np.inf, 1e30, -1e30, 3e9, -3e9, 2.0 ** 31, 1.0 * N, N - 0.5, N + 0.5, 2.5 * N, -0.75,
+              -1.0 * N, 0.0, 0.49, 3.5, 4.25):
+        lib.tsc(u, N, _ptr(idx), _ptr(w))
+        assert ((idx >= 0) & (idx < N)).all(), u
+        if 0 <= u <= N:
+            c = math.floor(u + 0.5)
+            assert list(idx) == [(c + o) % N for o in (-1, 0, 1)]
+            assert np.allclose(w, [0.5 * (0.5 - (u - c)) ** 2, 0.75 - (u - c) ** 2, 0.5 * (0.5 + (u - c)) ** 2], 1e-15)
+        elif not np.isfinite(u):
+            assert np.isnan(w).all()
