@@ -54,18 +54,18 @@ WIDE_FP64_PER_PASS = 5
 # (sm__inst_executed_pipe_fp64.sum x 32 / particle-steps of the launch, 128^3 particles, one step
 # per pass; profiles/), for its FP64-pipe roofline.  Dropped if the sources changed.
 PLAIN_FP64 = {"per_particle_step": 8831492 * 32 / 128 ** 3,
-              "sources_sha256": "80ae3655c29e4f3f:80f9684a0189b685:d5c895147bbe2b3b:2a492a4e0bbb3fee"}
+              "sources_sha256": "c8420730f99f5f5b:7570fd77cfe263fc:0e3e724159fc170b:25b8b0f4ce80e4b9"}
 
 # DRAM bytes per particle-step of the pass, from ncu (dram__bytes_read.sum + dram__bytes_write.sum,
-# mean over the 50 passes of a one-species 256^3 run with the schedule named in
+# mean over the passes of a one-species 256^3 run with the schedule named in
 # profiles/), by precision setting.  A launch's traffic is this times the particle-steps it
 # processes (the species are sorted one after the other, so each reads the grid on its own).
 # Valid only for the kernel sources they were measured on: their hash is checked and the figure
 # dropped if they changed.
-PUSH_TRAFFIC = {1: {"bytes_per_particle_step": (10.646e9 + 0.802e9) / (256 ** 3 * 8),
-                    "sources_sha256": "80ae3655c29e4f3f:80f9684a0189b685:d5c895147bbe2b3b:2a492a4e0bbb3fee"},
-                3: {"bytes_per_particle_step": (3.435e9 + 0.401e9) / (256 ** 3 * 4),
-                    "sources_sha256": "80ae3655c29e4f3f:80f9684a0189b685:d5c895147bbe2b3b:2a492a4e0bbb3fee"}}
+PUSH_TRAFFIC = {1: {"bytes_per_particle_step": (10.640e9 + 0.803e9) / (256 ** 3 * 8),
+                    "sources_sha256": "c8420730f99f5f5b:7570fd77cfe263fc:0e3e724159fc170b:25b8b0f4ce80e4b9"},
+                3: {"bytes_per_particle_step": (3.432e9 + 0.400e9) / (256 ** 3 * 4),
+                    "sources_sha256": "c8420730f99f5f5b:7570fd77cfe263fc:0e3e724159fc170b:25b8b0f4ce80e4b9"}}
 PUSH_SOURCES = ("k_particles.cu", "fdf_internal.cuh", "device_math.cuh", "wide_math.cuh")
 
 
