@@ -436,11 +436,8 @@ __global__ void __launch_bounds__(kThreads) k_initial(ParticleState st, int64_t 
 #pragma unroll
             for (int s = 0; s < 8; ++s) g[s] = w_f2d(gf[s]);
         }
-        // eps scales a term of ~1e-9 of q: a root through rsqrt_any serves it
         const double p = st.pmag[i];
-        const double e2 = p * p + m2a2;
-        const double eps = __double_as_longlong(e2) != 0 ? e2 * rsqrt_any(e2) : 0.0;
-        const double c = eps * tau0_6;          // eps tau0 / 6 (tau0/6 formed once)
+        const double c = sqrt_rn(p * p + m2a2) * tau0_6;        // eps tau0 / 6 (tau0/6 formed once)
         const double r = 1.0 - 0.5 * g[7];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
