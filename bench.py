@@ -54,7 +54,7 @@ WIDE_FP64_PER_PASS = 5
 # (sm__inst_executed_pipe_fp64.sum x 32 / particle-steps of the launch, 128^3 particles, one step
 # per pass; profiles/), for its FP64-pipe roofline.  Dropped if the sources changed.
 PLAIN_FP64 = {"per_particle_step": 8831492 * 32 / 128 ** 3,
-              "sources_sha256": "c8420730f99f5f5b:7570fd77cfe263fc:0e3e724159fc170b:25b8b0f4ce80e4b9"}
+              "sources_sha256": "57176a140ed16f72:7570fd77cfe263fc:0e3e724159fc170b:25b8b0f4ce80e4b9"}
 
 # DRAM bytes per particle-step of the pass, from ncu (dram__bytes_read.sum + dram__bytes_write.sum,
 # mean over the passes of a one-species 256^3 run with the schedule named in
@@ -62,10 +62,10 @@ PLAIN_FP64 = {"per_particle_step": 8831492 * 32 / 128 ** 3,
 # processes (the species are sorted one after the other, so each reads the grid on its own).
 # Valid only for the kernel sources they were measured on: their hash is checked and the figure
 # dropped if they changed.
-PUSH_TRAFFIC = {1: {"bytes_per_particle_step": (10.640e9 + 0.803e9) / (256 ** 3 * 8),
-                    "sources_sha256": "c8420730f99f5f5b:7570fd77cfe263fc:0e3e724159fc170b:25b8b0f4ce80e4b9"},
+PUSH_TRAFFIC = {1: {"bytes_per_particle_step": (10.710e9 + 0.803e9) / (256 ** 3 * 8),
+                    "sources_sha256": "57176a140ed16f72:7570fd77cfe263fc:0e3e724159fc170b:25b8b0f4ce80e4b9"},
                 3: {"bytes_per_particle_step": (3.432e9 + 0.400e9) / (256 ** 3 * 4),
-                    "sources_sha256": "c8420730f99f5f5b:7570fd77cfe263fc:0e3e724159fc170b:25b8b0f4ce80e4b9"}}
+                    "sources_sha256": "57176a140ed16f72:7570fd77cfe263fc:0e3e724159fc170b:25b8b0f4ce80e4b9"}}
 PUSH_SOURCES = ("k_particles.cu", "fdf_internal.cuh", "device_math.cuh", "wide_math.cuh")
 
 
